@@ -206,8 +206,6 @@ struct pd_grid {
     u64* rk2;
     uint8_t* flg;
     u64* hz;  // k+b buffer horizon
-    int* glist;  // flagged searches: groups holding a flagged query, and their count
-    int* gcount;
     u64* cmin;   // during a decimation: least live key of every 32-position chunk
     // small device scalars
     int* d_int;                  // [0] ngroups, [1..7] counters
@@ -218,14 +216,8 @@ struct pd_grid {
     int k1_exact;    // k = 1 density searches: nearest entries that must be exact (0: all 8;
                      //   the rest of the 8 stored are kept below the reported horizon)
     int k1_exact_rq; // ... in the re-searches of the rounds
-    int sparse_rq;   // k = 1 density re-searches over a list of the flagged points, 2 lanes
-                     //   each (else a warp per flagged leaf group)
     double compact_at;  // the rounds compact the grid once live < compact_at * built
                         //   (0: the cost's default)
-    int* rq_list;    // during a decimation: flagged Morton positions and their count
-    int* rq_count;
-    char* arena;     // during a decimation: scratch of the per-round compactions
-    size_t arena_cap;
     int trace;       // PD_TRACE set: one line per removal round on stderr
     int max_rounds;  // PD_MAX_ROUNDS: diagnostic stop (0 = none)
     // packed batch (pd_decimate_batch): nseg scans in tiles of edge
@@ -252,34 +244,6 @@ Scratch scratch_of(pd_grid* g) {
     s.alloc = scratch_alloc;
     s.free = scratch_free;
     s.self = g;
-    return s;
-}
-
-// Bump allocation from the grid's round arena (no allocator call per round:
-// the batch runs many small decimations from several host threads).  The
-// blocks of one compaction are released together by resetting the arena.
-struct ArenaUse {
-    pd_grid* g;
-    size_t used;
-};
-void* arena_alloc(void* self, size_t bytes) {
-    ArenaUse* a = (ArenaUse*)self;
-    size_t b = (bytes + 255) & ~(size_t)255;
-    if (!a->g->arena || a->used + b > a->g->arena_cap) return nullptr;
-    void* p = a->g->arena + a->used;
-    a->used += b;
-    return p;
-}
-void arena_free(void*, void*) {}
-// Scratch over the round arena when the decimation has one, else the allocator.
-Scratch round_scratch(pd_grid* g, ArenaUse* a) {
-    if (!g->arena) return scratch_of(g);
-    a->g = g;
-    a->used = 0;
-    Scratch s;
-    s.alloc = arena_alloc;
-    s.free = arena_free;
-    s.self = a;
     return s;
 }
 
@@ -363,7 +327,6 @@ int width_for(int k, int density_k1) {
     if (k <= 6) return 8;      // k nearest + at least 2 spare (k+b buffer)
     return 17;
 }
-int filt_width(int k) { return k <= 4 ? 4 : (k <= 8 ? 8 : 17); }
 
 // Octree leaf levels, cell hash and full-mode groups over pos/code[0, ng).
 int build_cells(pd_grid* g) {
@@ -462,8 +425,7 @@ extern "C" const char* pd_last_error(const pd_ctx* ctx) { return ctx ? ctx->err 
 // ============================================================ API: grid
 static int grid_release(pd_grid* g) {
     void* ptrs[] = {g->pos, g->code, g->leaf, g->alive, g->rgb, g->nrm, g->hash, g->groups,
-                    g->prim, g->nbr, g->rk2, g->flg, g->hz, g->d_int, g->d_u64, g->glist,
-                    g->gcount, g->cmin, g->nbr0, g->seg, g->seg_chunk0, g->seg_items};
+                    g->prim, g->nbr, g->rk2, g->flg, g->hz, g->d_int, g->d_u64, g->cmin, g->nbr0, g->seg, g->seg_chunk0, g->seg_items};
     for (void* p : ptrs) gfree(g, p);
     return PD_OK;
 }
@@ -499,8 +461,6 @@ extern "C" int pd_build_grid(pd_ctx* ctx, const int32_t* xyz_dev, const uint8_t*
     // result; the stored list is complete below the reported horizon)
     g->k1_exact = getenv("PD_K1_EXACT") ? atoi(getenv("PD_K1_EXACT")) : 2;
     g->k1_exact_rq = getenv("PD_K1_EXACT_RQ") ? atoi(getenv("PD_K1_EXACT_RQ")) : 3;
-    // diagnostic: 0 runs the re-searches per leaf group (same results)
-    g->sparse_rq = getenv("PD_SPARSE_REQUERY") ? atoi(getenv("PD_SPARSE_REQUERY")) : 1;
     // 0: by cost (decimate_impl); PD_COMPACT_AT overrides
     g->compact_at = getenv("PD_COMPACT_AT") ? atof(getenv("PD_COMPACT_AT")) : 0.0;
     if (!(g->compact_at > 0.0 && g->compact_at < 1.0)) g->compact_at = 0.0;
@@ -645,7 +605,6 @@ KnnArgs base_args(pd_grid* g, const pd_cost_params* cp) {
     a.rk2_out = g->rk2;
     a.flg_out = g->flg;
     a.hz_out = g->hz;
-    a.cmin = g->cmin;
     if (g->density_k1 && g->k1_exact > 0) a.r_exact = g->k1_exact;
     return a;
 }
@@ -889,31 +848,14 @@ BufView bufview(pd_grid* g, const pd_cost_params* cp) {
     return b;
 }
 
-// kNN over the leaf groups, querying only the points whose flag is set.
-int knn_flag(pd_grid* g, const pd_cost_params* cp, int filter, int S, const uint8_t* qflag,
-             u64* fout, const RoundDev* rd) {
+// Full searches of list[0 .. rd->nreq): the points whose stored neighbours no
+// longer settle their cost.
+int knn_requery(pd_grid* g, const pd_cost_params* cp, const int* list, const RoundDev* rd) {
     KnnArgs a = base_args(g, cp);
-    a.filter = filter;
-    a.S = S;
-    a.qflag = qflag;
-    a.rd = rd;
-    if (filter == FILT_BELOW_SELF) a.fprim_out = fout;
-    if (filter == FILT_BELOW_TAU) a.lam_out = fout;
-    if (filter == FILT_NONE && g->sparse_rq && g->rq_list) {
-        // k = 1 density re-searches: the flagged points, listed, 2 lanes each
-        // over their own cells (the weighted and k >= 2 rounds re-search few
-        // points per round, where a warp per flagged group measured faster)
-        ArenaUse au;
-        if (g->k1_exact_rq > 0) a.r_exact = g->k1_exact_rq;
-        CK(stable_compact(qflag, g->ng, g->rq_list, g->rq_count, round_scratch(g, &au), g->st));
-        CK(launch_knn_sparse(view_of(g), a, g->rq_list, g->rq_count, g->ng, g->st));
-        return PD_OK;
-    }
-    if (!g->glist) {  // groups never outnumber the points of the first build
-        ALLOC(g->glist, int, g->n);
-        ALLOC(g->gcount, int, 1);
-    }
-    CK(launch_knn_flagged(view_of(g), a, g->glist, g->gcount, g->st));
+    if (g->density_k1 && g->k1_exact_rq > 0) a.r_exact = g->k1_exact_rq;
+    a.qlist = list;
+    a.qcount = &rd->nreq;
+    CK(launch_knn_queries(view_of(g), a, g->ng, g->st));
     return PD_OK;
 }
 
@@ -1053,10 +995,6 @@ struct RoundScratch {
         for (void* p : ptrs) gfree(g, p);
         gfree(g, g->cmin);
         g->cmin = nullptr;
-        g->rq_list = nullptr;  // released with ptrs
-        g->rq_count = nullptr;
-        g->arena = nullptr;
-        g->arena_cap = 0;
         if (e0) cudaEventDestroy(e0);
         if (e1) cudaEventDestroy(e1);
     }
@@ -1156,29 +1094,17 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
     }
     g->stats.q_first = g->ng;
     int S = g->S;
-    int Sf = filt_width(k);
     int kchk = g->density_k1 ? S : k;
     bool use_buf = !g->density_k1 && S <= 8;
-    uint8_t *inP, *rej, *dirty, *fqf = nullptr, *dgf = nullptr;  // dgf: lambda search flags
-    int *cand, *slow, *src = nullptr, *csort = nullptr, *dep = nullptr;
-    u64 *fprim = nullptr, *lam = nullptr;
+    uint8_t *inP, *rej;
+    uint32_t* inPb = nullptr;  // bitmap of inP
+    int *cand, *slow, *rq, *fq = nullptr, *lq = nullptr, *src = nullptr, *dep = nullptr;
+    u64* lam = nullptr;
     int2* pairs = nullptr;
     int64_t cap = g->n;
     RALLOC(inP, uint8_t, cap);
     RALLOC(rej, uint8_t, cap);
-    RALLOC(dirty, uint8_t, cap);
-    if (g->sparse_rq && g->density_k1) {
-        RALLOC(g->rq_list, int, cap);
-        RALLOC(g->rq_count, int, 1);
-    }
-    {
-        // offsets of one compaction (a word per 1024 points) and the sums of
-        // its scan (a word per 1024 offsets, recursively), 256-byte aligned
-        size_t nb = (size_t)(cap + 1023) / 1024;
-        size_t words = nb + nb / 512 + 64;
-        g->arena_cap = words * 4 + 8 * 256;
-        RALLOC(g->arena, char, g->arena_cap);
-    }
+    RALLOC(rq, int, cap);
     RALLOC(cand, int, cap);
     RALLOC(slow, int, cap);
     if (g->density_k1) RALLOC(dep, int, cap);
@@ -1186,11 +1112,10 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
     CK(cudaMemsetAsync(rej, 0, cap, g->st));
     int pair_cap = 0;
     if (!g->density_k1) {
-        RALLOC(fqf, uint8_t, cap);
-        RALLOC(dgf, uint8_t, cap);
+        RALLOC(inPb, uint32_t, (cap + 31) / 32);
+        RALLOC(fq, int, cap);
+        RALLOC(lq, int, cap);
         RALLOC(src, int, cap);
-        RALLOC(csort, int, cap);
-        RALLOC(fprim, u64, cap);
         RALLOC(lam, u64, cap);
         pair_cap = (int)std::min<int64_t>(std::max<int64_t>(cap * 4, 1 << 16), 1 << 30);
         // diagnostic: a smaller danger-pair capacity forces the host settle of
@@ -1263,27 +1188,28 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
                                    rd, inP, rej, cand, slow, dep, h.fix_iters, g->st));
             } else {
                 BufView bv = bufview(g, cp);
-                CK(round_launch_kk_cand2(bv, g->alive, g->ng, S, k, rd, inP, cand, fqf, dgf, lam, src,
-                                         g->st));
-                CK(launch_chunk_min(g->prim, g->alive, g->ng, g->cmin, g->st));
+                CK(round_launch_kk_cand2(bv, g->alive, g->ng, S, k, rd, inP, inPb, cand, fq, lq,
+                                         lam, src, g->cmin, g->st));
                 {
                     Span t(T, &g->stats.ms_knn);
-                    rc = knn_flag(g, cp, FILT_BELOW_SELF, Sf, fqf, fprim, rd);
-                    if (rc) return rc;
-                }
-                CK(round_launch_kk_accept(fqf, g->prim, fprim, g->ng, rd, inP, cand, g->st));
-                {
-                    Span t(T, &g->stats.ms_knn);
-                    rc = knn_flag(g, cp, FILT_BELOW_TAU, Sf, dgf, lam, rd);
-                    if (rc) return rc;
+                    KnnArgs a = base_args(g, cp);
+                    a.rd = rd;
+                    a.qlist = fq;
+                    a.qcount = &rd->nfq;
+                    a.qlist2 = lq;
+                    a.qcount2 = &rd->nlq;
+                    a.lam_out = lam;
+                    a.inP = inP;
+                    a.inPb = inPb;
+                    a.cand = cand;
+                    a.ncand = &rd->ncand;
+                    a.cmin = g->cmin;
+                    CK(launch_knn_queries(v, a, g->ng, g->st));
                 }
                 {
                     Span t(T, &g->stats.ms_danger);
-                    // candidates in Morton order, so each source finds its own by search
-                    ArenaUse au;
-                    CK(stable_compact(inP, g->ng, csort, &rd->ncs, round_scratch(g, &au), g->st));
-                    CK(round_launch_danger(v, src, g->prim, g->alive, inP, rej, lam, g->nbr, S, k,
-                                           pairs, pair_cap, csort, rd, g->st));
+                    CK(round_launch_danger(v, src, g->prim, g->alive, inPb, rej, lam, g->nbr, S, k,
+                                           pairs, pair_cap, rd, g->st));
                 }
                 CK(round_launch_pairs_fix(pairs, pair_cap, inP, rej, rd, g->st));
             }
@@ -1291,17 +1217,17 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
             if (g->density_k1) {
                 // absorb removals in the stored 8 nearest; search where the new
                 // nearest shell may be incomplete
-                CK(round_launch_k1_update(bufview(g, cp), g->alive, g->ng, S, dirty, rd, g->st));
+                CK(round_launch_k1_update(bufview(g, cp), g->alive, g->ng, S, rq, rd, g->st));
             } else if (use_buf) {
                 // absorb removals in the k+b buffers; search only where < k remain
-                CK(round_launch_kk_update(bufview(g, cp), g->alive, g->ng, S, k, dirty, rd, g->st));
+                CK(round_launch_kk_update(bufview(g, cp), g->alive, g->ng, S, k, rq, rd, g->st));
             } else {
-                CK(round_launch_dirty(g->alive, g->nbr, g->ng, S, kchk, dirty, rd, g->st));
+                CK(round_launch_dirty(g->alive, g->nbr, g->ng, S, kchk, rq, rd, g->st));
             }
             if (g->trace) cudaEventRecord(tq0, g->st);
             {
                 Span t(T, &g->stats.ms_knn_requery);
-                rc = knn_flag(g, cp, FILT_NONE, S, dirty, nullptr, rd);
+                rc = knn_requery(g, cp, rq, rd);
                 if (rc) return rc;
             }
             if (g->trace) cudaEventRecord(tq1, g->st);
@@ -1378,14 +1304,14 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
                               &removed);
             if (rc) return rc;
             if (g->density_k1)
-                CK(round_launch_k1_update(bufview(g, cp), g->alive, g->ng, S, dirty, rd, g->st));
+                CK(round_launch_k1_update(bufview(g, cp), g->alive, g->ng, S, rq, rd, g->st));
             else if (use_buf)
-                CK(round_launch_kk_update(bufview(g, cp), g->alive, g->ng, S, k, dirty, rd, g->st));
+                CK(round_launch_kk_update(bufview(g, cp), g->alive, g->ng, S, k, rq, rd, g->st));
             else
-                CK(round_launch_dirty(g->alive, g->nbr, g->ng, S, kchk, dirty, rd, g->st));
+                CK(round_launch_dirty(g->alive, g->nbr, g->ng, S, kchk, rq, rd, g->st));
             {
                 Span t(T, &g->stats.ms_knn_requery);
-                rc = knn_flag(g, cp, FILT_NONE, S, dirty, nullptr, rd);
+                rc = knn_requery(g, cp, rq, rd);
                 if (rc) return rc;
             }
             h.live -= removed;

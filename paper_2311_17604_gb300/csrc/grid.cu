@@ -366,7 +366,7 @@ cudaError_t launch_node_count(const u64* code, const uint8_t* leaf, int64_t n, i
 }
 
 __device__ inline long long hash_insert(HashSlot* tab, u64 mask, u64 key) {
-    u64 h = mix64(key) & mask;
+    u64 h = hash_slot(key, mask);
     for (u64 it = 0; it <= mask; it++) {
         u64 prev = atomicCAS(&tab[h].key, PD_EMPTY_KEY, key);
         if (prev == PD_EMPTY_KEY || prev == key) return (long long)h;

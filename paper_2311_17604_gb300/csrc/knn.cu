@@ -240,21 +240,7 @@ struct TopPack {
     }
 };
 
-__device__ inline u64 box_d2(int ux, int uy, int uz, int bx, int by, int bz, int sh) {
-    long long q[3] = {ux, uy, uz};
-    int c[3] = {bx, by, bz};
-    u64 s = 0;
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        long long lo = (long long)c[a] << sh;
-        long long hi = ((long long)(c[a] + 1) << sh) - 1;
-        long long d = q[a] < lo ? lo - q[a] : (q[a] > hi ? q[a] - hi : 0);
-        s += (u64)(d * d);
-    }
-    return s;
-}
-
-// The same in 32-bit arithmetic, for levels whose cell edge is at most
+// box_d2 in 32-bit arithmetic, for levels whose cell edge is at most
 // 2^13 mm: the box is the query's own or an adjacent cell's leaf, so every
 // coordinate gap is below 2 * 2^13 and the sum below 2^30.
 __device__ inline u64 box_d2_32(int ux, int uy, int uz, int bx, int by, int bz, int sh) {
@@ -275,25 +261,19 @@ __device__ inline u64 box_d2_32(int ux, int uy, int uz, int bx, int by, int bz, 
 // cells [c-1, c+1]; ~0 when the cube holds the whole cloud.
 __device__ inline u64 gap2(const GridView& g, int ux, int uy, int uz, int L, int cx, int cy,
                            int cz) {
-    int sh = L + g.shift;
-    long long q[3] = {ux, uy, uz};
-    int c[3] = {cx, cy, cz};
-    int m[3] = {g.umax.x, g.umax.y, g.umax.z};
-    long long best = -1;
+    const int sh = L + g.shift;
+    const int q[3] = {ux, uy, uz};
+    const int c[3] = {cx, cy, cz};
+    const int m[3] = {g.umax.x, g.umax.y, g.umax.z};
+    int best = 0x7fffffff;
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-        long long lo = (long long)(c[a] - 1) << sh;
-        long long hi = (long long)(c[a] + 2) << sh;
-        if (lo > 0) {
-            long long d = q[a] - lo + 1;
-            if (best < 0 || d < best) best = d;
-        }
-        if (hi <= m[a]) {
-            long long d = hi - q[a];
-            if (best < 0 || d < best) best = d;
-        }
+        // faces are below 2^25 + 2 * 2^25: ints
+        const int lo = (c[a] - 1) * (1 << sh), hi = (c[a] + 2) * (1 << sh);
+        if (lo > 0) best = min(best, q[a] - lo + 1);
+        if (hi <= m[a]) best = min(best, hi - q[a]);
     }
-    return best < 0 ? ~0ull : (u64)best * (u64)best;
+    return best == 0x7fffffff ? ~0ull : (u64)((long long)best * best);
 }
 
 __device__ inline double nbr_weight(const KnnArgs& a, int q, int j) {
@@ -333,26 +313,17 @@ __device__ inline double cost_sum(const KnnArgs& a, int q, const TL& top, int k)
 }
 
 // Stream one range [b, e) of Morton positions against every lane's query.
-template <int S, int FILT, bool W, class TL, typename D>
+template <int S, bool W, class TL, typename D>
 __device__ __forceinline__ void scan_range(const GridView& g, const KnnArgs& a, uint32_t b,
-                                           uint32_t e, int q, int4 qp, bool todo, u64 tp, int ti,
-                                           u64 tpmax, TL& top, int4* sp, u64* sk, int* so,
-                                           int lane, int sub, int lpq) {
+                                           uint32_t e, int q, int4 qp, bool todo, TL& top,
+                                           int4* sp, int* so, int lane, int sub, int lpq) {
     for (uint32_t c = b; c < e; c += 32) {
-        if (FILT != FILT_NONE && a.cmin) {
-            // no key of these 32 positions is below any lane's threshold: skip
-            // (c, e and tpmax are warp-uniform, so the whole warp skips)
-            uint32_t last = min(c + 31u, e - 1u);
-            u64 m0 = a.cmin[c >> 5], m1 = a.cmin[last >> 5];
-            if ((m0 < m1 ? m0 : m1) > tpmax) continue;
-        }
         uint32_t j = c + lane;
         int4 v = make_int4(0, 0, 0, -1);
         if (j < e) {
             v = g.pos[j];
             bool ok = !a.alive || a.alive[j];
-            if (FILT != FILT_NONE) sk[lane] = a.prim[j];
-            if (FILT != FILT_NONE || W) so[lane] = v.w;
+            if (W) so[lane] = v.w;
             v.w = ok ? (int)j : -1;
         }
         sp[lane] = v;
@@ -362,9 +333,6 @@ __device__ __forceinline__ void scan_range(const GridView& g, const KnnArgs& a, 
             for (int t = sub; t < m; t += lpq) {
                 int4 cv = sp[t];
                 if (cv.w < 0 || cv.w == q) continue;
-                if (FILT != FILT_NONE) {
-                    if (!key_gt(tp, ti, sk[t], so[t])) continue;  // keep keys below threshold
-                }
                 int dx = cv.x - qp.x, dy = cv.y - qp.y, dz = cv.z - qp.z;
                 D dd;
                 if (sizeof(D) == 4) {
@@ -384,53 +352,43 @@ __device__ __forceinline__ void scan_range(const GridView& g, const KnnArgs& a, 
 // hzv: squared distance below which every live point is in the list (the
 // searched cube's gap and the skipped cells' boxes; the S-th distance when
 // the list is full).
-template <int S, int FILT, bool W, class TL>
+template <int S, bool W, class TL>
 __device__ __forceinline__ void write_result(const KnnArgs& a, int q, const TL& top, u64 hzv) {
     int found = 0;
 #pragma unroll
     for (int i = 0; i < S; i++) found += top.has(i);
-    if (FILT == FILT_NONE) {
-        if (a.density_k1) {
-            // all S nearest are stored (the k+b buffer); the shell is the
-            // prefix at the nearest distance d0, its size kept in flg >> 2
-            u64 d0 = top.dist(0);
-            int shell = 0;
+    if (a.density_k1) {
+        // all S nearest are stored (the k+b buffer); the shell is the
+        // prefix at the nearest distance d0, its size kept in flg >> 2
+        u64 d0 = top.dist(0);
+        int shell = 0;
 #pragma unroll
-            for (int i = 0; i < S; i++) {
-                bool h = top.has(i);
-                shell += (h && top.dist(i) == d0) ? 1 : 0;
-                a.nbr[(int64_t)q * S + i] = h ? top.ident(i) : -1;
-            }
-            if (!W && a.nbr0_out) a.nbr0_out[q] = top.has(0) ? top.ident(0) : -1;
-            a.prim_out[q] = key_prim_d2(d0);
-            a.rk2_out[q] = d0;
-            a.flg_out[q] = (uint8_t)((shell >= 2 ? 1 : 0) | (shell == S ? 2 : 0) | (shell << 2));
-            if (a.hz_out) {
-                u64 h = top.has(S - 1) ? top.dist(S - 1) : ~0ull;
-                a.hz_out[q] = hzv < h ? hzv : h;
-            }
-            if (a.cost_out) a.cost_out[q] = d0 == ~0ull ? 0.0 : __ddiv_rn(1.0, (double)d0);
-        } else {
-            int k = a.k;
-#pragma unroll
-            for (int i = 0; i < S; i++) a.nbr[(int64_t)q * S + i] = top.has(i) ? top.ident(i) : -1;
-            double c = cost_sum<S>(a, q, top, k);
-            a.prim_out[q] = key_prim_cost(c);
-            u64 dk = top.at(k - 1);
-            a.rk2_out[q] = dk;
-            bool tie = found > k && top.at(k) == dk;
-            a.flg_out[q] = (uint8_t)(tie ? 1 : 0);
-            if (a.hz_out) a.hz_out[q] = top.dist(S - 1);
-            if (a.cost_out) a.cost_out[q] = c;
+        for (int i = 0; i < S; i++) {
+            bool h = top.has(i);
+            shell += (h && top.dist(i) == d0) ? 1 : 0;
+            a.nbr[(int64_t)q * S + i] = h ? top.ident(i) : -1;
         }
-    } else if (FILT == FILT_BELOW_SELF) {
-        if (a.density_k1) {
-            a.fprim_out[q] = key_prim_d2(top.dist(0));
-        } else {
-            a.fprim_out[q] = key_prim_cost(cost_sum<S>(a, q, top, a.k));
+        if (!W && a.nbr0_out) a.nbr0_out[q] = top.has(0) ? top.ident(0) : -1;
+        a.prim_out[q] = key_prim_d2(d0);
+        a.rk2_out[q] = d0;
+        a.flg_out[q] = (uint8_t)((shell >= 2 ? 1 : 0) | (shell == S ? 2 : 0) | (shell << 2));
+        if (a.hz_out) {
+            u64 h = top.has(S - 1) ? top.dist(S - 1) : ~0ull;
+            a.hz_out[q] = hzv < h ? hzv : h;
         }
+        if (a.cost_out) a.cost_out[q] = d0 == ~0ull ? 0.0 : __ddiv_rn(1.0, (double)d0);
     } else {
-        a.lam_out[q] = top.at(a.k - 1);
+        int k = a.k;
+#pragma unroll
+        for (int i = 0; i < S; i++) a.nbr[(int64_t)q * S + i] = top.has(i) ? top.ident(i) : -1;
+        double c = cost_sum<S>(a, q, top, k);
+        a.prim_out[q] = key_prim_cost(c);
+        u64 dk = top.at(k - 1);
+        a.rk2_out[q] = dk;
+        bool tie = found > k && top.at(k) == dk;
+        a.flg_out[q] = (uint8_t)(tie ? 1 : 0);
+        if (a.hz_out) a.hz_out[q] = top.dist(S - 1);
+        if (a.cost_out) a.cost_out[q] = c;
     }
 }
 
@@ -438,14 +396,13 @@ __device__ __forceinline__ void write_result(const KnnArgs& a, int q, const TL& 
 // query's partial lists, and finish the queries whose R-th distance is
 // closer than the searched cube's faces.  PACK: every range of this level
 // has squared distances below 2^32 (packed lists, 32-bit distances).
-template <int S, int FILT, bool W, class TL, bool PACK>
+template <int S, bool W, class TL, bool PACK>
 __device__ __forceinline__ void knn_level(const GridView& g, const KnnArgs& a, int L, int R,
                                           int q, int4 qp, int ux, int uy, int uz, bool& todo,
-                                          u64 tp, int ti, u64 tpmax, int lane, int sub, int lpq,
-                                          int rt,
-                                          uint32_t rb, uint32_t re, int rl, int bx, int by,
-                                          int bz, int cx, int cy, int cz, int4* sp, u64* sk,
-                                          int* so, unsigned long long& wpairs) {
+                                          int lane, int sub, int lpq, int rt, uint32_t rb,
+                                          uint32_t re, int rl, int bx, int by, int bz, int cx,
+                                          int cy, int cz, int4* sp, int* so,
+                                          unsigned long long& wpairs) {
     TL top;
     top.init();
     u64 hzl = ~0ull;  // smallest box distance of a range this lane did not scan
@@ -478,11 +435,9 @@ __device__ __forceinline__ void knn_level(const GridView& g, const KnnArgs& a, i
             wpairs += (unsigned long long)(e - b) * (unsigned long long)nqt;
         }
         if (PACK || lv + g.shift <= 13)
-            scan_range<S, FILT, W, TL, uint32_t>(g, a, b, e, q, qp, todo, tp, ti, tpmax, top, sp,
-                                                 sk, so, lane, sub, lpq);
+            scan_range<S, W, TL, uint32_t>(g, a, b, e, q, qp, todo, top, sp, so, lane, sub, lpq);
         else
-            scan_range<S, FILT, W, TL, u64>(g, a, b, e, q, qp, todo, tp, ti, tpmax, top, sp, sk, so,
-                                            lane, sub, lpq);
+            scan_range<S, W, TL, u64>(g, a, b, e, q, qp, todo, top, sp, so, lane, sub, lpq);
     }
     // merge the partial lists of each query's lanes (butterfly)
     for (int off = lpq >> 1; off >= 1; off >>= 1) top.merge_xor(off, todo);
@@ -491,21 +446,21 @@ __device__ __forceinline__ void knn_level(const GridView& g, const KnnArgs& a, i
         u64 bound = top.at(R - 1);
         if (gg == ~0ull || bound < gg) {
             todo = false;
-            if (sub == 0) write_result<S, FILT, W>(a, q, top, hzl < gg ? hzl : gg);
+            if (sub == 0) write_result<S, W>(a, q, top, hzl < gg ? hzl : gg);
         }
     }
 }
 
 // One leaf group (<= 32 queries) for one warp.
-template <int S, int FILT, bool W>
+template <int S, bool W>
 __device__ __forceinline__ void knn_group(const GridView& g, const KnnArgs& a, int gid, int4* sp,
-                                          u64* sk, int* so, int lane) {
+                                          int* so, int lane) {
     int4 G = a.groups[gid];
     int cnt = G.y;
     int L = G.z;
     int q = -1;
     if (lane < cnt) {
-        q = a.list ? a.list[G.x + lane] : G.x + lane;
+        q = G.x + lane;
         if (a.qflag && !a.qflag[q]) q = -1;
     }
     // pack the active queries onto the 32 lanes: with nq queries each gets
@@ -522,58 +477,16 @@ __device__ __forceinline__ void knn_group(const GridView& g, const KnnArgs& a, i
         int qq = __shfl_sync(FULLM, q, srcl);
         q = qi < nq ? qq : -1;
     }
-    int q0 = a.list ? a.list[G.x] : G.x;
-    u64 c0 = g.code[q0];
+    u64 c0 = g.code[G.x];
     int4 qp = q >= 0 ? g.pos[q] : make_int4(0, 0, 0, 0);
     int ux = qp.x - g.origin.x, uy = qp.y - g.origin.y, uz = qp.z - g.origin.z;
-    u64 tp = 0;
-    int ti = 0;
-    if (FILT == FILT_BELOW_SELF && q >= 0) {
-        tp = a.prim[q];
-        ti = qp.w;
-    } else if (FILT == FILT_BELOW_TAU) {
-        if (a.rd && a.rd->seg) {
-            // packed batch: the threshold of the query's own scan (its
-            // neighbours are all in that scan)
-            if (q >= 0) round_tau(a.rd, qp, tp, ti);
-        } else if (a.rd) {
-            tp = a.rd->tau_prim;
-            ti = a.rd->tau_idx;
-        } else {
-            tp = a.tau_prim;
-            ti = a.tau_idx;
-        }
-    }
-    // the largest threshold of the warp's queries (chunk skipping); reduced
-    // over all 32 lanes so that every lane holds the same value: the skip in
-    // scan_range must be taken by the whole warp or by none of it
-    u64 tpmax = q >= 0 ? tp : 0;
-    if (FILT != FILT_NONE) {
-        for (int off = 16; off; off >>= 1) {
-            u64 o = __shfl_xor_sync(FULLM, tpmax, off);
-            tpmax = o > tpmax ? o : tpmax;
-        }
-    }
-    // exactness bound: the R-th smallest distance must be exact
-    // full searches: all S stored neighbours exact (the k+b neighbour buffer,
-    // so a removal can be absorbed without a new search; for the k = 1
-    // density cost the nearest shell is then complete); filtered searches: k.
-    const int R = FILT == FILT_NONE ? (a.r_exact > 0 && a.r_exact < S ? a.r_exact : S) : a.k;
+    // exactness bound: the R-th smallest distance must be exact: all S stored
+    // neighbours (the k+b neighbour buffer, so a removal can be absorbed
+    // without a new search; for the k = 1 density cost the nearest shell is
+    // then complete), or the first r_exact of them
+    const int R = a.r_exact > 0 && a.r_exact < S ? a.r_exact : S;
     bool todo = q >= 0;
     unsigned long long wpairs = 0;
-    if (FILT == FILT_BELOW_TAU && a.hz_out) {
-        // a lambda search runs when fewer than k lower-key points are among a
-        // query's stored neighbours; every live point closer than its horizon
-        // hz is stored, so lambda >= hz: start at the first level whose cell
-        // edge reaches sqrt(hz) (smallest over the group's queries)
-        u64 h = q >= 0 ? a.hz_out[q] : ~0ull;
-        for (int off = 16; off; off >>= 1) {
-            u64 o = __shfl_xor_sync(FULLM, h, off);
-            h = o < h ? o : h;
-        }
-        if (h != ~0ull)
-            while (L < g.B && (1ull << (2 * (L + g.shift))) < h) L++;
-    }
     while (__any_sync(FULLM, todo)) {
         int sh = 3 * L;
         int cx = (int)compact3(c0 >> sh), cy = (int)compact3(c0 >> (sh + 1)),
@@ -583,12 +496,12 @@ __device__ __forceinline__ void knn_group(const GridView& g, const KnnArgs& a, i
         int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
         uint32_t rb = 0, re = 0;
         int rl = L, rt = 0;
-        if (lane < 27) rt = resolve_cell(g, L, cx + dx, cy + dy, cz + dz, rb, re, &rl);
-        for (int j = 0; j < 27; j++) {  // a coarse leaf reached from two cells is scanned once
-            uint32_t bj = __shfl_sync(FULLM, rb, j);
-            int tj = __shfl_sync(FULLM, rt, j);
-            if (j < lane && rt == 2 && tj == 2 && bj == rb) rt = 0;
-        }
+        u64 prefix = L < g.B ? c0 >> sh : 0;
+        if (lane < 27 && prefix_offset(prefix, g.B - L, dx, dy, dz))
+            rt = resolve_prefix(g, L, prefix, rb, re, &rl);
+        // a coarse leaf reached from two cells is scanned once
+        const unsigned same = __match_any_sync(FULLM, rt == 2 ? rb : 0x80000000u + lane);
+        if (rt == 2 && __ffs(same) - 1 != lane) rt = 0;
         int bx = 0, by = 0, bz = 0;
         if (rt) {
             bx = (cx + dx) >> (rl - L);
@@ -599,13 +512,13 @@ __device__ __forceinline__ void knn_group(const GridView& g, const KnnArgs& a, i
         // within 3 cells of 2^13 mm (squared distances < 3 * 24576^2 < 2^32)
         bool pack = __all_sync(FULLM, !rt || rl + g.shift <= 13);
         if (pack)
-            knn_level<S, FILT, W, TopPack<S, W>, true>(g, a, L, R, q, qp, ux, uy, uz, todo, tp, ti,
-                                                       tpmax, lane, sub, lpq, rt, rb, re, rl, bx, by, bz,
-                                                       cx, cy, cz, sp, sk, so, wpairs);
+            knn_level<S, W, TopPack<S, W>, true>(g, a, L, R, q, qp, ux, uy, uz, todo, lane, sub,
+                                                 lpq, rt, rb, re, rl, bx, by, bz, cx, cy, cz, sp,
+                                                 so, wpairs);
         else
-            knn_level<S, FILT, W, TopList<S, W>, false>(g, a, L, R, q, qp, ux, uy, uz, todo, tp,
-                                                        ti, tpmax, lane, sub, lpq, rt, rb, re, rl, bx, by,
-                                                        bz, cx, cy, cz, sp, sk, so, wpairs);
+            knn_level<S, W, TopList<S, W>, false>(g, a, L, R, q, qp, ux, uy, uz, todo, lane, sub,
+                                                  lpq, rt, rb, re, rl, bx, by, bz, cx, cy, cz, sp,
+                                                  so, wpairs);
         L++;
     }
     // spread over PD_PAIR_SLOTS counters by SM (one address would serialise
@@ -620,241 +533,542 @@ __device__ __forceinline__ void knn_group(const GridView& g, const KnnArgs& a, i
 // The first full pass of the density path (S = 8, no weights) is held to 64
 // registers for 8 blocks per SM: more warps in flight measured faster than
 // the few bytes it spills (first pass of the 100M-point scan 70.4 -> 67.1 ms).
-template <int S, int FILT, bool W, bool LIST>
-__global__ void __launch_bounds__(PD_WARPS * 32, (S == 8 && !W && !LIST) ? 8 : 1)
+template <int S, bool W>
+__global__ void __launch_bounds__(PD_WARPS * 32, (S == 8 && !W) ? 8 : 1)
     knn_kernel(GridView g, KnnArgs a) {
     __shared__ int4 s_p[PD_WARPS][32];
-    __shared__ u64 s_k[PD_WARPS][32];
     __shared__ int s_o[PD_WARPS][32];
     int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (LIST) {  // persistent over the listed groups
-        int ng = *a.gcount;
-        for (int t = blockIdx.x * PD_WARPS + w; t < ng; t += gridDim.x * PD_WARPS)
-            knn_group<S, FILT, W>(g, a, a.glist[t], s_p[w], s_k[w], s_o[w], lane);
-    } else {
-        int gid = blockIdx.x * PD_WARPS + w;
-        if (gid < a.ngroups) knn_group<S, FILT, W>(g, a, gid, s_p[w], s_k[w], s_o[w], lane);
-    }
+    int gid = blockIdx.x * PD_WARPS + w;
+    if (gid < a.ngroups) knn_group<S, W>(g, a, gid, s_p[w], s_o[w], lane);
 }
 
-// Sparse re-searches: the listed queries (Morton positions, list[0 .. *count))
-// run SP_SLOTS to a warp, SP_LANES lanes per query, each query over the
-// 3x3x3 cells of its own leaf level.  The lanes of a query resolve its 27
-// cells (every SP_LANES-th one) into shared memory; a coarse leaf reached
-// from two cells is kept once.  Each lane then walks the staged ranges on its
-// own, taking positions b + sub, b + sub + SP_LANES, ... of every range whose
-// box is not beyond its own partial bound (never closer than the merged one;
-// the smallest box distance it skipped bounds the reported horizon), and
-// keeps a partial list; the partial lists merge once per level.  Lists are
-// packed (one 64-bit key per entry, 32-bit distances) when every range of the
-// warp's level lies within 3 cells of 2^13 mm.  Used for the re-searches of
-// the removal rounds, where the flagged queries are few per leaf group and a
-// warp per group would idle most lanes.  2 lanes per query (16 queries per
-// warp) measured faster than 4 or 8 and level with 1.
-#define SP_LANES 2
-#define SP_SLOTS (32 / SP_LANES)
+// ------------------------------------------------------------------ one warp per query
+// The searches of the removal rounds: re-searches of points that lost too
+// many stored neighbours, and the filtered searches of the candidate and
+// danger tests.  A round has few of them, scattered over the cloud, so a
+// round's search time is the latency of one query's chain of dependent loads,
+// not the arithmetic: one warp serves one query.  Lanes 0..26 resolve the 27
+// cells at once, the non-empty ranges are laid end to end, and every lane
+// takes every 32nd candidate of that sequence, the next step's loads issued
+// before this step's are used.  The 32 nearest so far are kept sorted across
+// the lanes (lane i holds the i-th); a step's candidates below the S-th are
+// inserted one by one, or, when there are many (the first step), sorted
+// (bitonic) and merged.  Measured against the kernels it replaces (k = 1: 2
+// lanes per query walking the ranges in turn; otherwise a warp per leaf group
+// with a flagged point), all rounds of one decimation: 9.8M outdoor points,
+// k = 4, re-searches 114 -> 16 ms, filtered and lambda searches 116 -> 18.6 ms;
+// 100M site points, k = 1, 41.2 -> 33.7 ms; 200k room points, k = 1, 1.51 -> 0.25 ms.
+template <bool PACK>
+struct WarpKey {  // (d^2, tie), ordered; PACK: d^2 < 2^32, both in one word
+    u64 d;
+    uint32_t t;
+    __device__ __forceinline__ static WarpKey make(u64 dd, uint32_t tie) {
+        WarpKey k;
+        k.d = PACK ? (dd << 32) | tie : dd;
+        k.t = tie;
+        return k;
+    }
+    __device__ __forceinline__ static WarpKey none() {
+        WarpKey k;
+        k.d = ~0ull;
+        k.t = 0xffffffffu;
+        return k;
+    }
+    __device__ __forceinline__ bool less(const WarpKey& o) const {
+        return PACK ? d < o.d : (d < o.d || (d == o.d && t < o.t));
+    }
+    __device__ __forceinline__ bool has() const { return d != ~0ull; }
+    __device__ __forceinline__ u64 dist() const { return PACK && has() ? d >> 32 : d; }
+    __device__ __forceinline__ uint32_t tie() const { return PACK ? (uint32_t)d : t; }
+    __device__ __forceinline__ WarpKey from(int src) const {
+        WarpKey k;
+        k.d = __shfl_sync(FULLM, d, src);
+        k.t = PACK ? 0u : __shfl_sync(FULLM, t, src);
+        return k;
+    }
+    __device__ __forceinline__ WarpKey across(int mask) const {
+        WarpKey k;
+        k.d = __shfl_xor_sync(FULLM, d, mask);
+        k.t = PACK ? 0u : __shfl_xor_sync(FULLM, t, mask);
+        return k;
+    }
+    __device__ __forceinline__ WarpKey before() const {
+        WarpKey k;
+        k.d = __shfl_up_sync(FULLM, d, 1);
+        k.t = PACK ? 0u : __shfl_up_sync(FULLM, t, 1);
+        return k;
+    }
+};
 
-template <int S, bool W, class TL, bool PACK>
-__device__ __forceinline__ void sparse_level(const GridView& g, const KnnArgs& a, int R, int q,
-                                             int4 qp, int ux, int uy, int uz, int L, int cx,
-                                             int cy, int cz, int sub, bool& todo,
-                                             const uint32_t* __restrict__ sb,
-                                             const uint32_t* __restrict__ se,
-                                             const uint8_t* __restrict__ sl) {
-    TL top;
-    top.init();
-    u64 hzl = ~0ull;
-    if (todo) {
-        for (int r = 0; r < 27; r++) {
-            const int lv = sl[r];
-            if (lv == 0xff) continue;
-            const uint32_t b = sb[r], e = se[r];
-            const int o = kCellOrder[r];
-            const int sh = lv - L;
-            const u64 bd = box_d2(ux, uy, uz, (cx + o % 3 - 1) >> sh, (cy + (o / 3) % 3 - 1) >> sh,
-                                  (cz + o / 9 - 1) >> sh, lv + g.shift);
-            const u64 bound = top.at(R - 1);
-            if (bound != ~0ull && bd > bound) {
-                if (bd < hzl) hzl = bd;
-                continue;
-            }
-            // 4 candidates per lane and step, their loads issued together
-            for (uint32_t j0 = b + sub; j0 < e; j0 += 4 * SP_LANES) {
-                int4 v4[4];
-                bool ok[4];
+// A candidate's fields, loaded ahead of their use.
+struct WarpLoad {
+    int4 v;
+    u64 key;
+    uint8_t live;
+};
+// Whether it counts: live, not the query itself, below the threshold in a
+// filtered search.
+template <int FILT>
+__device__ __forceinline__ bool warp_counts(const WarpLoad& c, uint32_t j, int q, u64 tp, int ti) {
+    const bool ok = c.live && (int)j != q;
+    return FILT == FILT_NONE ? ok : ok && key_gt(tp, ti, c.key, c.v.w);
+}
+
+// The 32 nearest so far, sorted across the lanes, in the order (d^2, tie): the
+// tie is the input index with W, the Morton position otherwise.  More
+// candidates than SORT_AT in one step are sorted and merged (about 170
+// instructions) rather than inserted one by one (about 12 each).
+template <bool W, bool PACK>
+struct WarpList {
+    static const int SORT_AT = 12;
+    WarpKey<PACK> best, last, cap;  // last: the least of cap and the S-th key
+    int bpid;
+    // cap_d, cap_t: no key above this one is wanted (cap_d ~0: no cap)
+    __device__ __forceinline__ void init(u64 cap_d, uint32_t cap_t) {
+        best = WarpKey<PACK>::none();
+        cap = best;
+        if (cap_d != ~0ull) {
+            cap = WarpKey<PACK>::make(cap_d, cap_t);
+            if (PACK) cap.d++;
+            else cap.t++;
+        }
+        last = cap;
+        bpid = -1;
+    }
+    __device__ __forceinline__ u64 bound() const { return last.dist(); }
+    __device__ __forceinline__ u64 dist() const { return best.dist(); }
+    __device__ __forceinline__ bool has() const { return best.has(); }
+    __device__ __forceinline__ int id() const { return W ? bpid : (int)best.tie(); }
+    __device__ __forceinline__ uint32_t tie() const { return best.tie(); }
+    __device__ __forceinline__ void take(bool ok, const int4& v, uint32_t j, const int4& qp, int S,
+                                         int lane) {
+        u64 dd;
+        if (PACK) {
+            const int dx = v.x - qp.x, dy = v.y - qp.y, dz = v.z - qp.z;
+            dd = (u64)((uint32_t)(dx * dx) + (uint32_t)(dy * dy) + (uint32_t)(dz * dz));
+        } else {
+            dd = sqd(v, qp);
+        }
+        WarpKey<PACK> c =
+            ok ? WarpKey<PACK>::make(dd, W ? (uint32_t)v.w : j) : WarpKey<PACK>::none();
+        int cpid = (int)j;
+        unsigned m = __ballot_sync(FULLM, c.less(last));
+        if (!m) return;
+        if (__popc(m) > SORT_AT) {
 #pragma unroll
-                for (int w = 0; w < 4; w++) {
-                    const uint32_t j = j0 + (uint32_t)(w * SP_LANES);
-                    ok[w] = j < e && (int)j != q;
-                    v4[w] = ok[w] ? g.pos[j] : make_int4(0, 0, 0, 0);
-                    if (ok[w] && a.alive) ok[w] = a.alive[j] != 0;
-                }
+            for (int k = 2; k <= 32; k <<= 1) {
 #pragma unroll
-                for (int w = 0; w < 4; w++) {
-                    if (!ok[w]) continue;
-                    const int j = (int)(j0 + (uint32_t)(w * SP_LANES));
-                    u64 dd;
-                    if (PACK) {
-                        const int dx = v4[w].x - qp.x, dy = v4[w].y - qp.y, dz = v4[w].z - qp.z;
-                        dd = (u64)((uint32_t)(dx * dx) + (uint32_t)(dy * dy) + (uint32_t)(dz * dz));
-                    } else {
-                        const long long dx = (long long)v4[w].x - qp.x,
-                                        dy = (long long)v4[w].y - qp.y,
-                                        dz = (long long)v4[w].z - qp.z;
-                        dd = (u64)(dx * dx + dy * dy + dz * dz);
-                    }
-                    const int co = W ? v4[w].w : j;
-                    if (top.beats_last(dd, j, co)) top.insert(dd, j, co);
+                for (int i = k >> 1; i > 0; i >>= 1) {
+                    const WarpKey<PACK> o = c.across(i);
+                    const int op = W ? __shfl_xor_sync(FULLM, cpid, i) : 0;
+                    const bool low = ((lane & k) == 0) == ((lane & i) == 0);
+                    const bool sw = low ? o.less(c) : c.less(o);
+                    c = sw ? o : c;
+                    if (W) cpid = sw ? op : cpid;
+                }
+            }
+            {   // the 32 least of both lists, a bitonic sequence
+                const WarpKey<PACK> o = c.across(31);
+                const int op = W ? __shfl_xor_sync(FULLM, cpid, 31) : 0;
+                const bool sw = o.less(best);
+                best = sw ? o : best;
+                if (W) bpid = sw ? op : bpid;
+            }
+#pragma unroll
+            for (int i = 16; i > 0; i >>= 1) {
+                const WarpKey<PACK> o = best.across(i);
+                const int op = W ? __shfl_xor_sync(FULLM, bpid, i) : 0;
+                const bool sw = (lane & i) == 0 ? o.less(best) : best.less(o);
+                best = sw ? o : best;
+                if (W) bpid = sw ? op : bpid;
+            }
+        } else {
+            while (m) {
+                const int src = __ffs(m) - 1;
+                m &= m - 1;
+                const WarpKey<PACK> k = c.from(src);
+                const int kp = W ? __shfl_sync(FULLM, cpid, src) : 0;
+                const WarpKey<PACK> prev = best.before();
+                const int pp = W ? __shfl_up_sync(FULLM, bpid, 1) : 0;
+                if (k.less(best)) {
+                    const bool here = lane == 0 || !k.less(prev);
+                    best = here ? k : prev;
+                    if (W) bpid = here ? kp : pp;
                 }
             }
         }
+        last = best.from(S - 1);
+        if (cap.less(last)) last = cap;
     }
-    // merge the 4 partial lists and horizons of each query (all lanes take part)
-    for (int off = SP_LANES >> 1; off >= 1; off >>= 1) {
-        top.merge_xor(off, todo);
-        const u64 ho = __shfl_xor_sync(FULLM, hzl, off);
-        hzl = ho < hzl ? ho : hzl;
-    }
-    if (todo) {
-        const u64 gg = L >= g.B ? ~0ull : gap2(g, ux, uy, uz, L, cx, cy, cz);
-        const u64 bound = top.at(R - 1);
-        if (gg == ~0ull || bound < gg) {
-            todo = false;
-            if (sub == 0) write_result<S, FILT_NONE, W>(a, q, top, hzl < gg ? hzl : gg);
-        }
-    }
-}
+};
 
-template <int S, bool W>
-__global__ void __launch_bounds__(PD_WARPS * 32) knn_sparse_kernel(GridView g, KnnArgs a,
-                                                                  const int* __restrict__ list,
-                                                                  const int* __restrict__ count) {
-    __shared__ uint32_t s_b[PD_WARPS][SP_SLOTS][27], s_e[PD_WARPS][SP_SLOTS][27];
-    __shared__ uint8_t s_l[PD_WARPS][SP_SLOTS][28];
-    const int lane = threadIdx.x & 31, sub = lane & (SP_LANES - 1), slot = lane / SP_LANES;
-    const int w = threadIdx.x >> 5;
-    uint32_t* sb = s_b[w][slot];
-    uint32_t* se = s_e[w][slot];
-    uint8_t* sl = s_l[w][slot];
-    const int nq = *count;
-    const int wid = blockIdx.x * PD_WARPS + w;
-    const int nwarps = gridDim.x * PD_WARPS;
-    const int R = a.r_exact > 0 && a.r_exact < S ? a.r_exact : S;
-    for (int base = wid * SP_SLOTS; base < nq; base += nwarps * SP_SLOTS) {  // warp-uniform
-        const int qs = base + slot;
-        const int q = qs < nq ? list[qs] : -1;
-        bool todo = q >= 0;
-        int4 qp = make_int4(0, 0, 0, 0);
-        u64 c0 = 0;
-        int L = 0;
-        if (todo) {
-            qp = g.pos[q];
-            c0 = g.code[q];
-            L = g.leaf[q];
-        }
-        const int ux = qp.x - g.origin.x, uy = qp.y - g.origin.y, uz = qp.z - g.origin.z;
-        while (__any_sync(FULLM, todo)) {
-            int cx = 0, cy = 0, cz = 0;
-            if (L < g.B) {
-                cx = (int)compact3(c0 >> (3 * L));
-                cy = (int)compact3(c0 >> (3 * L + 1));
-                cz = (int)compact3(c0 >> (3 * L + 2));
-            }
-            // resolve the 27 cells into shared memory, the lanes of a query
-            // taking every SP_LANES-th one
-            bool small = true;  // every range of this lane within 3 cells of 2^13 mm
-            if (todo) {
-                const int lim = 1 << (g.B - L);  // todo lanes have L < B or L == B
-                for (int r = sub; r < 27; r += SP_LANES) {
-                    const int o = kCellOrder[r];
-                    const int ex = cx + o % 3 - 1, ey = cy + (o / 3) % 3 - 1, ez = cz + o / 9 - 1;
-                    uint32_t b = 0, e = 0;
-                    int rl = L;
-                    int rt = resolve_cell(g, L, ex, ey, ez, b, e, &rl);
-                    if (rt == 2) {
-                        // a coarse leaf covers every cell that agrees with this one
-                        // above its level: keep it at the first such cell only
-                        const int sh = rl - L;
-                        for (int r2 = 0; r2 < r; r2++) {
-                            const int o2 = kCellOrder[r2];
-                            const int fx = cx + o2 % 3 - 1, fy = cy + (o2 / 3) % 3 - 1,
-                                      fz = cz + o2 / 9 - 1;
-                            if (fx < 0 || fy < 0 || fz < 0 || fx >= lim || fy >= lim || fz >= lim)
-                                continue;
-                            if ((fx >> sh) == (ex >> sh) && (fy >> sh) == (ey >> sh) &&
-                                (fz >> sh) == (ez >> sh)) {
-                                rt = 0;
-                                break;
-                            }
-                        }
-                    }
-                    sb[r] = b;
-                    se[r] = e;
-                    sl[r] = rt ? (uint8_t)rl : (uint8_t)0xff;
-                    if (rt && rl + g.shift > 13) small = false;
+// The same without an order among equal distances (a density cost does not
+// depend on it: whichever of several equally far points is stored, the others
+// lie at the horizon), for levels with d^2 < 2^27: a step is sorted as one
+// 32-bit key per lane (d^2 << 5 | lane), a third of the instructions, and the
+// positions follow from the lane.
+struct WarpList32 {
+    static const int SORT_AT = 6;
+    uint32_t best, last, cap;
+    int bid;
+    __device__ __forceinline__ void init(u64 cap_d, uint32_t) {
+        best = ~0u;
+        bid = -1;
+        cap = cap_d < (1u << 27) ? (uint32_t)cap_d + 1 : ~0u;
+        last = cap;
+    }
+    __device__ __forceinline__ u64 bound() const { return last == ~0u ? ~0ull : last; }
+    __device__ __forceinline__ u64 dist() const { return best == ~0u ? ~0ull : best; }
+    __device__ __forceinline__ bool has() const { return best != ~0u; }
+    __device__ __forceinline__ int id() const { return bid; }
+    __device__ __forceinline__ uint32_t tie() const { return 0; }
+    __device__ __forceinline__ void merge(int o_, int lane) {
+        const uint32_t o = __shfl_xor_sync(FULLM, best, o_);
+        const int oi = __shfl_xor_sync(FULLM, bid, o_);
+        const bool sw = (lane & o_) == 0 ? o < best : best < o;
+        best = sw ? o : best;
+        bid = sw ? oi : bid;
+    }
+    __device__ __forceinline__ void take(bool ok, const int4& v, uint32_t j, const int4& qp, int S,
+                                         int lane) {
+        const int dx = v.x - qp.x, dy = v.y - qp.y, dz = v.z - qp.z;
+        const uint32_t dd = (uint32_t)(dx * dx) + (uint32_t)(dy * dy) + (uint32_t)(dz * dz);
+        const bool in = ok && dd < last;
+        unsigned m = __ballot_sync(FULLM, in);
+        if (!m) return;
+        if (__popc(m) > SORT_AT) {
+            uint32_t key = in ? (dd << 5) | lane : ~0u;
+#pragma unroll
+            for (int k = 2; k <= 32; k <<= 1) {
+#pragma unroll
+                for (int i = k >> 1; i > 0; i >>= 1) {
+                    const uint32_t o = __shfl_xor_sync(FULLM, key, i);
+                    const bool low = ((lane & k) == 0) == ((lane & i) == 0);
+                    key = low ? min(key, o) : max(key, o);
                 }
             }
-            const bool pack = __all_sync(FULLM, small);
-            __syncwarp();
-            if (pack)
-                sparse_level<S, W, TopPack<S, W>, true>(g, a, R, q, qp, ux, uy, uz, L, cx, cy, cz,
-                                                        sub, todo, sb, se, sl);
-            else
-                sparse_level<S, W, TopList<S, W>, false>(g, a, R, q, qp, ux, uy, uz, L, cx, cy,
-                                                         cz, sub, todo, sb, se, sl);
-            __syncwarp();
-            L++;
+            uint32_t d = key == ~0u ? ~0u : key >> 5;
+            int id = __shfl_sync(FULLM, (int)j, (int)(key & 31));
+            if (__shfl_sync(FULLM, best, 0) == ~0u) {  // the first points
+                best = d;
+                bid = id;
+            } else {
+                // the least of both lists, a bitonic sequence (8 or 32 lanes of it)
+                const int f = S <= 8 ? 7 : 31;
+                d = __shfl_xor_sync(FULLM, d, f);
+                id = __shfl_xor_sync(FULLM, id, f);
+                const bool sw = d < best;
+                best = sw ? d : best;
+                bid = sw ? id : bid;
+                if (S > 8) {
+                    merge(16, lane);
+                    merge(8, lane);
+                }
+                merge(4, lane);
+                merge(2, lane);
+                merge(1, lane);
+            }
+        } else {
+            while (m) {
+                const int src = __ffs(m) - 1;
+                m &= m - 1;
+                const uint32_t k = __shfl_sync(FULLM, dd, src);
+                const int kid = __shfl_sync(FULLM, (int)j, src);
+                const uint32_t prev = __shfl_up_sync(FULLM, best, 1);
+                const int pid = __shfl_up_sync(FULLM, bid, 1);
+                if (k < best) {
+                    const bool here = lane == 0 || k >= prev;
+                    best = here ? k : prev;
+                    bid = here ? kid : pid;
+                }
+            }
+        }
+        last = min(cap, __shfl_sync(FULLM, best, S - 1));
+    }
+};
+
+struct WarpRanges {  // non-empty ranges laid end to end
+    uint32_t first[33];  // prefix counts
+    uint32_t start[32];
+};
+
+template <int FILT>
+__device__ __forceinline__ WarpLoad warp_load(const GridView& g, const KnnArgs& a, bool in,
+                                              uint32_t j) {
+    WarpLoad c;
+    c.v = make_int4(0, 0, 0, 0);
+    c.key = 0;
+    c.live = 0;
+    if (in) {
+        c.v = g.pos[j];
+        c.live = a.alive[j];
+        if (FILT != FILT_NONE) c.key = a.prim[j];
+    }
+    return c;
+}
+// Nodes of at most this many points are scanned; larger ones are entered by
+// their children, nearest box first, and only where the box reaches the S-th
+// distance so far: a sparse point next to a dense region (far returns, scan
+// edges) would otherwise read the whole region.  Filtered searches scan up to
+// the second limit, 1024 positions a step, by the chunks' least keys.
+#define WARP_SCAN 64
+#define WARP_SCAN_FILT 2048
+
+// The 32 nearest so far of one warp's query and how candidates join them.
+template <int FILT, class List>
+struct WarpSearch {
+    const GridView& g;
+    const KnnArgs& a;
+    const int q, S, lane;
+    const int4 qp;
+    const u64 tp;
+    const int ti;
+    WarpRanges& wr;
+    List top;
+
+    __device__ __forceinline__ WarpSearch(const GridView& g_, const KnnArgs& a_, int q_, int S_,
+                                          int lane_, int4 qp_, u64 tp_, int ti_, WarpRanges& wr_)
+        : g(g_), a(a_), q(q_), S(S_), lane(lane_), qp(qp_), tp(tp_), ti(ti_), wr(wr_) {}
+    __device__ __forceinline__ void take(const WarpLoad& c, uint32_t j) {
+        top.take(warp_counts<FILT>(c, j, q, tp, ti), c.v, j, qp, S, lane);
+    }
+    // the lanes' ranges [b, b + cnt), laid end to end
+    __device__ __forceinline__ void scan(uint32_t b, uint32_t cnt) {
+        const unsigned act = __ballot_sync(FULLM, cnt > 0);
+        if (!act) return;
+        const uint32_t inc = warp_inclusive(cnt, lane);
+        const uint32_t total = __shfl_sync(FULLM, inc, 31);
+        __syncwarp();  // the previous scan's readers are done
+        if (cnt) {
+            const int at = __popc(act & ((1u << lane) - 1u));
+            wr.first[at] = inc - cnt;
+            wr.start[at] = b;
+        }
+        if (lane == 0) wr.first[__popc(act)] = total;
+        __syncwarp();
+        int r = 0;
+        uint32_t t = lane;
+        auto place = [&](uint32_t x) -> uint32_t {  // x ascends from call to call
+            while (x >= wr.first[r + 1]) r++;
+            return wr.start[r] + (x - wr.first[r]);
+        };
+        uint32_t jn = t < total ? place(t) : 0;
+        WarpLoad next = warp_load<FILT>(g, a, t < total, jn);
+        for (uint32_t base = 0; base < total; base += 32) {  // warp-uniform
+            const WarpLoad cur = next;
+            const uint32_t j = jn;
+            t += 32;
+            jn = t < total ? place(t) : 0;
+            next = warp_load<FILT>(g, a, t < total, jn);
+            take(cur, j);
         }
     }
-}
-
-// One warp per aligned chunk of 32 Morton positions: the least live key primary.
-__global__ void chunk_min_kernel(const u64* __restrict__ prim, const uint8_t* __restrict__ alive,
-                                 int64_t n, u64* cmin) {
-    int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int lane = threadIdx.x & 31;
-    int64_t nc = (n + 31) >> 5;
-    if (c >= nc) return;  // whole warps leave together
-    int64_t j = c * 32 + lane;
-    u64 v = (j < n && alive[j]) ? prim[j] : ~0ull;
-    for (int off = 16; off; off >>= 1) {
-        u64 o = __shfl_xor_sync(FULLM, v, off);
-        v = o < v ? o : v;
+    // one long range, the chunks of 32 without a key below the threshold skipped
+    __device__ __forceinline__ void scan_chunks(uint32_t b, uint32_t e) {
+        for (uint32_t c0 = b >> 5; c0 <= (e - 1) >> 5; c0 += 32) {
+            const uint32_t ch = c0 + lane;
+            unsigned m = __ballot_sync(FULLM, ch <= (e - 1) >> 5 && a.cmin[ch] <= tp);
+            while (m) {
+                const uint32_t j = (c0 + (uint32_t)__ffs(m) - 1) * 32 + lane;
+                m &= m - 1;
+                take(warp_load<FILT>(g, a, j >= b && j < e, j), j);
+            }
+        }
     }
-    if (lane == 0) cmin[c] = v;
-}
-
-// Append every group holding a flagged query to glist (one atomic per warp).
-__global__ void flagged_groups_kernel(const int4* __restrict__ groups, int ngroups,
-                                      const uint8_t* __restrict__ qflag, int* glist, int* gcount) {
-    int gid = blockIdx.x * blockDim.x + threadIdx.x;
-    bool any = false;
-    if (gid < ngroups) {
-        int4 G = groups[gid];
-        for (int i = 0; i < G.y && !any; i++) any = qflag[G.x + i] != 0;
+    // the points of the lanes' nodes (put: which lanes hold one to scan now)
+    __device__ __forceinline__ void scan_nodes(const WarpNode& n, bool put) {
+        const uint32_t cnt = put ? n.count() : 0;
+        if (FILT == FILT_NONE) {
+            scan(n.b, cnt);
+        } else {
+            scan(n.b, cnt <= WARP_SCAN ? cnt : 0);
+            unsigned m = __ballot_sync(FULLM, cnt > WARP_SCAN);
+            while (m) {
+                const int src = __ffs(m) - 1;
+                m &= m - 1;
+                const u64 bx = __shfl_sync(FULLM, n.box, src);
+                if (bx > top.bound()) continue;
+                scan_chunks(__shfl_sync(FULLM, n.b, src), __shfl_sync(FULLM, n.e, src));
+            }
+        }
     }
-    const int slot = block_append(any, gcount);
-    if (any) glist[slot] = gid;
+    // every candidate of the cells in n that can be among the S nearest
+    __device__ __forceinline__ void search(WarpNode n, int ux, int uy, int uz) {
+        const uint32_t lim = FILT == FILT_NONE ? WARP_SCAN : WARP_SCAN_FILT;
+        bool held = n.count() > lim && n.lv > 0;
+        // the cell and its face neighbours first; their S-th distance then rules
+        // out most of the edge and corner cells
+        bool now = !held && n.count() > 0;
+        scan_nodes(n, now && lane < 7);
+        now = now && lane >= 7 && n.box <= top.bound();
+        scan_nodes(n, now);
+        for (;;) {
+            held = held && n.box <= top.bound();
+            u64 near = held ? (n.box << 5) | lane : ~0ull;  // box < 2^52
+            if (__all_sync(FULLM, near == ~0ull)) break;
+            for (int o = 16; o; o >>= 1) {
+                const u64 v = __shfl_xor_sync(FULLM, near, o);
+                near = v < near ? v : near;
+            }
+            const int src = (int)(near & 31);
+            const WarpNode c = warp_children(g, n, src, ux, uy, uz, lane);
+            if (lane == src) held = false;
+            now = c.count() > 0 && c.box <= top.bound();
+            bool keep = now && c.count() > lim && c.lv > 0;
+            const bool was = keep;
+            warp_keep(n, held, c, keep, lane);
+            if (was && !keep) now = false;  // kept for later; no room: scanned now
+            scan_nodes(c, now);
+        }
+    }
+};
+
+// One search level of one query; returns true when its R nearest are exact.
+template <int FILT, bool W, class List>
+__device__ __forceinline__ bool warp_level(const GridView& g, const KnnArgs& a, int q, int4 qp,
+                                           int S, int R, u64 tp, int ti, WarpRanges& wr,
+                                           const WarpNode& n, int ux, int uy, int uz, u64 gg,
+                                           u64& cap_d, uint32_t& cap_t, int lane) {
+    WarpSearch<FILT, List> ws(g, a, q, S, lane, qp, tp, ti, wr);
+    ws.top.init(cap_d, cap_t);
+    ws.search(n, ux, uy, uz);
+    const List& top = ws.top;
+    const u64 dl = top.dist();
+    const u64 bound = __shfl_sync(FULLM, dl, R - 1);
+    if (!(gg == ~0ull || bound < gg)) {
+        cap_d = __shfl_sync(FULLM, dl, S - 1);
+        cap_t = __shfl_sync(FULLM, top.tie(), S - 1);
+        return false;
+    }
+    // lane i holds the i-th nearest
+    const bool has = top.has() && lane < S;
+    const u64 d = has ? dl : ~0ull;
+    const int id = has ? top.id() : -1;
+    const int found = __popc(__ballot_sync(FULLM, has));
+    if (FILT == FILT_BELOW_TAU) {
+        if (lane == 0) a.lam_out[q] = bound;  // R = k
+        return true;
+    }
+    if (FILT == FILT_NONE && lane < S) a.nbr[(int64_t)q * S + lane] = id;
+    if (FILT == FILT_NONE && a.density_k1) {
+        const u64 d0 = __shfl_sync(FULLM, d, 0), ds = __shfl_sync(FULLM, d, S - 1);
+        const int shell = __popc(__ballot_sync(FULLM, has && d == d0));
+        if (lane == 0) {
+            if (!W && a.nbr0_out) a.nbr0_out[q] = id;
+            a.prim_out[q] = key_prim_d2(d0);
+            a.rk2_out[q] = d0;
+            a.flg_out[q] = (uint8_t)((shell >= 2 ? 1 : 0) | (shell == S ? 2 : 0) | (shell << 2));
+            // every live point closer than the cube's faces and the S-th was seen
+            a.hz_out[q] = gg < ds ? gg : ds;
+        }
+        return true;
+    }
+    // the terms side by side, the sum in order (each operation rounded)
+    const double term =
+        has && lane < a.k ? __ddiv_rn(nbr_weight(a, q, id), (double)d) : 0.0;
+    double c = 0.0;
+    for (int i = 0; i < a.k && i < found; i++) c = __dadd_rn(c, __shfl_sync(FULLM, term, i));
+    const u64 prim = key_prim_cost(c);
+    if (FILT == FILT_BELOW_SELF) {
+        // condition (A): the cost over the smaller keys is the cost itself
+        if (lane == 0 && prim == a.prim[q]) {
+            a.inP[q] = 1;
+            atomicOr(&a.inPb[q >> 5], 1u << (q & 31));
+            a.cand[atomicAdd(a.ncand, 1)] = q;
+        }
+        return true;
+    }
+    const u64 dk = __shfl_sync(FULLM, d, a.k - 1);
+    const u64 dn = __shfl_sync(FULLM, d, a.k), ds = __shfl_sync(FULLM, d, S - 1);
+    if (lane == 0) {
+        a.prim_out[q] = prim;
+        a.rk2_out[q] = dk;
+        a.flg_out[q] = (uint8_t)(found > a.k && dn == dk ? 1 : 0);
+        a.hz_out[q] = ds;
+    }
+    return true;
 }
 
-template <int S, int FILT>
-static cudaError_t launch_knn_t(const GridView& g, const KnnArgs& a, cudaStream_t st) {
-    if (a.ngroups <= 0) return cudaSuccess;
-    unsigned blocks = (unsigned)((a.ngroups + PD_WARPS - 1) / PD_WARPS);
-    // list mode: a persistent grid (about 6 resident blocks per SM)
-    if (a.glist && blocks > (unsigned)device_sms() * 6u) blocks = (unsigned)device_sms() * 6u;
-    if (a.glist) {
-        if (a.term != 0)
-            knn_kernel<S, FILT, true, true><<<blocks, PD_WARPS * 32, 0, st>>>(g, a);
-        else
-            knn_kernel<S, FILT, false, true><<<blocks, PD_WARPS * 32, 0, st>>>(g, a);
-    } else if (FILT == FILT_NONE) {  // full passes: one warp per group
-        if (a.term != 0)
-            knn_kernel<S, FILT_NONE, true, false><<<blocks, PD_WARPS * 32, 0, st>>>(g, a);
-        else
-            knn_kernel<S, FILT_NONE, false, false><<<blocks, PD_WARPS * 32, 0, st>>>(g, a);
+template <bool W>
+struct WarpLists {
+    typedef WarpList32 Near;
+};
+template <>
+struct WarpLists<true> {
+    typedef WarpList<true, true> Near;
+};
+
+template <int FILT, bool W>
+__device__ __forceinline__ void warp_query(const GridView& g, const KnnArgs& a, int q,
+                                           WarpRanges& wr, int lane) {
+    const int4 qp = g.pos[q];
+    const u64 c0 = g.code[q];
+    int L = g.leaf[q];
+    const int S = FILT == FILT_NONE ? a.S : a.k;
+    const int R = FILT == FILT_NONE && a.r_exact > 0 && a.r_exact < S ? a.r_exact : S;
+    const int ux = qp.x - g.origin.x, uy = qp.y - g.origin.y, uz = qp.z - g.origin.z;
+    u64 tp = 0;
+    int ti = 0;
+    if (FILT == FILT_BELOW_SELF) {
+        tp = a.prim[q];
+        ti = qp.w;
+    } else if (FILT == FILT_BELOW_TAU) {
+        round_tau(a.rd, qp, tp, ti);  // packed batch: the query's own scan's
+        // fewer than k lower keys are stored, and every live point closer than
+        // the horizon is: start where the cell edge reaches it
+        const u64 h = a.hz_out[q];
+        if (h != ~0ull)
+            while (L < g.B && (1ull << (2 * (L + g.shift))) < h) L++;
+    }
+    u64 cap_d = ~0ull;  // the S-th key found so far bounds the next level's search
+    uint32_t cap_t = 0;
+    for (;; L++) {
+        const WarpNode n = warp_cells(g, L, c0, ux, uy, uz, lane);
+        const int sh = L + g.shift;
+        const u64 gg = L >= g.B ? ~0ull : gap2(g, ux, uy, uz, L, ux >> sh, uy >> sh, uz >> sh);
+        // every coordinate difference is below 3 cells: d^2 < 27 * 4^(level)
+        const bool near = __all_sync(FULLM, n.lv + g.shift <= (W ? 13 : 11));
+        const bool done =
+            near ? warp_level<FILT, W, typename WarpLists<W>::Near>(
+                       g, a, q, qp, S, R, tp, ti, wr, n, ux, uy, uz, gg, cap_d, cap_t, lane)
+                 : warp_level<FILT, W, WarpList<W, false>>(g, a, q, qp, S, R, tp, ti, wr, n, ux,
+                                                           uy, uz, gg, cap_d, cap_t, lane);
+        if (done || L >= g.B) break;
+    }
+}
+
+// FILTERED: qlist holds the points whose cost over smaller keys is wanted
+// (condition (A)), qlist2 the danger sources whose lambda is wanted.
+template <bool FILTERED, bool W>
+// 10 blocks per SM (48 registers) without weights, 8 with: the chain of
+// dependent loads wants warps in flight (100M-point scan, searches of all rounds:
+// 40.6 ms at 8 blocks, 33.7 at 10, 34 at 12 with more spilled).
+__global__ void __launch_bounds__(PD_WARPS * 32, W ? 8 : 10) knn_query_kernel(GridView g, KnnArgs a) {
+    __shared__ WarpRanges s_r[PD_WARPS];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n1 = *a.qcount, n2 = FILTERED ? *a.qcount2 : 0;
+    const int step = gridDim.x * PD_WARPS;
+    for (int t = blockIdx.x * PD_WARPS + w; t < n1 + n2; t += step) {
+        if (!FILTERED) warp_query<FILT_NONE, W>(g, a, a.qlist[t], s_r[w], lane);
+        else if (t < n1) warp_query<FILT_BELOW_SELF, W>(g, a, a.qlist[t], s_r[w], lane);
+        else warp_query<FILT_BELOW_TAU, W>(g, a, a.qlist2[t - n1], s_r[w], lane);
+    }
+}
+
+cudaError_t launch_knn_queries(const GridView& g, const KnnArgs& a, int64_t cap, cudaStream_t st) {
+    if (cap <= 0) return cudaSuccess;
+    const bool filtered = a.qlist2 != nullptr;
+    int64_t blocks = (cap + PD_WARPS - 1) / PD_WARPS;
+    const int64_t lim = (int64_t)device_sms() * 10;
+    if (blocks > lim) blocks = lim;
+    const dim3 gr((unsigned)blocks), bl(PD_WARPS * 32);
+    if (filtered) {
+        if (a.term != 0) knn_query_kernel<true, true><<<gr, bl, 0, st>>>(g, a);
+        else knn_query_kernel<true, false><<<gr, bl, 0, st>>>(g, a);
     } else {
-        return cudaErrorInvalidValue;  // filtered searches always run over a group list
+        if (a.term != 0) knn_query_kernel<false, true><<<gr, bl, 0, st>>>(g, a);
+        else knn_query_kernel<false, false><<<gr, bl, 0, st>>>(g, a);
     }
     note_launch();
     return cudaGetLastError();
@@ -862,66 +1076,16 @@ static cudaError_t launch_knn_t(const GridView& g, const KnnArgs& a, cudaStream_
 
 template <int S>
 static cudaError_t launch_knn_s(const GridView& g, const KnnArgs& a, cudaStream_t st) {
-    switch (a.filter) {
-        case FILT_NONE: return launch_knn_t<S, FILT_NONE>(g, a, st);
-        case FILT_BELOW_SELF: return launch_knn_t<S, FILT_BELOW_SELF>(g, a, st);
-        default: return launch_knn_t<S, FILT_BELOW_TAU>(g, a, st);
-    }
-}
-
-cudaError_t launch_chunk_min(const u64* prim, const uint8_t* alive, int64_t n, u64* cmin,
-                             cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    int64_t threads = ((n + 31) >> 5) * 32;
-    chunk_min_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(prim, alive, n, cmin);
-    note_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t launch_knn_flagged(const GridView& g, const KnnArgs& a, int* glist, int* gcount,
-                               cudaStream_t st) {
     if (a.ngroups <= 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(gcount, 0, sizeof(int), st);
-    if (e) return e;
-    flagged_groups_kernel<<<(unsigned)((a.ngroups + 255) / 256), 256, 0, st>>>(
-        a.groups, a.ngroups, a.qflag, glist, gcount);
-    note_launch();
-    KnnArgs b = a;
-    b.glist = glist;
-    b.gcount = gcount;
-    return launch_knn(g, b, st);
-}
-
-template <int S>
-static cudaError_t launch_sparse_s(const GridView& g, const KnnArgs& a, const int* list,
-                                   const int* count, int64_t cap, cudaStream_t st) {
-    int64_t warps = (cap + 32 / SP_LANES - 1) / (32 / SP_LANES);
-    int64_t blocks = (warps + PD_WARPS - 1) / PD_WARPS;
-    int64_t lim = (int64_t)device_sms() * 12;
-    if (blocks > lim) blocks = lim;
-    if (blocks < 1) blocks = 1;
-    if (a.term != 0)
-        knn_sparse_kernel<S, true><<<(unsigned)blocks, PD_WARPS * 32, 0, st>>>(g, a, list, count);
-    else
-        knn_sparse_kernel<S, false><<<(unsigned)blocks, PD_WARPS * 32, 0, st>>>(g, a, list, count);
+    const unsigned blocks = (unsigned)((a.ngroups + PD_WARPS - 1) / PD_WARPS);
+    if (a.term != 0) knn_kernel<S, true><<<blocks, PD_WARPS * 32, 0, st>>>(g, a);
+    else knn_kernel<S, false><<<blocks, PD_WARPS * 32, 0, st>>>(g, a);
     note_launch();
     return cudaGetLastError();
-}
-
-cudaError_t launch_knn_sparse(const GridView& g, const KnnArgs& a, const int* list,
-                              const int* count, int64_t cap, cudaStream_t st) {
-    if (a.filter != FILT_NONE || cap <= 0) return cap <= 0 ? cudaSuccess : cudaErrorInvalidValue;
-    switch (a.S) {
-        case 4: return launch_sparse_s<4>(g, a, list, count, cap, st);
-        case 8: return launch_sparse_s<8>(g, a, list, count, cap, st);
-        case 17: return launch_sparse_s<17>(g, a, list, count, cap, st);
-        default: return cudaErrorInvalidValue;
-    }
 }
 
 cudaError_t launch_knn(const GridView& g, const KnnArgs& a, cudaStream_t st) {
     switch (a.S) {
-        case 4: return launch_knn_s<4>(g, a, st);
         case 8: return launch_knn_s<8>(g, a, st);
         case 17: return launch_knn_s<17>(g, a, st);
         default: return cudaErrorInvalidValue;

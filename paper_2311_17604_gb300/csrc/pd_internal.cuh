@@ -71,17 +71,16 @@ __host__ __device__ inline unsigned long long morton3(uint32_t x, uint32_t y, ui
 __device__ inline unsigned long long cell_key(unsigned long long prefix, int L, int B) {
     return (1ull << (3 * (B - L))) | prefix;
 }
-__device__ inline unsigned long long mix64(unsigned long long k) {
-    k ^= k >> 33;
-    k *= 0xff51afd7ed558ccdull;
-    k ^= k >> 33;
-    k *= 0xc4ceb9fe1a85ec53ull;
-    k ^= k >> 33;
-    return k;
+// Slot of a key: the upper half of a multiplication by 2^64 over the golden
+// ratio (Fibonacci hashing, Knuth, TAOCP vol. 3, 6.4).  A search resolves 27
+// cells and the ancestors of the empty ones, so the hash is most of its set-up:
+// one 64-bit multiplication instead of a two-multiplication finaliser.
+__device__ inline unsigned long long hash_slot(unsigned long long k, unsigned long long mask) {
+    return ((k * 0x9e3779b97f4a7c15ull) >> 32) & mask;
 }
 __device__ inline bool hash_find(const HashSlot* tab, unsigned long long mask,
                                  unsigned long long key, uint32_t& b, uint32_t& e) {
-    unsigned long long h = mix64(key) & mask;
+    unsigned long long h = hash_slot(key, mask);
     for (unsigned long long i = 0; i <= mask; i++) {
         unsigned long long k = tab[h].key;
         if (k == key) {
@@ -95,14 +94,11 @@ __device__ inline bool hash_find(const HashSlot* tab, unsigned long long mask,
     return false;
 }
 
-// Range of the level-L cell (cx,cy,cz).  Returns 0 = empty, 1 = the cell is an
-// octree node (its exact range), 2 = the cell lies inside a coarser leaf
-// (the whole leaf's range is returned; *lvl_out = that leaf's level).
-__device__ inline int resolve_cell(const GridView& g, int L, int cx, int cy, int cz,
-                                   uint32_t& b, uint32_t& e, int* lvl_out) {
-    int lim = 1 << (g.B - L);
-    if (cx < 0 || cy < 0 || cz < 0 || cx >= lim || cy >= lim || cz >= lim) return 0;
-    unsigned long long prefix = morton3((uint32_t)cx, (uint32_t)cy, (uint32_t)cz);
+// Range of the level-L cell with this Morton prefix.  Returns 0 = empty, 1 =
+// the cell is an octree node (its exact range), 2 = the cell lies inside a
+// coarser leaf (the whole leaf's range is returned; *lvl_out = that leaf's level).
+__device__ inline int resolve_prefix(const GridView& g, int L, unsigned long long prefix,
+                                     uint32_t& b, uint32_t& e, int* lvl_out) {
     if (hash_find(g.hash, g.hmask, cell_key(prefix, L, g.B), b, e)) {
         *lvl_out = L;
         return 1;
@@ -116,6 +112,32 @@ __device__ inline int resolve_cell(const GridView& g, int L, int cx, int cy, int
         }
     }
     return 0;
+}
+// The same for the cell (cx,cy,cz); 0 outside the grid.
+__device__ inline int resolve_cell(const GridView& g, int L, int cx, int cy, int cz,
+                                   uint32_t& b, uint32_t& e, int* lvl_out) {
+    int lim = 1 << (g.B - L);
+    if (cx < 0 || cy < 0 || cz < 0 || cx >= lim || cy >= lim || cz >= lim) return 0;
+    return resolve_prefix(g, L, morton3((uint32_t)cx, (uint32_t)cy, (uint32_t)cz), b, e, lvl_out);
+}
+// The prefix of the cell at offset (dx, dy, dz), each in -1..1, from the cell
+// with prefix p of 3 nb bits: additions on the interleaved bits of each axis.
+// False outside the grid.
+__device__ inline bool prefix_offset(unsigned long long& p, int nb, int dx, int dy, int dz) {
+    const unsigned long long full = (1ull << (3 * nb)) - 1;
+    const int d[3] = {dx, dy, dz};
+    unsigned long long out = 0;
+    bool in = true;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const unsigned long long m = (0x1249249249249249ull << a) & full;
+        const unsigned long long v = p & m;
+        if (d[a] > 0) in = in && v != m;
+        if (d[a] < 0) in = in && v != 0;
+        out |= (d[a] > 0 ? (p | ~m) + 1 : (d[a] < 0 ? v - 1 : v)) & m;
+    }
+    p = out;
+    return in;
 }
 
 // ---------------------------------------------------------------- keys
@@ -189,31 +211,6 @@ __device__ __forceinline__ void block_add(unsigned long long* dst, unsigned long
         if (t) atomicAdd(dst, t);
     }
 }
-// Two counters at once (one reduction, two atomics per block).
-__device__ __forceinline__ void block_add2(unsigned long long* d1, unsigned long long v1,
-                                           unsigned long long* d2, unsigned long long v2) {
-    __shared__ unsigned long long s_p1[32], s_p2[32];
-    for (int o = 16; o; o >>= 1) {
-        v1 += __shfl_xor_sync(0xffffffffu, v1, o);
-        v2 += __shfl_xor_sync(0xffffffffu, v2, o);
-    }
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __syncthreads();
-    if (lane == 0) {
-        s_p1[w] = v1;
-        s_p2[w] = v2;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long t1 = 0, t2 = 0;
-        for (int i = 0; i < (int)(blockDim.x >> 5); i++) {
-            t1 += s_p1[i];
-            t2 += s_p2[i];
-        }
-        if (t1) atomicAdd(d1, t1);
-        if (t2) atomicAdd(d2, t2);
-    }
-}
 // Appends for every thread with want set; returns the thread's slot in the
 // list (meaningful where want is set).
 __device__ __forceinline__ int block_append(bool want, int* count) {
@@ -236,6 +233,41 @@ __device__ __forceinline__ int block_append(bool want, int* count) {
     return s_w[32] + s_w[w] + __popc(m & ((1u << lane) - 1u));
 }
 
+// Appends to N lists at once: two block barriers for all of them instead of
+// three per list.  slot[i] is meaningful where want[i] is set.
+template <int N>
+__device__ __forceinline__ void block_append_n(const bool (&want)[N], int* const (&count)[N],
+                                               int (&slot)[N]) {
+    __shared__ int s_w[N][33];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    unsigned m[N];
+#pragma unroll
+    for (int i = 0; i < N; i++) m[i] = __ballot_sync(0xffffffffu, want[i]);
+    __syncthreads();  // s_w may still be read by a previous call
+    if (lane == 0) {
+#pragma unroll
+        for (int i = 0; i < N; i++) s_w[i][w] = __popc(m[i]);
+    }
+    __syncthreads();
+    if (threadIdx.x < N) {
+        int acc = 0;
+        for (int i = 0; i < (int)(blockDim.x >> 5); i++) {
+            const int c = s_w[threadIdx.x][i];
+            s_w[threadIdx.x][i] = acc;
+            acc += c;
+        }
+        int* dst = count[0];
+#pragma unroll
+        for (int i = 1; i < N; i++)
+            if ((int)threadIdx.x == i) dst = count[i];
+        s_w[threadIdx.x][32] = acc ? atomicAdd(dst, acc) : 0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < N; i++)
+        slot[i] = s_w[i][32] + s_w[i][w] + __popc(m[i] & ((1u << lane) - 1u));
+}
+
 // Streaming multiprocessors of the current device (queried once per device
 // and cached); persistent and grid-stride launches size their grids from it.
 int device_sms();
@@ -248,5 +280,120 @@ __device__ inline int warp_lane() { return threadIdx.x & 31; }
 // (cell o = (dx+1) + 3 (dy+1) + 9 (dz+1)).  Nearer cells first tighten the
 // k-th distance bound early, which prunes more of the farther cells.
 static __device__ __constant__ const unsigned char kCellOrder[27] = {13, 4, 10, 12, 14, 16, 22, 1, 3, 5, 7, 9, 11, 15, 17, 19, 21, 23, 25, 0, 2, 6, 8, 18, 20, 24, 26};
+
+
+// Squared distance from a point (relative to the grid's origin) to the box of
+// cell (bx, by, bz) with edge 2^sh; 0 inside.
+__device__ __forceinline__ unsigned long long box_d2(int ux, int uy, int uz, int bx, int by,
+                                                     int bz, int sh) {
+    const int q[3] = {ux, uy, uz};
+    const int c[3] = {bx, by, bz};
+    unsigned long long s = 0;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        // coordinates and cell faces are below 2^27, so the gap is an int
+        const int lo = c[a] << sh, hi = lo + ((1 << sh) - 1);
+        const int d = max(max(lo - q[a], q[a] - hi), 0);
+        s += (unsigned long long)((long long)d * d);
+    }
+    return s;
+}
+
+// ---------------------------------------------------------------- one warp, one point
+// An octree node held by one lane: positions [b, e), its level and cell, and
+// the squared distance from the warp's point to its box.  b == e: none.
+struct WarpNode {
+    uint32_t b, e;
+    int lv, x, y, z;
+    unsigned long long box;
+    __device__ __forceinline__ uint32_t count() const { return e - b; }
+};
+
+// Lane i < 27 takes the level-L cell kCellOrder[i] of the cube around the cell
+// of the point (ux, uy, uz) with Morton code c0; a coarser leaf reached from
+// several cells is kept once.
+__device__ __forceinline__ WarpNode warp_cells(const GridView& g, int L, unsigned long long c0,
+                                               int ux, int uy, int uz, int lane) {
+    WarpNode n;
+    const int o = lane < 27 ? kCellOrder[lane] : 13;
+    const int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
+    n.lv = L;
+    n.b = n.e = 0;
+    n.x = n.y = n.z = 0;
+    n.box = ~0ull;
+    unsigned long long prefix = L < g.B ? c0 >> (3 * L) : 0;
+    int rt = 0;
+    if (lane < 27 && prefix_offset(prefix, g.B - L, dx, dy, dz))
+        rt = resolve_prefix(g, L, prefix, n.b, n.e, &n.lv);
+    const unsigned same = __match_any_sync(0xffffffffu, rt == 2 ? n.b : 0x80000000u + lane);
+    if (rt == 2 && __ffs(same) - 1 != lane) rt = 0;
+    if (rt) {
+        const int sh = L + g.shift, up = n.lv - L;
+        n.x = ((ux >> sh) + dx) >> up;
+        n.y = ((uy >> sh) + dy) >> up;
+        n.z = ((uz >> sh) + dz) >> up;
+        n.box = box_d2(ux, uy, uz, n.x, n.y, n.z, n.lv + g.shift);
+    } else {
+        n.b = n.e = 0;
+        n.lv = L;
+    }
+    return n;
+}
+
+// Lane i < 8 takes child i of lane src's node (above level 0).
+__device__ __forceinline__ WarpNode warp_children(const GridView& g, const WarpNode& n, int src,
+                                                  int ux, int uy, int uz, int lane) {
+    WarpNode c;
+    c.lv = __shfl_sync(0xffffffffu, n.lv, src) - 1;
+    c.x = 2 * __shfl_sync(0xffffffffu, n.x, src) + (lane & 1);
+    c.y = 2 * __shfl_sync(0xffffffffu, n.y, src) + ((lane >> 1) & 1);
+    c.z = 2 * __shfl_sync(0xffffffffu, n.z, src) + ((lane >> 2) & 1);
+    c.b = c.e = 0;
+    c.box = ~0ull;
+    if (lane < 8 &&
+        hash_find(g.hash, g.hmask,
+                  cell_key(morton3((uint32_t)c.x, (uint32_t)c.y, (uint32_t)c.z), c.lv, g.B), c.b,
+                  c.e))
+        c.box = box_d2(ux, uy, uz, c.x, c.y, c.z, c.lv + g.shift);
+    else
+        c.b = c.e = 0;
+    return c;
+}
+
+// The free lanes of `held` (no node kept) take the nodes of the lanes with
+// `put` set, in lane order; put is cleared where a node was taken.
+__device__ __forceinline__ void warp_keep(WarpNode& n, bool& held, const WarpNode& c, bool& put,
+                                          int lane) {
+    const unsigned pm = __ballot_sync(0xffffffffu, put), fm = __ballot_sync(0xffffffffu, !held);
+    if (!pm) return;
+    const int np = __popc(pm), nf = __popc(fm);
+    const unsigned below = (1u << lane) - 1u;
+    const int rank = __popc(fm & below);
+    const bool take = !held && rank < np;
+    const int src = take ? (int)__fns(pm, 0, rank + 1) : 0;
+    WarpNode t;
+    t.b = __shfl_sync(0xffffffffu, c.b, src);
+    t.e = __shfl_sync(0xffffffffu, c.e, src);
+    t.lv = __shfl_sync(0xffffffffu, c.lv, src);
+    t.x = __shfl_sync(0xffffffffu, c.x, src);
+    t.y = __shfl_sync(0xffffffffu, c.y, src);
+    t.z = __shfl_sync(0xffffffffu, c.z, src);
+    t.box = __shfl_sync(0xffffffffu, c.box, src);
+    if (take) {
+        n = t;
+        held = true;
+    }
+    if (put && __popc(pm & below) < nf) put = false;
+}
+
+// Inclusive prefix sum over the lanes.
+__device__ __forceinline__ uint32_t warp_inclusive(uint32_t v, int lane) {
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, v, s);
+        if (lane >= s) v += y;
+    }
+    return v;
+}
 
 }  // namespace pd

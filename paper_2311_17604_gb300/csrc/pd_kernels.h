@@ -94,7 +94,8 @@ struct RoundDev {
     int done;
     unsigned pre[8];
     int len[2];
-    int ncand, nslow, nsrc, npairs, overflow, ncs;
+    int ncand, nslow, nsrc, npairs, overflow;
+    int nreq, nfq, nlq;  // this round's re-searches, filtered and lambda searches
     int ndep;  // k = 1: candidates with a shell member of larger input index
     int changed[PD_FIX_ITERS];
     int fix_unconverged;
@@ -142,13 +143,9 @@ enum { FILT_NONE = 0, FILT_BELOW_SELF = 1, FILT_BELOW_TAU = 2 };
 struct KnnArgs {
     const int4* groups;
     int ngroups;
-    const int* list;          // list mode: group.x is an offset into list
-    const uint8_t* alive;     // NULL = every point live
-    const u64* prim;          // keys (filter modes)
-    int filter;
-    u64 tau_prim;
-    int tau_idx;
-    const RoundDev* rd;       // when set, tau is read from rd (device)
+    const uint8_t* alive;     // NULL = every point live (launch_knn only)
+    const u64* prim;          // keys (filtered searches)
+    const RoundDev* rd;       // round state: the thresholds of the lambda searches
     const uint8_t* qflag;     // when set, only flagged points of each group are queried
     int k;
     int S;                    // stored neighbours (template width)
@@ -165,34 +162,32 @@ struct KnnArgs {
     uint8_t* flg_out;
     u64* hz_out;              // horizon: S-th stored squared distance (~0 if fewer)
     double* cost_out;         // cost in Morton order (optional)
-    // outputs (filter modes)
-    u64* fprim_out;           // FILT_BELOW_SELF: key primary over lower keys
-    u64* lam_out;             // FILT_BELOW_TAU: k-th squared distance over keys < tau
     unsigned long long* pairs_out;  // optional: + (query, candidate) pairs scanned, spread
                                     //   over PD_PAIR_SLOTS counters (their sum is the count)
+    int r_exact;              // full searches: nearest entries that must be exact
+                              //   (0 = all S; the k = 1 density cost keeps the
+                              //   rest below the horizon)
+    // launch_knn_queries: the queries (Morton positions), counts on the device.
+    // qlist2 NULL: full searches of qlist.  Otherwise filtered searches: the
+    // points of qlist whose cost over smaller keys equals their own join the
+    // candidates (inP, its bitmap inPb, cand, *ncand); lam_out of those of qlist2
+    // takes the k-th squared distance over keys below the threshold.
+    const int* qlist;
+    const int* qcount;
+    const int* qlist2;
+    const int* qcount2;
+    u64* lam_out;
+    uint8_t* inP;
+    uint32_t* inPb;
+    int* cand;
+    int* ncand;
     const u64* cmin;          // filtered searches: least live key primary of every aligned
                               //   32-position chunk (chunks above the threshold are skipped)
-    const int* glist;         // group-list mode: process groups glist[0 .. *gcount)
-    const int* gcount;        //   (device count; a persistent grid walks the list)
-    int r_exact;              // full searches: nearest entries that must be exact
-                              //   (0 = all S; the k = 1 density cost re-searches
-                              //   with 1 and keeps the rest below the horizon)
 };
-// Flagged mode without a host read: list the groups that hold a flagged query
-// (a.qflag), then run the search over that list only.  glist: ngroups ints,
-// gcount: one int, both device scratch.
-// cmin[c] = least key primary of the live points at Morton positions
-// [32c, 32c + 32) (~0 when none), for the chunk skipping of filtered searches.
-cudaError_t launch_chunk_min(const u64* prim, const uint8_t* alive, int64_t n, u64* cmin,
-                             cudaStream_t st);
-cudaError_t launch_knn_flagged(const GridView& g, const KnnArgs& a, int* glist, int* gcount,
-                               cudaStream_t st);
+// Full searches of every point (a.qflag: of the flagged ones), a warp per leaf group.
 cudaError_t launch_knn(const GridView& g, const KnnArgs& a, cudaStream_t st);
-// Full (FILT_NONE) searches of the listed Morton positions list[0 .. *count)
-// (count on the device, at most cap), 2 lanes per query, each over its own
-// leaf cells: for sparse re-searches.
-cudaError_t launch_knn_sparse(const GridView& g, const KnnArgs& a, const int* list,
-                              const int* count, int64_t cap, cudaStream_t st);
+// Searches of the listed queries, one warp each; at most cap of them.
+cudaError_t launch_knn_queries(const GridView& g, const KnnArgs& a, int64_t cap, cudaStream_t st);
 // Internal neighbour-weight term: unit weights with equal distances ordered by
 // input index (the normals' 16-NN order).
 #define PD_TERM_INDEX_TIE 3
@@ -223,19 +218,19 @@ cudaError_t round_launch_k1(const GridView& g, const u64* prim, const uint8_t* a
                             const int* nbr, const int* nbr0, const uint8_t* flg, const u64* rk2,
                             int64_t n, int S, RoundDev* rd, uint8_t* inP, uint8_t* rej, int* cand,
                             int* slow, int* dep, int fix_iters, cudaStream_t st);
-cudaError_t round_launch_kk_accept(const uint8_t* fq_flag, const u64* prim, const u64* fprim,
-                                   int64_t n, RoundDev* rd, uint8_t* inP, int* cand,
-                                   cudaStream_t st);
+// inPb: bitmap of inP over the Morton positions.
 cudaError_t round_launch_danger(const GridView& g, const int* src, const u64* prim,
-                                const uint8_t* alive, const uint8_t* inP, uint8_t* rej,
+                                const uint8_t* alive, const uint32_t* inPb, uint8_t* rej,
                                 const u64* lam, const int* nbr, int S, int k, int2* pairs,
-                                int pair_cap, const int* csorted, RoundDev* rd, cudaStream_t st);
+                                int pair_cap, RoundDev* rd, cudaStream_t st);
 cudaError_t round_launch_pairs_fix(const int2* pairs, int pair_cap, const uint8_t* inP,
                                    uint8_t* rej, RoundDev* rd, cudaStream_t st);
 cudaError_t round_launch_remove(const int* cand, uint8_t* inP, uint8_t* rej, uint8_t* alive,
                                 RoundDev* rd, cudaStream_t st);
+// Lists (list[0 .. rd->nreq)) the live points that lost one of their first
+// kchk stored neighbours.
 cudaError_t round_launch_dirty(const uint8_t* alive, const int* nbr, int64_t n, int S, int kchk,
-                               uint8_t* dirty, RoundDev* rd, cudaStream_t st);
+                               int* list, RoundDev* rd, cudaStream_t st);
 struct BufView {  // the k+b neighbour buffer of every point
     const int4* pos;
     u64* prim;
@@ -251,14 +246,17 @@ struct BufView {  // the k+b neighbour buffer of every point
 };
 // k = 1 density cost: absorb removals in the stored nearest entries (the
 // shell at the new nearest distance must lie below the search horizon);
-// dirty[s] = 1 where a new search is needed.
+// list[0 .. rd->nreq) takes the points that need a new search.
 cudaError_t round_launch_k1_update(const BufView& b, const uint8_t* alive, int64_t n, int S,
-                                   uint8_t* dirty, RoundDev* rd, cudaStream_t st);
+                                   int* list, RoundDev* rd, cudaStream_t st);
 cudaError_t round_launch_kk_update(const BufView& b, const uint8_t* alive, int64_t n, int S, int k,
-                                   uint8_t* dirty, RoundDev* rd, cudaStream_t st);
+                                   int* list, RoundDev* rd, cudaStream_t st);
+// Candidates (inP, its bitmap, cand), danger sources (src, lam) and the lists
+// of the searches that the stored neighbours do not settle (fq, lq); cmin as
+// in KnnArgs.
 cudaError_t round_launch_kk_cand2(const BufView& b, const uint8_t* alive, int64_t n, int S, int k,
-                                  RoundDev* rd, uint8_t* inP, int* cand, uint8_t* fq_flag,
-                                  uint8_t* lq_flag, u64* lam, int* src, cudaStream_t st);
+                                  RoundDev* rd, uint8_t* inP, uint32_t* inPb, int* cand, int* fq,
+                                  int* lq, u64* lam, int* src, u64* cmin, cudaStream_t st);
 }  // namespace pd
 
 // ---------------------------------------------------------------- normals.cu

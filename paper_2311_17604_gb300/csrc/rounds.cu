@@ -156,83 +156,79 @@ __global__ void k1_fix_kernel(const int* __restrict__ cand, const int* __restric
     }
 }
 
-// Danger pairs.  One warp per source x: collect every live point y with
-// d^2(x,y) < lam(x) (lam = k-th squared distance from x to keys below tau),
-// then for each candidate p among them with key(p) < key(x) count the points
-// y != p of key below key(p) with d^2(x,y) <= d^2(x,p); fewer than k means p
-// could enter x's k nearest before it is popped: record (x, p).
 #define DG_CAP 512
+#define DG_SCAN 64   // larger octree nodes are entered by their children
 #define DG_WARPS 2
 #define DG_BLOCKS_PER_SM 14  // resident blocks per SM (registers capped to fit)
 #define PD_DG_SMAX 8  // stored neighbours used as shields (S up to 8)
 
-__device__ inline u64 box_d2x(int ux, int uy, int uz, int bx, int by, int bz, int sh) {
-    long long q[3] = {ux, uy, uz};
-    int c[3] = {bx, by, bz};
-    u64 s = 0;
-    for (int a = 0; a < 3; a++) {
-        long long lo = (long long)c[a] << sh;
-        long long hi = ((long long)(c[a] + 1) << sh) - 1;
-        long long d = q[a] < lo ? lo - q[a] : (q[a] > hi ? q[a] - hi : 0);
-        s += (u64)(d * d);
-    }
-    return s;
-}
-
-// Cells of the level-L cube around a point that hold every point closer than
-// sqrt(lam); returns the level (the first whose cube covers that ball).
-__device__ inline int cover_level(const GridView& g, int ux, int uy, int uz, u64 c0, int L0,
-                                  u64 lam, int& cx, int& cy, int& cz) {
-    for (int L = L0;; L++) {
-        cx = cy = cz = 0;
-        if (L >= g.B) return g.B;
-        cx = (int)compact3(c0 >> (3 * L));
-        cy = (int)compact3(c0 >> (3 * L + 1));
-        cz = (int)compact3(c0 >> (3 * L + 2));
-        int sh = L + g.shift;
-        long long q[3] = {ux, uy, uz};
-        int c[3] = {cx, cy, cz};
-        int m[3] = {g.umax.x, g.umax.y, g.umax.z};
-        long long best = -1;
+// The first level from L0 whose 3x3x3 cells around a point hold every point
+// closer than sqrt(lam).
+__device__ inline int cover_level(const GridView& g, int ux, int uy, int uz, int L0, u64 lam) {
+    for (int L = L0; L < g.B; L++) {
+        const int sh = L + g.shift;
+        const int q[3] = {ux, uy, uz};
+        const int m[3] = {g.umax.x, g.umax.y, g.umax.z};
+        int best = 0x7fffffff;
+#pragma unroll
         for (int a = 0; a < 3; a++) {
-            long long lo = (long long)(c[a] - 1) << sh, hi = (long long)(c[a] + 2) << sh;
-            if (lo > 0 && (best < 0 || q[a] - lo + 1 < best)) best = q[a] - lo + 1;
-            if (hi <= m[a] && (best < 0 || hi - q[a] < best)) best = hi - q[a];
+            const int c = q[a] >> sh;  // faces are below 2^25 + 2 * 2^25: ints
+            const int lo = (c - 1) * (1 << sh), hi = (c + 2) * (1 << sh);
+            if (lo > 0) best = min(best, q[a] - lo + 1);
+            if (hi <= m[a]) best = min(best, hi - q[a]);
         }
-        if (best < 0 || lam <= (u64)best * (u64)best) return L;
+        if (best == 0x7fffffff || lam <= (u64)((long long)best * best)) return L;
     }
+    return g.B;
 }
 
 // Danger pairs (condition (B), k >= 2).  One warp per source x (key above
 // tau, lam = k-th squared distance from x to keys below tau):
-//   1. collect the candidates p (in P so far, key below x's) with d^2(x,p) < lam;
+//   1. collect the candidates p (in P so far, key below x's) with d^2(x,p) < lam,
+//      from the candidates' bitmap over the ranges' positions (in Morton order
+//      within a range, the ranges in kCellOrder);
 //   2. for 32 candidates at a time stream every live point y with
 //      d^2(x,y) < lam and count, per candidate, the y != p with
 //      d^2(x,y) <= d^2(x,p) and key(y) < key(p), stopping once all 32 counts
 //      reach k; a count below k means p could enter x's k nearest before p is
 //      popped: record (x, p).
 // Candidates beyond the list capacity are rejected without counting.
+// A source's time is a chain of dependent loads, so the ranges are laid end to
+// end (32 bitmap words, then 32 points a step, the next step's loads issued
+// before this step's are used) instead of walked one by one, and octree nodes
+// above DG_SCAN points are entered by their children (9.8M outdoor points, k =
+// 4, 287 rounds: 95.6 -> 47.3 ms).
 struct DangerSmem {
     int c_j[DG_WARPS][DG_CAP];
     u64 c_d[DG_WARPS][DG_CAP];
-    u64 st_d[DG_WARPS][32];  // staged points within the batch's farthest candidate:
-    u64 st_k[DG_WARPS][32];  // d^2 to the source, key, input index, Morton position
-    int st_o[DG_WARPS][32];
-    int st_j[DG_WARPS][32];
+    union {
+        struct {  // staged points within the batch's farthest candidate:
+            u64 d[32], k[32];  // d^2 to the source, key, input index, Morton position
+            int o[32], j[32];
+        } st;
+        int raw[192];  // candidate positions before the distance test
+    } u[DG_WARPS];
 };
 
+// The range that holds item x of ranges laid end to end (inc: this lane's
+// inclusive prefix count); every lane must call it.
+__device__ __forceinline__ int range_of(uint32_t inc, uint32_t x) {
+    int r = 0;
+#pragma unroll
+    for (int step = 16; step; step >>= 1) {
+        const uint32_t v = __shfl_sync(FULLM, inc, r + step - 1);
+        if (v <= x) r += step;
+    }
+    return r;
+}
 __device__ void danger_one(const GridView& g, int x, const u64* __restrict__ prim,
-                           const uint8_t* __restrict__ alive, const uint8_t* __restrict__ inP,
+                           const uint8_t* __restrict__ alive, const uint32_t* __restrict__ inPb,
                            uint8_t* rej, const u64* __restrict__ lam, const int* __restrict__ nbr,
                            int S, int k, int2* pairs, int* npairs, int pair_cap, int* overflow,
-                           unsigned long long* diag, const int* __restrict__ csorted,
-                           const int* __restrict__ ncs, DangerSmem& sm, int w, int lane) {
-    int(&c_j)[DG_WARPS][DG_CAP] = sm.c_j;
-    u64(&c_d)[DG_WARPS][DG_CAP] = sm.c_d;
-    u64(&st_d)[DG_WARPS][32] = sm.st_d;
-    u64(&st_k)[DG_WARPS][32] = sm.st_k;
-    int(&st_o)[DG_WARPS][32] = sm.st_o;
-    int(&st_j)[DG_WARPS][32] = sm.st_j;
+                           unsigned long long* diag, DangerSmem& sm, int w, int lane) {
+    int(&c_j)[DG_CAP] = sm.c_j[w];
+    u64(&c_d)[DG_CAP] = sm.c_d[w];
+    auto& u = sm.u[w];
     __syncwarp();
     int4 xp = g.pos[x];
     u64 px = prim[x];
@@ -242,79 +238,64 @@ __device__ void danger_one(const GridView& g, int x, const u64* __restrict__ pri
         return;
     }
     int ux = xp.x - g.origin.x, uy = xp.y - g.origin.y, uz = xp.z - g.origin.z;
-    int cx, cy, cz;
-    int L = cover_level(g, ux, uy, uz, g.code[x], g.leaf[x], lx, cx, cy, cz);
-    int o = lane < 27 ? kCellOrder[lane] : 13;
-    int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
-    uint32_t rb = 0, re = 0;
-    int rl = L, rt = 0;
-    if (lane < 27) rt = resolve_cell(g, L, cx + dx, cy + dy, cz + dz, rb, re, &rl);
-    for (int j = 0; j < 27; j++) {
-        uint32_t bj = __shfl_sync(FULLM, rb, j);
-        int tj = __shfl_sync(FULLM, rt, j);
-        if (j < lane && rt == 2 && tj == 2 && bj == rb) rt = 0;
-    }
-    // squared distance from x to each resolved range's box: ranges entirely
-    // beyond lam (or beyond the candidates being counted) are skipped
-    u64 rbox = ~0ull;
-    if (rt) {
-        int sh = rl - L;
-        rbox = box_d2x(ux, uy, uz, (cx + dx) >> sh, (cy + dy) >> sh, (cz + dz) >> sh,
-                       rl + g.shift);
-        if (rbox >= lx) rt = 0;
-    }
-    // 1. candidates: when a Morton-sorted list of them is given, each range
-    // [b, e) maps to a slice of that list by binary search; otherwise the
-    // range's points are streamed and filtered
+    const int L = cover_level(g, ux, uy, uz, g.leaf[x], lx);
+    // nodes entirely beyond lam (or beyond the candidates being counted) are skipped
+    WarpNode cell = warp_cells(g, L, g.code[x], ux, uy, uz, lane);
+    const uint32_t rb = cell.b, re = cell.e;
+    const bool rt = cell.count() > 0 && cell.box < lx;
+    // 1. candidates
     int nc = 0;
-    uint32_t cs_lo = 0, cs_hi = 0;
-    if (csorted && rt) {
-        int nlist = *ncs;
-        int lo = 0, hi = nlist;
-        while (lo < hi) {
-            int mid = (lo + hi) >> 1;
-            if ((uint32_t)csorted[mid] < rb) lo = mid + 1;
-            else hi = mid;
-        }
-        cs_lo = (uint32_t)lo;
-        hi = nlist;
-        while (lo < hi) {
-            int mid = (lo + hi) >> 1;
-            if ((uint32_t)csorted[mid] < re) lo = mid + 1;
-            else hi = mid;
-        }
-        cs_hi = (uint32_t)lo;
-    }
-    for (int r = 0; r < 27; r++) {
-        int tr = __shfl_sync(FULLM, rt, r);
-        if (!tr) continue;
-        uint32_t b = __shfl_sync(FULLM, rb, r), e = __shfl_sync(FULLM, re, r);
-        if (csorted) {
-            b = __shfl_sync(FULLM, cs_lo, r);
-            e = __shfl_sync(FULLM, cs_hi, r);
-        }
-        for (uint32_t c = b; c < e; c += 32) {
-            uint32_t jj = c + lane;
-            uint32_t j = (csorted && jj < e) ? (uint32_t)csorted[jj] : jj;
-            bool take = false;
-            u64 d2 = 0;
-            if (jj < e && (int)j != x && alive[j] && inP[j]) {
-                int4 v = g.pos[j];
-                long long ddx = v.x - xp.x, ddy = v.y - xp.y, ddz = v.z - xp.z;
-                d2 = (u64)(ddx * ddx + ddy * ddy + ddz * ddz);
-                take = d2 < lx && key_gt(px, xp.w, prim[j], v.w);
+    {
+        const uint32_t w0 = rb >> 5, words = rt ? ((re - 1) >> 5) - w0 + 1 : 0;
+        const uint32_t inc = warp_inclusive(words, lane);
+        const uint32_t total = __shfl_sync(FULLM, inc, 31);
+        for (uint32_t base = 0; base < total; base += 32) {
+            const uint32_t t = base + lane;
+            const int r = range_of(inc, t < total ? t : total - 1);
+            const uint32_t b = __shfl_sync(FULLM, rb, r), e = __shfl_sync(FULLM, re, r);
+            const uint32_t wb = __shfl_sync(FULLM, w0, r) +
+                                (t - (__shfl_sync(FULLM, inc, r) - __shfl_sync(FULLM, words, r)));
+            uint32_t bits = 0;
+            if (t < total) {
+                bits = inPb[wb];
+                if (wb == (b >> 5)) bits &= 0xffffffffu << (b & 31);
+                if (wb == (e - 1) >> 5) bits &= 0xffffffffu >> (31 - ((e - 1) & 31));
             }
-            unsigned bal = __ballot_sync(FULLM, take);
-            int slot = nc + __popc(bal & ((1u << lane) - 1u));
-            if (take) {
-                if (slot < DG_CAP) {
-                    c_j[w][slot] = (int)j;
-                    c_d[w][slot] = d2;
-                } else {
-                    rej[j] = 1;
+            const uint32_t end = warp_inclusive((uint32_t)__popc(bits), lane);
+            const uint32_t tot = __shfl_sync(FULLM, end, 31);
+            uint32_t at = end - (uint32_t)__popc(bits);  // place of this lane's next bit
+            for (uint32_t win = 0; win < tot; win += 192) {
+                __syncwarp();
+                while (bits && at < win + 192) {
+                    u.raw[at - win] = (int)(wb * 32 + (uint32_t)__ffs(bits) - 1);
+                    bits &= bits - 1;
+                    at++;
+                }
+                __syncwarp();
+                const uint32_t m = min(192u, tot - win);
+                for (uint32_t c = 0; c < m; c += 32) {
+                    bool take = false;
+                    u64 d2 = 0;
+                    int j = 0;
+                    if (c + lane < m) {
+                        j = u.raw[c + lane];
+                        const int4 v = g.pos[j];
+                        d2 = sqd(v, xp);
+                        take = j != x && d2 < lx && key_gt(px, xp.w, prim[j], v.w);
+                    }
+                    const unsigned bal = __ballot_sync(FULLM, take);
+                    const int slot = nc + __popc(bal & ((1u << lane) - 1u));
+                    if (take) {
+                        if (slot < DG_CAP) {
+                            c_j[slot] = j;
+                            c_d[slot] = d2;
+                        } else {
+                            rej[j] = 1;
+                        }
+                    }
+                    nc += __popc(bal);
                 }
             }
-            nc += __popc(bal);
         }
     }
     if (diag && lane == 0) {
@@ -322,88 +303,87 @@ __device__ void danger_one(const GridView& g, int x, const u64* __restrict__ pri
     }
     nc = min(nc, DG_CAP);
     __syncwarp();
-    // x's stored neighbours are live points near x: the cheapest shields
-    int sn_j[PD_DG_SMAX];
-    u64 sn_d[PD_DG_SMAX], sn_k[PD_DG_SMAX];
-    int sn_i[PD_DG_SMAX];
-#pragma unroll
-    for (int i = 0; i < PD_DG_SMAX; i++) {
-        sn_j[i] = -1;
-        sn_d[i] = ~0ull;
-        sn_k[i] = 0;
-        sn_i[i] = 0;
-        if (nbr && i < S && nc > 0) {
-            int y = nbr[(int64_t)x * S + i];
-            if (y >= 0) {
-                int4 v = g.pos[y];
-                long long ddx = v.x - xp.x, ddy = v.y - xp.y, ddz = v.z - xp.z;
-                sn_j[i] = y;
-                sn_d[i] = (u64)(ddx * ddx + ddy * ddy + ddz * ddz);
-                sn_k[i] = prim[y];
-                sn_i[i] = v.w;
-            }
+    if (nc == 0) return;
+    // x's stored neighbours are live points near x: the cheapest shields, one
+    // per lane
+    int sn_j = -1, sn_i = 0;
+    u64 sn_d = ~0ull, sn_k = 0;
+    if (nbr && lane < S) {
+        sn_j = nbr[(int64_t)x * S + lane];
+        if (sn_j >= 0) {
+            const int4 v = g.pos[sn_j];
+            sn_d = sqd(v, xp);
+            sn_k = prim[sn_j];
+            sn_i = v.w;
         }
     }
     // 2. counting, 32 candidates at a time
     for (int a0 = 0; a0 < nc; a0 += 32) {
         int a = a0 + lane;
         bool done = a >= nc;
-        int p = done ? -1 : c_j[w][a];
-        u64 dp = done ? 0 : c_d[w][a];
+        int p = done ? -1 : c_j[a];
+        u64 dp = done ? 0 : c_d[a];
         u64 pp = done ? 0 : prim[p];
         int ip = done ? 0 : g.pos[p].w;
         int cnt = 0;
-        if (!done) {
-#pragma unroll
-            for (int i = 0; i < PD_DG_SMAX; i++)
-                if (sn_j[i] >= 0 && sn_j[i] != p && sn_d[i] <= dp &&
-                    key_gt(pp, ip, sn_k[i], sn_i[i]))
-                    cnt++;
-            if (cnt >= k) done = true;
-            cnt = 0;  // the stream below recounts every point (stored ones included)
+        for (int i = 0; i < PD_DG_SMAX; i++) {
+            const int yj = __shfl_sync(FULLM, sn_j, i), yi = __shfl_sync(FULLM, sn_i, i);
+            const u64 yd = __shfl_sync(FULLM, sn_d, i), yk = __shfl_sync(FULLM, sn_k, i);
+            if (yj >= 0 && yj != p && yd <= dp && key_gt(pp, ip, yk, yi)) cnt++;
         }
+        if (cnt >= k) done = true;
+        cnt = 0;  // the stream below recounts every point (stored ones included)
+        if (__all_sync(FULLM, done)) continue;
         u64 dmax = done ? 0 : dp;  // farthest candidate of this batch
         for (int o2 = 16; o2; o2 >>= 1) {
             u64 other = __shfl_xor_sync(FULLM, dmax, o2);
             dmax = other > dmax ? other : dmax;
         }
-        for (int r = 0; r < 27; r++) {
-            int tr = __shfl_sync(FULLM, rt, r);
-            if (!tr) continue;
-            if (__all_sync(FULLM, done)) break;
-            if (__shfl_sync(FULLM, rbox, r) > dmax) continue;
-            uint32_t b = __shfl_sync(FULLM, rb, r), e = __shfl_sync(FULLM, re, r);
-            for (uint32_t c = b; c < e; c += 32) {
-                // each lane loads one point and its distance to x; only points
-                // within the batch's farthest open candidate can shield, and
-                // they are compacted into the staging buffer
-                uint32_t j = c + lane;
-                bool near = false;
-                u64 d2 = 0, ky = 0;
-                int oy = 0;
-                if (j < e) {  // independent loads, issued together
-                    uint8_t al = alive[j];
-                    int4 v = g.pos[j];
-                    ky = prim[j];
-                    long long ddx = v.x - xp.x, ddy = v.y - xp.y, ddz = v.z - xp.z;
-                    d2 = (u64)(ddx * ddx + ddy * ddy + ddz * ddz);
-                    near = al && (int)j != x && d2 <= dmax;
-                    oy = v.w;
+        // Streams the lanes' ranges [b, b + len): true once every count reached k.
+        auto stream = [&](uint32_t b, uint32_t len) -> bool {
+            const uint32_t inc = warp_inclusive(len, lane);
+            const uint32_t total = __shfl_sync(FULLM, inc, 31);
+            uint32_t jn = 0;  // a step's point: its fields loaded one step ahead
+            int4 vn = make_int4(0, 0, 0, 0);
+            u64 kn = 0;
+            uint8_t an = 0;
+            auto load = [&](uint32_t t) {
+                const int r = range_of(inc, t < total ? t : total - 1);
+                jn = __shfl_sync(FULLM, b, r) +
+                     (t - (__shfl_sync(FULLM, inc, r) - __shfl_sync(FULLM, len, r)));
+                an = 0;
+                if (t < total) {
+                    an = alive[jn];
+                    vn = g.pos[jn];
+                    kn = prim[jn];
                 }
-                unsigned nb = __ballot_sync(FULLM, near);
+            };
+            if (total) load(lane);
+            for (uint32_t base = 0; base < total; base += 32) {
+                const uint32_t j = jn;
+                const int4 v = vn;
+                const u64 ky = kn;
+                const uint8_t al = an;
+                load(base + 32 + lane);
+                // only points within the farthest open candidate can shield:
+                // they are compacted into the staging buffer
+                const u64 d2 = sqd(v, xp);
+                const bool near = al && (int)j != x && d2 <= dmax;
+                const unsigned nb = __ballot_sync(FULLM, near);
+                if (!nb) continue;
                 if (near) {
-                    int slot = __popc(nb & ((1u << lane) - 1u));
-                    st_d[w][slot] = d2;
-                    st_k[w][slot] = ky;
-                    st_o[w][slot] = oy;
-                    st_j[w][slot] = (int)j;
+                    const int slot = __popc(nb & ((1u << lane) - 1u));
+                    u.st.d[slot] = d2;
+                    u.st.k[slot] = ky;
+                    u.st.o[slot] = v.w;
+                    u.st.j[slot] = (int)j;
                 }
                 __syncwarp();
-                int mm = __popc(nb);
+                const int mm = __popc(nb);
                 if (!done) {
                     for (int tt = 0; tt < mm; tt++) {
-                        if (st_j[w][tt] == p) continue;
-                        if (st_d[w][tt] <= dp && key_gt(pp, ip, st_k[w][tt], st_o[w][tt])) {
+                        if (u.st.j[tt] == p) continue;
+                        if (u.st.d[tt] <= dp && key_gt(pp, ip, u.st.k[tt], u.st.o[tt])) {
                             if (++cnt >= k) {
                                 done = true;
                                 break;
@@ -412,8 +392,31 @@ __device__ void danger_one(const GridView& g, int x, const u64* __restrict__ pri
                     }
                 }
                 __syncwarp();
-                if (__all_sync(FULLM, done)) break;
+                if (__all_sync(FULLM, done)) return true;
             }
+            return false;
+        };
+        // small nodes at once, then the large ones by their children, nearest first
+        WarpNode n = cell;
+        const bool in = rt && n.box <= dmax;
+        bool held = in && n.count() > DG_SCAN && n.lv > 0;
+        bool fin = stream(n.b, in && !held ? n.count() : 0);
+        while (!fin) {
+            u64 next = held ? (n.box << 5) | lane : ~0ull;
+            if (__all_sync(FULLM, next == ~0ull)) break;
+            for (int o2 = 16; o2; o2 >>= 1) {
+                const u64 v = __shfl_xor_sync(FULLM, next, o2);
+                next = v < next ? v : next;
+            }
+            const int from = (int)(next & 31);
+            const WarpNode c = warp_children(g, n, from, ux, uy, uz, lane);
+            if (lane == from) held = false;
+            bool now = c.count() > 0 && c.box <= dmax;
+            bool keep = now && c.count() > DG_SCAN && c.lv > 0;
+            const bool was = keep;
+            warp_keep(n, held, c, keep, lane);
+            if (was && !keep) now = false;
+            fin = stream(c.b, now ? c.count() : 0);
         }
         if (!done) {
             int ps = atomicAdd(npairs, 1);
@@ -426,16 +429,15 @@ __device__ void danger_one(const GridView& g, int x, const u64* __restrict__ pri
 __global__ void __launch_bounds__(DG_WARPS * 32, DG_BLOCKS_PER_SM)
     danger_kernel(GridView g, const int* __restrict__ src, const int* __restrict__ nsrc,
                   const u64* __restrict__ prim, const uint8_t* __restrict__ alive,
-                  const uint8_t* __restrict__ inP, uint8_t* rej, const u64* __restrict__ lam,
+                  const uint32_t* __restrict__ inPb, uint8_t* rej, const u64* __restrict__ lam,
                   const int* __restrict__ nbr, int S, int k, int2* pairs, int* npairs,
-                  int pair_cap, int* overflow, unsigned long long* diag,
-                  const int* __restrict__ csorted, const int* __restrict__ ncs) {
+                  int pair_cap, int* overflow, unsigned long long* diag) {
     __shared__ DangerSmem sm;
     int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int ns = *nsrc;
     for (int t = blockIdx.x * DG_WARPS + w; t < ns; t += gridDim.x * DG_WARPS)
-        danger_one(g, src[t], prim, alive, inP, rej, lam, nbr, S, k, pairs, npairs, pair_cap,
-                   overflow, diag, csorted, ncs, sm, w, lane);
+        danger_one(g, src[t], prim, alive, inPb, rej, lam, nbr, S, k, pairs, npairs, pair_cap,
+                   overflow, diag, sm, w, lane);
 }
 
 // Fallback: accept every live point with key >= tau (tau = the top key).
@@ -582,13 +584,12 @@ cudaError_t launch_k1_fix(const int* cand, const int* ncand, int max_cand, const
     return cudaGetLastError();
 }
 cudaError_t round_launch_danger(const GridView& g, const int* src, const u64* prim,
-                                const uint8_t* alive, const uint8_t* inP, uint8_t* rej,
+                                const uint8_t* alive, const uint32_t* inPb, uint8_t* rej,
                                 const u64* lam, const int* nbr, int S, int k, int2* pairs,
-                                int pair_cap, const int* csorted, RoundDev* rd, cudaStream_t st) {
-    danger_kernel<<<device_sms() * DG_BLOCKS_PER_SM, DG_WARPS * 32, 0, st>>>(g, src, &rd->nsrc, prim, alive, inP, rej,
-                                                     lam, S <= PD_DG_SMAX ? nbr : nullptr, S, k,
-                                                     pairs, &rd->npairs, pair_cap, &rd->overflow,
-                                                     &rd->cap_over, csorted, &rd->ncs); note_launch();
+                                int pair_cap, RoundDev* rd, cudaStream_t st) {
+    danger_kernel<<<device_sms() * DG_BLOCKS_PER_SM, DG_WARPS * 32, 0, st>>>(
+        g, src, &rd->nsrc, prim, alive, inPb, rej, lam, S <= PD_DG_SMAX ? nbr : nullptr, S, k,
+        pairs, &rd->npairs, pair_cap, &rd->overflow, &rd->cap_over); note_launch();
     return cudaGetLastError();
 }
 cudaError_t launch_accept_above(const u64* prim, const int4* pos, const uint8_t* alive, int64_t n,

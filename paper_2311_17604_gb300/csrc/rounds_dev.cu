@@ -42,6 +42,7 @@ __global__ void round_setup_kernel(RoundDev* rd) {
     rd->len[0] = rd->len[1] = 0;
     rd->ncand = rd->nslow = rd->nsrc = rd->npairs = rd->overflow = 0;
     rd->ndep = 0;
+    rd->nreq = rd->nfq = rd->nlq = 0;
     rd->removed = 0;
     rd->cap_over = 0;
     rd->fix_unconverged = 0;
@@ -68,6 +69,9 @@ __global__ void round_finish_kernel(RoundDev* rd) {
     if (threadIdx.x != 0) return;
     rd->live -= (long long)rd->removed;
     rd->tot_sources += (unsigned long long)rd->nsrc;
+    rd->tot_filtered += (unsigned long long)rd->nfq;
+    rd->tot_lambda += (unsigned long long)rd->nlq;
+    rd->tot_requery += (unsigned long long)rd->nreq;
     // a held round (settled on the host) updates its band there, from the
     // points it finally removes: the band must not depend on whether the
     // device fixpoint happened to converge within its sweeps
@@ -351,15 +355,6 @@ __global__ void k1d_fix_kernel(const int* __restrict__ cand, const int4* __restr
     }
 }
 
-__global__ void kkd_accept_kernel(const uint8_t* __restrict__ fq_flag, const u64* __restrict__ prim,
-                                  const u64* __restrict__ fprim, int64_t n, RoundDev* rd,
-                                  uint8_t* inP, int* cand) {
-    int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    bool acc = s < n && fq_flag[s] && fprim[s] == prim[s];
-    if (acc) inP[s] = 1;
-    list_append(acc, (int)s, &rd->ncand, cand);
-}
-
 __global__ void pairs_fix_kernel(const int2* __restrict__ pairs, int pair_cap, const uint8_t* inP,
                                  uint8_t* rej, int iter, RoundDev* rd) {
     if (iter > 0 && !rd->changed[iter - 1]) return;
@@ -406,19 +401,16 @@ __global__ void removed_kernel(const int* __restrict__ cand, uint8_t* inP, uint8
 }
 
 __global__ void dirtyd_kernel(const uint8_t* __restrict__ alive, const int* __restrict__ nbr,
-                              int64_t n, int S, int kchk, uint8_t* dirty, RoundDev* rd) {
+                              int64_t n, int S, int kchk, int* list, RoundDev* rd) {
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     bool d = false;
-    if (s < n) {
-        if (alive[s]) {
-            for (int i = 0; i < kchk; i++) {
-                int x = nbr[s * S + i];
-                if (x >= 0 && !alive[x]) d = true;
-            }
+    if (s < n && alive[s]) {
+        for (int i = 0; i < kchk; i++) {
+            int x = nbr[s * S + i];
+            if (x >= 0 && !alive[x]) d = true;
         }
-        dirty[s] = d ? 1 : 0;
     }
-    block_add(&rd->tot_requery, d ? 1ull : 0ull);
+    list_append(d, (int)s, &rd->nreq, list);
 }
 
 // ------------------------------------------------------------------ k = 1 buffer
@@ -434,12 +426,12 @@ __global__ void dirtyd_kernel(const uint8_t* __restrict__ alive, const int* __re
 // 40 registers, 6 blocks of 256 per SM: the update waits on dependent loads,
 // and more threads in flight measured faster (rules of the 100M-point scan
 // 52.9 -> 51.5 ms)
-__global__ void __launch_bounds__(256, 6) k1d_update_kernel(BufView b, const uint8_t* __restrict__ alive, int64_t n, int S,
-                                  uint8_t* dirty, RoundDev* rd) {
+__global__ void __launch_bounds__(256, 6)
+    k1d_update_kernel(BufView b, const uint8_t* __restrict__ alive, int64_t n, int S, int* list,
+                      RoundDev* rd) {
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    bool upd = false, req = false;
+    bool req = false;
     if (s < n) {
-        uint8_t dv = 0;
         // only a removed shell member changes the key or the shell; removed
         // entries past the shell stay stored (stale) until the shell changes
         // the point's flag, shell size and first entry are loaded together
@@ -488,16 +480,13 @@ __global__ void __launch_bounds__(256, 6) k1d_update_kernel(BufView b, const uin
                     for (int i = 0; i < K1_SMAX; i++)
                         if (i < S) b.nbr[s * S + i] = ids[i];
                     if (b.nbr0) b.nbr0[s] = ids[0];
-                    upd = true;
                 } else {
-                    dv = 1;
                     req = true;
                 }
             }
         }
-        dirty[s] = dv;
     }
-    block_add2(&rd->tot_updated, upd ? 1ull : 0ull, &rd->tot_requery, req ? 1ull : 0ull);
+    list_append(req, (int)s, &rd->nreq, list);
 }
 
 // ------------------------------------------------------------------ k+b buffer
@@ -512,12 +501,12 @@ __global__ void __launch_bounds__(256, 6) k1d_update_kernel(BufView b, const uin
 // Held to 48 registers for 5 blocks per SM: the loop over the stored entries
 // waits on dependent loads, and the recomputation that spills runs only for
 // points that lost a neighbour.
-__global__ void __launch_bounds__(256, 5) kkd_update_kernel(BufView b, const uint8_t* __restrict__ alive, int64_t n, int S,
-                                  int k, uint8_t* dirty, RoundDev* rd) {
+__global__ void __launch_bounds__(256, 5)
+    kkd_update_kernel(BufView b, const uint8_t* __restrict__ alive, int64_t n, int S, int k,
+                      int* list, RoundDev* rd) {
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    bool upd = false, req = false;
+    bool req = false;
     if (s < n) {
-        uint8_t dv = 0;
         if (alive[s]) {
             int ids[UPD_SMAX];
             int r = 0;
@@ -559,16 +548,13 @@ __global__ void __launch_bounds__(256, 5) kkd_update_kernel(BufView b, const uin
 #pragma unroll
                     for (int i = 0; i < UPD_SMAX; i++)
                         if (i < S) b.nbr[s * S + i] = ids[i];
-                    upd = true;
                 } else {
-                    dv = 1;
                     req = true;
                 }
             }
         }
-        dirty[s] = dv;
     }
-    block_add2(&rd->tot_updated, upd ? 1ull : 0ull, &rd->tot_requery, req ? 1ull : 0ull);
+    list_append(req, (int)s, &rd->nreq, list);
 }
 
 // Candidate test (k >= 2) using the stored buffer where it suffices:
@@ -577,22 +563,29 @@ __global__ void __launch_bounds__(256, 5) kkd_update_kernel(BufView b, const uin
 //       least as far as every stored one); otherwise a filtered search.
 //   lam (danger sources): the k-th stored squared distance of key below tau,
 //       when k such entries are stored; otherwise a search.
+// Alongside: the bitmap of the candidates and the least live key of every
+// 32-position chunk (a warp holds one chunk).
 __global__ void kkd_cand2_kernel(BufView b, const uint8_t* __restrict__ alive, int64_t n, int S,
-                                 int k, RoundDev* rd, uint8_t* inP, int* cand, uint8_t* fq_flag,
-                                 uint8_t* lq_flag, u64* lam, int* src) {
+                                 int k, RoundDev* rd, uint8_t* inP, uint32_t* inPb, int* cand,
+                                 int* fq_list, int* lq_list, u64* lam, int* src, u64* cmin) {
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    u64 low = ~0ull;
     bool fq = false, lq = false, isc = false, iss = false;
     if (s < n) {
         if (alive[s]) {
             u64 ps = b.prim[s];
-            int4 qs = b.pos[s];
-            int is = qs.w;
-            u64 tp = rd->tau_prim;
-            int ti = rd->tau_idx;
+            low = ps;
             // packed batch: tp is the least threshold over the scans; a point
             // above it takes its own scan's threshold
-            if (rd->seg && ps >= tp) round_tau(rd, qs, tp, ti);
-            if (!key_gt(tp, ti, ps, is)) {
+            u64 tp = rd->tau_prim;
+            int ti = rd->tau_idx;
+            int4 qs = make_int4(0, 0, 0, 0);
+            if (ps >= tp) {  // below the threshold on the primary: no index needed
+                qs = b.pos[s];
+                if (rd->seg) round_tau(rd, qs, tp, ti);
+            }
+            const int is = qs.w;
+            if (ps >= tp && !key_gt(tp, ti, ps, is)) {
                 uint8_t fl = b.flg[s];
                 bool lower = !(fl & 1);
                 bool band_nbr = (fl & 1) != 0;
@@ -647,12 +640,24 @@ __global__ void kkd_cand2_kernel(BufView b, const uint8_t* __restrict__ alive, i
                 }
             }
         }
-        fq_flag[s] = fq ? 1 : 0;
-        lq_flag[s] = lq ? 1 : 0;
     }
-    list_append(isc, (int)s, &rd->ncand, cand);
-    list_append(iss, (int)s, &rd->nsrc, src);
-    block_add2(&rd->tot_filtered, fq ? 1ull : 0ull, &rd->tot_lambda, lq ? 1ull : 0ull);
+    const unsigned cb = __ballot_sync(FULLM, isc);
+    for (int o = 16; o; o >>= 1) {
+        const u64 v = __shfl_xor_sync(FULLM, low, o);
+        low = v < low ? v : low;
+    }
+    if ((threadIdx.x & 31) == 0 && s < n) {
+        inPb[s >> 5] = cb;
+        cmin[s >> 5] = low;
+    }
+    const bool want[4] = {isc, iss, fq, lq};
+    int* const count[4] = {&rd->ncand, &rd->nsrc, &rd->nfq, &rd->nlq};
+    int slot[4];
+    block_append_n(want, count, slot);
+    if (isc) cand[slot[0]] = (int)s;
+    if (iss) src[slot[1]] = (int)s;
+    if (fq) fq_list[slot[2]] = (int)s;
+    if (lq) lq_list[slot[3]] = (int)s;
 }
 
 // ------------------------------------------------------------------ launchers
@@ -698,13 +703,6 @@ cudaError_t round_launch_k1(const GridView& g, const u64* prim, const uint8_t* a
     return cudaGetLastError();
 }
 
-cudaError_t round_launch_kk_accept(const uint8_t* fq_flag, const u64* prim, const u64* fprim,
-                                   int64_t n, RoundDev* rd, uint8_t* inP, int* cand,
-                                   cudaStream_t st) {
-    kkd_accept_kernel<<<GRID1(n), 0, st>>>(fq_flag, prim, fprim, n, rd, inP, cand); note_launch();
-    return cudaGetLastError();
-}
-
 cudaError_t round_launch_pairs_fix(const int2* pairs, int pair_cap, const uint8_t* inP,
                                    uint8_t* rej, RoundDev* rd, cudaStream_t st) {
     for (int it = 0; it < PD_FIX_ITERS_KK; it++) {
@@ -720,8 +718,8 @@ cudaError_t round_launch_remove(const int* cand, uint8_t* inP, uint8_t* rej, uin
 }
 
 cudaError_t round_launch_dirty(const uint8_t* alive, const int* nbr, int64_t n, int S, int kchk,
-                               uint8_t* dirty, RoundDev* rd, cudaStream_t st) {
-    dirtyd_kernel<<<GRID1(n), 0, st>>>(alive, nbr, n, S, kchk, dirty, rd); note_launch();
+                               int* list, RoundDev* rd, cudaStream_t st) {
+    dirtyd_kernel<<<GRID1(n), 0, st>>>(alive, nbr, n, S, kchk, list, rd); note_launch();
     return cudaGetLastError();
 }
 
@@ -729,21 +727,21 @@ cudaError_t round_launch_dirty(const uint8_t* alive, const int* nbr, int64_t n, 
 
 namespace pd {
 cudaError_t round_launch_k1_update(const BufView& b, const uint8_t* alive, int64_t n, int S,
-                                   uint8_t* dirty, RoundDev* rd, cudaStream_t st) {
+                                   int* list, RoundDev* rd, cudaStream_t st) {
     if (S > K1_SMAX) return cudaErrorInvalidValue;
-    k1d_update_kernel<<<GRID1(n), 0, st>>>(b, alive, n, S, dirty, rd); note_launch();
+    k1d_update_kernel<<<GRID1(n), 0, st>>>(b, alive, n, S, list, rd); note_launch();
     return cudaGetLastError();
 }
 cudaError_t round_launch_kk_update(const BufView& b, const uint8_t* alive, int64_t n, int S, int k,
-                                   uint8_t* dirty, RoundDev* rd, cudaStream_t st) {
-    kkd_update_kernel<<<GRID1(n), 0, st>>>(b, alive, n, S, k, dirty, rd); note_launch();
+                                   int* list, RoundDev* rd, cudaStream_t st) {
+    kkd_update_kernel<<<GRID1(n), 0, st>>>(b, alive, n, S, k, list, rd); note_launch();
     return cudaGetLastError();
 }
 cudaError_t round_launch_kk_cand2(const BufView& b, const uint8_t* alive, int64_t n, int S, int k,
-                                  RoundDev* rd, uint8_t* inP, int* cand, uint8_t* fq_flag,
-                                  uint8_t* lq_flag, u64* lam, int* src, cudaStream_t st) {
-    kkd_cand2_kernel<<<GRID1(n), 0, st>>>(b, alive, n, S, k, rd, inP, cand, fq_flag, lq_flag, lam,
-                                          src); note_launch();
+                                  RoundDev* rd, uint8_t* inP, uint32_t* inPb, int* cand, int* fq,
+                                  int* lq, u64* lam, int* src, u64* cmin, cudaStream_t st) {
+    kkd_cand2_kernel<<<GRID1(n), 0, st>>>(b, alive, n, S, k, rd, inP, inPb, cand, fq, lq, lam,
+                                          src, cmin); note_launch();
     return cudaGetLastError();
 }
 }  // namespace pd
