@@ -850,9 +850,10 @@ BufView bufview(pd_grid* g, const pd_cost_params* cp) {
 
 // Full searches of list[0 .. rd->nreq): the points whose stored neighbours no
 // longer settle their cost.
-int knn_requery(pd_grid* g, const pd_cost_params* cp, const int* list, const RoundDev* rd) {
+int knn_requery(pd_grid* g, const pd_cost_params* cp, const int* list, RoundDev* rd) {
     KnnArgs a = base_args(g, cp);
     if (g->density_k1 && g->k1_exact_rq > 0) a.r_exact = g->k1_exact_rq;
+    a.finish = rd;
     a.qlist = list;
     a.qcount = &rd->nreq;
     CK(launch_knn_queries(view_of(g), a, g->ng, g->st));
@@ -878,10 +879,11 @@ int settle_round(pd_grid* g, RoundDev* rd, const RoundDev& h, uint8_t* inP, uint
             CK(cudaMemcpyAsync(&rd->seg_rank_one, &one, sizeof(int), cudaMemcpyHostToDevice,
                                g->st));
             CK(seg_launch_select(g->prim, g->pos, g->alive, g->ng, *sel, seg_hist, rd, g->seg,
-                                 g->seg_chunk0, g->seg_items, g->nseg, g->st));
+                                 g->seg_items, g->nseg, g->st));
             CK(cudaMemcpyAsync(&rd->seg_rank_one, &zero, sizeof(int), cudaMemcpyHostToDevice,
                                g->st));
             CK(seg_launch_accept(g->prim, g->pos, g->alive, g->ng, rd, inP, cand, d + 4, g->st));
+            CK(cudaMemsetAsync(&rd->tau_prim, 0xff, sizeof(u64), g->st));  // as a round leaves it
             CK(launch_remove(cand, d + 4, g->nseg, inP, rej, g->alive, g->d_u64, g->st));
         } else {
             Sel top;
@@ -1128,10 +1130,8 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
         ALLOC(g->cmin, u64, (cap + 31) / 32 + 1);
     }
     SelBuffers sb;
-    RALLOC(sb.p[0], u64, cap);
-    RALLOC(sb.p[1], u64, cap);
-    RALLOC(sb.i[0], int, cap);
-    RALLOC(sb.i[1], int, cap);
+    RALLOC(sb.p, u64, cap);
+    RALLOC(sb.i, int, cap);
     RALLOC(sb.hist, uint32_t, 4096);
     CK(cudaMemsetAsync(sb.hist, 0, 4096 * sizeof(uint32_t), g->st));
     RoundDev* rd;
@@ -1148,6 +1148,7 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
         h.seg_chunk0 = g->seg_chunk0;
         h.nseg = g->nseg;
         h.seg_shift = g->seg_shift;
+        h.tau_prim = ~0ull;  // lowered by the scans' thresholds
     }
     h.live = live;
     h.m = m;
@@ -1160,12 +1161,14 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
         h.fix_iters = std::max(1, std::min(PD_FIX_ITERS, atoi(getenv("PD_FIX_SWEEPS"))));
     CK(cudaMemcpyAsync(rd, &h, sizeof(h), cudaMemcpyHostToDevice, g->st));
     int64_t built = live;
+    bool long_list = live > ((int64_t)32 << 20);  // then: whether the last round's list was long
     // small clouds are bound by launches: from the third round on, a round's
     // launches are captured into a CUDA graph and replayed (PD_ROUND_GRAPH:
-    // 1 always, 0 never; default for grids up to 8M points and packed batches)
-    bool round_graph = g->n <= ((int64_t)8 << 20) || g->nseg > 0;
+    // 1 always, 0 never; default for grids up to 32M points and packed batches)
+    bool round_graph = g->n <= ((int64_t)32 << 20) || g->nseg > 0;
     if (getenv("PD_ROUND_GRAPH")) round_graph = atoi(getenv("PD_ROUND_GRAPH")) != 0;
     void* graph_pos = nullptr;
+    bool graph_long = false;
     long long graph_kernels = 0;
     if (g->trace) {
         cudaEventCreate(&rs.tq0);
@@ -1174,14 +1177,14 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
     cudaEvent_t tq0 = rs.tq0, tq1 = rs.tq1;
     auto issue_round = [&]() -> int {
             GridView v = view_of(g);
-            CK(round_launch_setup(rd, g->st));
             {
                 Span t(T, &g->stats.ms_select);
                 if (g->nseg)
                     CK(seg_launch_select(g->prim, g->pos, g->alive, g->ng, sb, seg_hist, rd,
-                                         g->seg, g->seg_chunk0, g->seg_items, g->nseg, g->st));
+                                         g->seg, g->seg_items, g->nseg, g->st));
                 else
-                    CK(round_launch_select(g->prim, g->pos, g->alive, g->ng, sb, rd, g->st));
+                    CK(round_launch_select(g->prim, g->pos, g->alive, g->ng, sb, long_list, rd,
+                                           g->st));
             }
             if (g->density_k1) {
                 CK(round_launch_k1(v, g->prim, g->alive, g->nbr, g->nbr0, g->flg, g->rk2, g->ng, S,
@@ -1209,11 +1212,11 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
                 {
                     Span t(T, &g->stats.ms_danger);
                     CK(round_launch_danger(v, src, g->prim, g->alive, inPb, rej, lam, g->nbr, S, k,
-                                           pairs, pair_cap, rd, g->st));
+                                           pairs, pair_cap, g->ng, rd, g->st));
                 }
-                CK(round_launch_pairs_fix(pairs, pair_cap, inP, rej, rd, g->st));
+                CK(round_launch_pairs_fix(pairs, pair_cap, inP, rej, g->ng, rd, g->st));
             }
-            CK(round_launch_remove(cand, inP, rej, g->alive, rd, g->st));
+            CK(round_launch_remove(cand, inP, rej, g->alive, g->ng, rd, g->st));
             if (g->density_k1) {
                 // absorb removals in the stored 8 nearest; search where the new
                 // nearest shell may be incomplete
@@ -1231,7 +1234,6 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
                 if (rc) return rc;
             }
             if (g->trace) cudaEventRecord(tq1, g->st);
-            CK(round_launch_finish(rd, g->st));
             return PD_OK;
     };
     while (live > m) {
@@ -1248,7 +1250,7 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
         }
         int rr = PD_OK;
         const bool replay = round_graph && g->stats.rounds >= 3 && !g->trace;
-        if (replay && (!rs.gx || graph_pos != (void*)g->pos)) {
+        if (replay && (!rs.gx || graph_pos != (void*)g->pos || graph_long != long_list)) {
             // capture this round's launches once per grid layout (compaction
             // replaces the arrays) on a private stream, then replay the graph
             if (rs.gx) {
@@ -1272,6 +1274,7 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
             if (!eb && !rc_cap && !ee && graph &&
                 cudaGraphInstantiate(&rs.gx, graph, 0) == cudaSuccess) {
                 graph_pos = (void*)g->pos;
+                graph_long = long_list;
                 // the captured launches ran nothing; each replay runs its kernel nodes
                 graph_kernels = count_kernel_nodes(graph);
                 __atomic_fetch_sub(&g_launch_count, graph_kernels, __ATOMIC_RELAXED);
@@ -1296,6 +1299,7 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
         }
         CK(cudaMemcpyAsync(&h, rd, sizeof(h), cudaMemcpyDeviceToHost, g->st));
         CK(cudaStreamSynchronize(g->st));
+        long_list = !g->nseg && h.len > PD_SEL_LONG;
         if (h.overflow || h.fix_unconverged) {
             // settle on the host: finish the fixpoint, or (danger overflow / too
             // few low points) take only the global maximum, always removable
@@ -1318,7 +1322,7 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
             h.removed = (unsigned long long)removed;
             if (!g->density_k1) {
                 // an overflowing round always narrows the band, as before
-                h.band = host_next_band(h.band, h.band_max, h.band_mode,
+                h.band = next_band(h.band, h.band_max, h.band_mode,
                                         h.cap_over + (h.overflow ? 1 : 0), h.ncand, h.removed);
                 CK(cudaMemcpyAsync(&rd->band, &h.band, sizeof(h.band), cudaMemcpyHostToDevice,
                                    g->st));
@@ -1422,10 +1426,8 @@ static int wup_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* ke
     RALLOC(mark_p, u64, cap);
     RALLOC(mark_i, int, cap);
     SelBuffers sb;
-    RALLOC(sb.p[0], u64, cap);
-    RALLOC(sb.p[1], u64, cap);
-    RALLOC(sb.i[0], int, cap);
-    RALLOC(sb.i[1], int, cap);
+    RALLOC(sb.p, u64, cap);
+    RALLOC(sb.i, int, cap);
     RALLOC(sb.hist, uint32_t, 4096);
     CK(cudaMemsetAsync(sb.hist, 0, 4096 * sizeof(uint32_t), g->st));
     RoundDev* rd;
@@ -1460,11 +1462,12 @@ static int wup_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* ke
         memset(&h, 0, sizeof(h));
         h.live = live;
         h.m = m;
+        h.density_k1 = 1;  // rank: all that must go
         CK(cudaMemcpyAsync(rd, &h, sizeof(h), cudaMemcpyHostToDevice, g->st));
-        CK(wup_launch_setup(rd, g->st));
         {
             Span t(T, &g->stats.ms_select);
-            CK(round_launch_select(g->prim, g->pos, g->alive, g->ng, sb, rd, g->st));
+            CK(round_launch_select(g->prim, g->pos, g->alive, g->ng, sb,
+                                   g->ng > ((int64_t)4 << 20), rd, g->st));
             CK(wup_launch_exact_tau(g->prim, g->pos, g->alive, g->ng, rd, tmin, imin, g->st));
         }
         // 3. removal rounds above w_up

@@ -1047,6 +1047,7 @@ template <bool FILTERED, bool W>
 __global__ void __launch_bounds__(PD_WARPS * 32, W ? 8 : 10) knn_query_kernel(GridView g, KnnArgs a) {
     __shared__ WarpRanges s_r[PD_WARPS];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (!FILTERED && a.finish && blockIdx.x == 0 && threadIdx.x == 0) round_finish(a.finish);
     const int n1 = *a.qcount, n2 = FILTERED ? *a.qcount2 : 0;
     const int step = gridDim.x * PD_WARPS;
     for (int t = blockIdx.x * PD_WARPS + w; t < n1 + n2; t += step) {
@@ -1059,10 +1060,7 @@ __global__ void __launch_bounds__(PD_WARPS * 32, W ? 8 : 10) knn_query_kernel(Gr
 cudaError_t launch_knn_queries(const GridView& g, const KnnArgs& a, int64_t cap, cudaStream_t st) {
     if (cap <= 0) return cudaSuccess;
     const bool filtered = a.qlist2 != nullptr;
-    int64_t blocks = (cap + PD_WARPS - 1) / PD_WARPS;
-    const int64_t lim = (int64_t)device_sms() * 10;
-    if (blocks > lim) blocks = lim;
-    const dim3 gr((unsigned)blocks), bl(PD_WARPS * 32);
+    const dim3 gr(list_blocks(cap, 128, 10)), bl(PD_WARPS * 32);
     if (filtered) {
         if (a.term != 0) knn_query_kernel<true, true><<<gr, bl, 0, st>>>(g, a);
         else knn_query_kernel<true, false><<<gr, bl, 0, st>>>(g, a);

@@ -189,6 +189,45 @@ __device__ inline unsigned long long sqd(int4 a, int4 b) {
     return (unsigned long long)(dx * dx + dy * dy + dz * dz);
 }
 
+// ---------------------------------------------------------------- stored neighbours
+// The 8 stored neighbours of a point, two 16-byte accesses (a scalar access per
+// entry touches every line of the warp's kilobyte 8 times).
+__device__ __forceinline__ void load_nbr8(const int* __restrict__ nbr, long long s, int (&x)[8]) {
+    const int4* p = reinterpret_cast<const int4*>(nbr + s * 8);
+    const int4 a = p[0], b = p[1];
+    x[0] = a.x;
+    x[1] = a.y;
+    x[2] = a.z;
+    x[3] = a.w;
+    x[4] = b.x;
+    x[5] = b.y;
+    x[6] = b.z;
+    x[7] = b.w;
+}
+__device__ __forceinline__ void store_nbr8(int* nbr, long long s, const int (&x)[8]) {
+    int4* p = reinterpret_cast<int4*>(nbr + s * 8);
+    p[0] = make_int4(x[0], x[1], x[2], x[3]);
+    p[1] = make_int4(x[4], x[5], x[6], x[7]);
+}
+// Moves the live entries to the front, in order, and sets the rest to -1 (in
+// registers: every index is a compile-time one); returns their number.
+__device__ __forceinline__ int keep_live8(const uint8_t* __restrict__ alive, int (&x)[8]) {
+    bool live[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++) live[i] = x[i] >= 0 && alive[x[i]];
+    int r = 0;
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        const int v = x[i];
+        x[i] = -1;
+#pragma unroll
+        for (int j = 0; j <= i; j++)
+            if (live[i] && j == r) x[j] = v;
+        r += live[i];
+    }
+    return r;
+}
+
 // ---------------------------------------------------------------- launches
 // Number of kernels this library has launched (process-wide, host counter).
 extern long long g_launch_count;

@@ -62,8 +62,9 @@ cudaError_t launch_take_xyz(const int* list, const int* count, int64_t cap, cons
                             int32_t* out, cudaStream_t st);
 
 // ---------------------------------------------------------------- round state
-#define PD_FIX_ITERS 32    // device fixpoint sweeps of a k = 1 round (the most)
-#define PD_FIX_ITERS_KK 8  // ... of a k >= 2 round (danger pairs)
+#define PD_FIX_ITERS 6     // fixpoint launches of a k = 1 round (the most), each of up to
+#define PD_FIX_ITERS_KK 3  //   PD_FIX_INNER sweeps, and of a k >= 2 round (danger pairs)
+#define PD_FIX_INNER 16
 
 // ---------------------------------------------------------------- packed batches
 // Many independent scans decimated in one grid (batch.cu).  Scan i is moved
@@ -72,15 +73,16 @@ cudaError_t launch_take_xyz(const int* list, const int* count, int64_t cap, cons
 // and every scan occupies one contiguous range of the Morton order.  The
 // removal threshold of a round (R2) is selected per scan.
 #define PD_SEG_MAX 4096      // scans of one packed batch (16 tiles per axis)
-#define PD_SEG_CHUNK 8192    // grid positions per work item of the per-scan passes
+#define PD_SEG_CHUNK 4096    // grid positions per work item of the per-scan passes
 struct SegDev {
     long long live, m, need, rank;
     unsigned long long tau_prim;  // this round's threshold (~0: nothing to remove)
     int tau_idx;
     int done;                     // selection finished for this round
     unsigned pre[8];
-    int len[2];                   // selection lists: [b, b + len) of the ping-pong buffers
+    int len;                      // selection list: [b, b + len) of the list buffers
     int b, e;                     // the scan's grid positions [b, e)
+    unsigned ticket;              // blocks that finished a pass over the scan (0 between)
 };
 
 // Per-round control block in device memory (read by the host once per round).
@@ -93,7 +95,9 @@ struct RoundDev {
     int tau_idx;
     int done;
     unsigned pre[8];
-    int len[2];
+    int len;                   // length of the selection list
+    unsigned ticket;           // blocks that finished a launch (0 between launches)
+    int finished;              // the round's counts are added up
     int ncand, nslow, nsrc, npairs, overflow;
     int nreq, nfq, nlq;  // this round's re-searches, filtered and lambda searches
     int ndep;  // k = 1: candidates with a shell member of larger input index
@@ -131,9 +135,9 @@ __device__ __forceinline__ void round_tau(const RoundDev* rd, int4 p, unsigned l
 #endif
 
 struct SelBuffers {
-    u64* p[2];
-    int* i[2];
-    uint32_t* hist;
+    u64* p;  // the selection list: keys and input indices
+    int* i;
+    uint32_t* hist;  // 4096 words, zero between launches
 };
 
 // ---------------------------------------------------------------- knn.cu
@@ -172,6 +176,7 @@ struct KnnArgs {
     // points of qlist whose cost over smaller keys equals their own join the
     // candidates (inP, its bitmap inPb, cand, *ncand); lam_out of those of qlist2
     // takes the k-th squared distance over keys below the threshold.
+    RoundDev* finish;         // full searches: the round to add up
     const int* qlist;
     const int* qcount;
     const int* qlist2;
@@ -202,15 +207,60 @@ struct SelectResult {
 
 namespace pd {
 // ---------------------------------------------------------------- rounds_dev.cu
-cudaError_t round_launch_setup(RoundDev* rd, cudaStream_t st);
+// Sizes of launches that walk lists whose length the device knows: n / per
+// blocks, at most `per_sm` per multiprocessor (an idle block costs about as
+// much as a little work).
+inline unsigned list_blocks(int64_t n, int64_t per, int per_sm) {
+    int64_t b = n / per + 1;
+    const int64_t lim = (int64_t)device_sms() * per_sm;
+    return (unsigned)(b < lim ? b : lim);
+}
 // The candidate band of the next round (k >= 2 and weighted costs) from this
 // round's counts; the same arithmetic runs on the device after a normal round
 // and on the host after a round it settled.
-double host_next_band(double band, double band_max, int band_mode, unsigned long long cap_over,
-                      long long ncand, unsigned long long removed);
-cudaError_t round_launch_finish(RoundDev* rd, cudaStream_t st);
+__device__ __host__ inline double next_band(double band, double band_max, int band_mode,
+                                            unsigned long long cap_over, long long ncand,
+                                            unsigned long long removed) {
+    bool shrink = cap_over != 0;
+    double grow = 1.5;
+    if (band_mode == 1) {
+        double yield = ncand > 0 ? (double)removed / ncand : 1.0;
+        shrink = shrink || yield < 0.5;
+        grow = yield > 0.8 ? 1.25 : 1.0;
+    }
+    double b = shrink ? band * 0.5 : band * grow;
+    if (b > band_max) b = band_max;
+    if (b < 1e-7) b = 1e-7;
+    return b;
+}
+#ifdef __CUDACC__
+// Adds up a round once its removals and re-search list are complete; one
+// thread of the re-search launch calls it.
+__device__ inline void round_finish(RoundDev* rd) {
+    if (rd->seg) rd->tau_prim = ~0ull;  // the next selection lowers it
+    if (rd->finished) return;  // the second update of a round settled on the host
+    rd->finished = 1;
+    rd->live -= (long long)rd->removed;
+    rd->tot_sources += (unsigned long long)rd->nsrc;
+    rd->tot_filtered += (unsigned long long)rd->nfq;
+    rd->tot_lambda += (unsigned long long)rd->nlq;
+    rd->tot_requery += (unsigned long long)rd->nreq;
+    // a held round (settled on the host) updates its band there, from the
+    // points it finally removes: the band must not depend on whether the
+    // device fixpoint happened to converge within its sweeps
+    if (!rd->density_k1 && !(rd->overflow || rd->fix_unconverged)) {
+        rd->band = next_band(rd->band, rd->band_max, rd->band_mode, rd->cap_over, rd->ncand,
+                             rd->removed);
+    }
+}
+#endif
+// select.cu: the round's threshold (rank from the live count, target and
+// band), and the round's counters opened.  long_list: the list of the keys that
+// agree in their leading digits is walked by the whole grid, not by one cluster
+// (the caller's guess from the round before, PD_SEL_LONG; either is correct).
+#define PD_SEL_LONG 262144
 cudaError_t round_launch_select(const u64* prim, const int4* pos, const uint8_t* alive, int64_t n,
-                                SelBuffers& b, RoundDev* rd, cudaStream_t st);
+                                SelBuffers& b, bool long_list, RoundDev* rd, cudaStream_t st);
 // dep: list of the candidates that have a shell member of larger input index
 // (the only ones condition (B) can reject; the fixpoint sweeps walk it).
 // nbr0: the first stored entries apart (may be NULL).
@@ -222,11 +272,11 @@ cudaError_t round_launch_k1(const GridView& g, const u64* prim, const uint8_t* a
 cudaError_t round_launch_danger(const GridView& g, const int* src, const u64* prim,
                                 const uint8_t* alive, const uint32_t* inPb, uint8_t* rej,
                                 const u64* lam, const int* nbr, int S, int k, int2* pairs,
-                                int pair_cap, RoundDev* rd, cudaStream_t st);
+                                int pair_cap, int64_t n, RoundDev* rd, cudaStream_t st);
 cudaError_t round_launch_pairs_fix(const int2* pairs, int pair_cap, const uint8_t* inP,
-                                   uint8_t* rej, RoundDev* rd, cudaStream_t st);
+                                   uint8_t* rej, int64_t n, RoundDev* rd, cudaStream_t st);
 cudaError_t round_launch_remove(const int* cand, uint8_t* inP, uint8_t* rej, uint8_t* alive,
-                                RoundDev* rd, cudaStream_t st);
+                                int64_t n, RoundDev* rd, cudaStream_t st);
 // Lists (list[0 .. rd->nreq)) the live points that lost one of their first
 // kchk stored neighbours.
 cudaError_t round_launch_dirty(const uint8_t* alive, const int* nbr, int64_t n, int S, int kchk,
@@ -295,10 +345,8 @@ cudaError_t launch_sample_rows(const int* pool, int64_t npool, u64 seed, long lo
 cudaError_t launch_normal_fallback(const float* mlp, const float* onorm, const float* pca,
                                    int64_t n, float min_norm, float* out, cudaStream_t st);
 // ---------------------------------------------------------------- wup.cu
-// The paper's iterative w_up scheme: set the rank (live - m) for the key
-// selection of w_up, then run one removal round (marks, picks, removal,
+// The paper's iterative w_up scheme: one removal round (marks, picks, removal,
 // stored-list update).  S <= 8, k <= S.
-cudaError_t wup_launch_setup(RoundDev* rd, cudaStream_t st);
 // Replace the selection's bin boundary by the smallest live key at or above
 // it (the exact rank-th largest key).  tmin, imin: device scratch words.
 cudaError_t wup_launch_exact_tau(const u64* prim, const int4* pos, const uint8_t* alive,
@@ -339,7 +387,7 @@ cudaError_t seg_launch_ranges(const int4* pos, int64_t ng, SegDev* seg, int* chu
 // nseg x 4096 words, zero on entry and on return.
 cudaError_t seg_launch_select(const u64* prim, const int4* pos, const uint8_t* alive, int64_t ng,
                               SelBuffers& b, uint32_t* hist, RoundDev* rd, SegDev* seg,
-                              const int* chunk0, const int* items, int nseg, cudaStream_t st);
+                              const int* items, int nseg, cudaStream_t st);
 // cnt[scan] += flagged points of the scan.
 cudaError_t seg_launch_count(const uint8_t* flag, const int4* pos, int64_t ng, int shift,
                              unsigned long long* cnt, cudaStream_t st);

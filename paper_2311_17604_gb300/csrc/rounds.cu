@@ -586,8 +586,8 @@ cudaError_t launch_k1_fix(const int* cand, const int* ncand, int max_cand, const
 cudaError_t round_launch_danger(const GridView& g, const int* src, const u64* prim,
                                 const uint8_t* alive, const uint32_t* inPb, uint8_t* rej,
                                 const u64* lam, const int* nbr, int S, int k, int2* pairs,
-                                int pair_cap, RoundDev* rd, cudaStream_t st) {
-    danger_kernel<<<device_sms() * DG_BLOCKS_PER_SM, DG_WARPS * 32, 0, st>>>(
+                                int pair_cap, int64_t n, RoundDev* rd, cudaStream_t st) {
+    danger_kernel<<<list_blocks(n, 128, DG_BLOCKS_PER_SM), DG_WARPS * 32, 0, st>>>(
         g, src, &rd->nsrc, prim, alive, inPb, rej, lam, S <= PD_DG_SMAX ? nbr : nullptr, S, k,
         pairs, &rd->npairs, pair_cap, &rd->overflow, &rd->cap_over); note_launch();
     return cudaGetLastError();

@@ -30,23 +30,11 @@
 namespace pd {
 
 #define FULLM 0xffffffffu
-#define WUP_SMAX 8
 
 __device__ __forceinline__ bool wup_cand(const uint8_t* __restrict__ alive,
                                          const uint8_t* __restrict__ wdirty, u64 p, int i,
                                          const RoundDev* rd, int64_t s) {
     return alive[s] && !wdirty[s] && !key_gt(rd->tau_prim, rd->tau_idx, p, i);
-}
-
-__global__ void wup_setup_kernel(RoundDev* rd) {
-    if (threadIdx.x != 0) return;
-    rd->need = rd->live - rd->m;
-    rd->rank = rd->need;  // the need-th largest key is the smallest one above w_up
-    rd->done = 0;
-    rd->len[0] = rd->len[1] = 0;
-    rd->ncand = 0;
-    rd->removed = 0;
-    rd->overflow = 0;
 }
 
 // The key selection returns the lower boundary of the bin that holds the
@@ -150,30 +138,20 @@ __global__ void wup_update_kernel(BufView b, const uint8_t* __restrict__ alive, 
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     bool upd = false;
     if (s < n && alive[s] && !wdirty[s]) {
-        int ids[WUP_SMAX];
-        int r = 0;
+        int ids[8];
+        load_nbr8(b.nbr, s, ids);
         bool dead = false;
 #pragma unroll
-        for (int i = 0; i < WUP_SMAX; i++) {
-            ids[i] = -1;
-            if (i < S) {
-                int x = b.nbr[s * S + i];
-                if (x >= 0) {
-                    if (alive[x]) ids[r++] = x;
-                    else dead = true;
-                }
-            }
-        }
+        for (int i = 0; i < 8; i++) dead |= ids[i] >= 0 && !alive[ids[i] >= 0 ? ids[i] : s];
         if (dead) {
-#pragma unroll
-            for (int i = 0; i < WUP_SMAX; i++)
-                if (i < S) b.nbr[s * S + i] = ids[i];
+            const int r = keep_live8(alive, ids);
+            store_nbr8(b.nbr, s, ids);
             if (r >= k) {
                 int4 ps = b.pos[s];
                 double c = 0.0;
                 u64 dk = 0;
 #pragma unroll
-                for (int i = 0; i < WUP_SMAX; i++) {
+                for (int i = 0; i < 8; i++) {
                     if (i < k) {
                         u64 d2 = sqd(ps, b.pos[ids[i]]);
                         c = __dadd_rn(c, __ddiv_rn(1.0, (double)d2));
@@ -192,12 +170,6 @@ __global__ void wup_update_kernel(BufView b, const uint8_t* __restrict__ alive, 
 }
 
 #define WGRID(n) (unsigned)(((n) + 255) / 256), 256
-
-cudaError_t wup_launch_setup(RoundDev* rd, cudaStream_t st) {
-    wup_setup_kernel<<<1, 32, 0, st>>>(rd);
-    note_launch();
-    return cudaGetLastError();
-}
 
 // w_up as a key: tau <- the smallest live key >= the selection's boundary.
 // tw: one u64 and one int of device scratch.
@@ -219,7 +191,7 @@ cudaError_t wup_launch_exact_tau(const u64* prim, const int4* pos, const uint8_t
 cudaError_t wup_launch_round(const BufView& b, uint8_t* alive, uint8_t* wdirty, int64_t n, int S,
                              int k, RoundDev* rd, u64* mark_p, int* mark_i, uint8_t* pick,
                              cudaStream_t st) {
-    if (S > WUP_SMAX || k > S || n <= 0) return cudaErrorInvalidValue;
+    if (S != 8 || k > S || n <= 0) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(mark_p, 0, (size_t)n * sizeof(u64), st);
     if (!e) e = cudaMemsetAsync(mark_i, 0xff, (size_t)n * sizeof(int), st);
     if (e) return e;
