@@ -1889,6 +1889,8 @@ extern "C" int pd_quality_report(pd_ctx* ctx, const int32_t* xyz_dev, const uint
         QGET(sn, u64, nr);
         QGET(sn2, u64, nr);
         QGET(hist, uint32_t, (size_t)nr * H);
+        int* next;
+        QGET(next, int, 1);
         std::vector<u64> hr2(nr);
         for (int j = 0; j < nr; j++) hr2[j] = (u64)radii_mm[j] * (u64)radii_mm[j];
         QCK(cudaMemcpyAsync(r2, hr2.data(), nr * sizeof(u64), cudaMemcpyHostToDevice, st));
@@ -1896,7 +1898,8 @@ extern "C" int pd_quality_report(pd_ctx* ctx, const int32_t* xyz_dev, const uint
         QCK(cudaMemsetAsync(sn2, 0, nr * sizeof(u64), st));
         QCK(cudaMemsetAsync(hist, 0, (size_t)nr * H * sizeof(uint32_t), st));
         QCK(cudaEventRecord(c0, st));
-        QCK(launch_radius_counts(view_of(g), P, L, r2, nr, sn, sn2, hist, H, st));
+        QCK(launch_radius_counts(view_of(g), g->groups, g->ngroups, L, radii_mm[nr - 1], r2, nr, sn,
+                                 sn2, hist, H, next, st));
         QCK(cudaEventRecord(c1, st));
         std::vector<u64> T(nr), U(nr);
         std::vector<uint32_t> hh((size_t)nr * H);
