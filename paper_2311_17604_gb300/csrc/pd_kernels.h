@@ -328,21 +328,21 @@ void api_error(pd_ctx* c, const char* what, long long v);
 int grid_knn16(pd_grid* g, cudaStream_t st, GridNbrs* out);
 cudaError_t launch_features(const int4* pos, const int* nbr, int S, int64_t n, uint16_t* feat,
                             float* pca, uint8_t* valid, cudaStream_t st);
-cudaError_t launch_mlp_forward(const float* prm, const uint16_t* feat, const int* rows, int64_t n,
-                               float* outn, float* onorm, float* h1s, float* h2s, float* raw,
-                               cudaStream_t st);
+cudaError_t launch_mlp_forward(const float* prm, const uint16_t* feat, int64_t n, float* outn,
+                               float* onorm, cudaStream_t st);
 // Partials: mlp_backward_part_floats() floats of scratch; the gradient is
 // reduced over blocks in a fixed order (deterministic).
 int64_t mlp_backward_part_floats();
-cudaError_t launch_mlp_backward(const float* prm, const uint16_t* feat, const int* rows,
-                                const float* labels, int64_t n, const float* h1s,
-                                const float* h2s, const float* raw, float* grad, float* loss,
-                                float* part, cudaStream_t st);
-cudaError_t launch_adam(float* prm, float* m, float* v, const float* grad, int t, float lr,
-                        cudaStream_t st);
+// Mean loss and gradient over rows 0..n-1.
+cudaError_t launch_mlp_gradient(const float* prm, const uint16_t* feat, const float* labels,
+                                int64_t n, float* grad, float* loss, float* part,
+                                cudaStream_t st);
+// Step t (1-based) of Adam over b rows sampled from the pool.  overlap: the
+// launch ahead in the stream is the step before (its tail may overlap).
+cudaError_t launch_mlp_step(float* prm, float* m, float* v, const uint16_t* feat, const int* pool,
+                            int64_t npool, u64 seed, int t, const float* labels, int64_t b,
+                            float lr, float* loss, float* part, bool overlap, cudaStream_t st);
 cudaError_t launch_mlp_init(float* prm, u64 seed, cudaStream_t st);
-cudaError_t launch_sample_rows(const int* pool, int64_t npool, u64 seed, long long t, int b,
-                               int* rows, cudaStream_t st);
 cudaError_t launch_normal_fallback(const float* mlp, const float* onorm, const float* pca,
                                    int64_t n, float min_norm, float* out, cudaStream_t st);
 // ---------------------------------------------------------------- wup.cu
