@@ -658,7 +658,10 @@ struct Span {
 int knn_all(pd_grid* g, const pd_cost_params* cp, double* cost_s) {
     KnnArgs a = base_args(g, cp);
     a.cost_out = cost_s;
-    CK(launch_knn(view_of(g), a, g->st));
+    Temps tmp(g);
+    int* rest;
+    TALLOC(tmp, rest, int, g->ng);
+    CK(launch_knn(view_of(g), a, g->ng, rest, g->d_int + 7, g->st));
     return PD_OK;
 }
 
@@ -1077,6 +1080,8 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
         CK(seg_launch_ranges(g->pos, g->ng, g->seg, g->seg_chunk0, g->seg_items, g->nseg,
                              g->seg_shift, g->st));
     // ---- first neighbour pass
+    int* rq;  // the queries it leaves to the per-query search; later a round's re-searches
+    RALLOC(rq, int, g->n);
     {
         unsigned long long* dpairs;
         RALLOC(dpairs, unsigned long long, PD_PAIR_SLOTS);
@@ -1085,7 +1090,7 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
             Span t(T, &g->stats.ms_knn_first);
             KnnArgs a = base_args(g, cp);
             a.pairs_out = dpairs;
-            CK(launch_knn(view_of(g), a, g->st));
+            CK(launch_knn(view_of(g), a, g->ng, rq, g->d_int + 7, g->st));
         }
         unsigned long long hp[PD_PAIR_SLOTS];
         CK(cudaMemcpyAsync(hp, dpairs, sizeof(hp), cudaMemcpyDeviceToHost, g->st));
@@ -1100,13 +1105,12 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
     bool use_buf = !g->density_k1 && S <= 8;
     uint8_t *inP, *rej;
     uint32_t* inPb = nullptr;  // bitmap of inP
-    int *cand, *slow, *rq, *fq = nullptr, *lq = nullptr, *src = nullptr, *dep = nullptr;
+    int *cand, *slow, *fq = nullptr, *lq = nullptr, *src = nullptr, *dep = nullptr;
     u64* lam = nullptr;
     int2* pairs = nullptr;
     int64_t cap = g->n;
     RALLOC(inP, uint8_t, cap);
     RALLOC(rej, uint8_t, cap);
-    RALLOC(rq, int, cap);
     RALLOC(cand, int, cap);
     RALLOC(slow, int, cap);
     if (g->density_k1) RALLOC(dep, int, cap);
@@ -1421,6 +1425,8 @@ static int wup_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* ke
     uint8_t *wdirty, *pick;
     u64* mark_p;
     int* mark_i;
+    int* rest;
+    RALLOC(rest, int, cap);
     RALLOC(wdirty, uint8_t, cap);
     RALLOC(pick, uint8_t, cap);
     RALLOC(mark_p, u64, cap);
@@ -1454,7 +1460,7 @@ static int wup_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* ke
             Span t(T, &g->stats.ms_knn);
             KnnArgs a = base_args(g, &c2);
             a.qflag = g->alive;
-            CK(launch_knn(view_of(g), a, g->st));
+            CK(launch_knn(view_of(g), a, g->ng, rest, g->d_int + 7, g->st));
         }
         CK(cudaMemsetAsync(wdirty, 0, g->ng, g->st));
         // 2. w_up: the (live - m)-th largest key is the smallest one above it
@@ -1738,7 +1744,10 @@ int grid_knn16(pd_grid* g, cudaStream_t st, GridNbrs* out) {
     if (rc) return rc;
     KnnArgs a = base_args(g, &cp);
     a.term = PD_TERM_INDEX_TIE;
-    CK(launch_knn(view_of(g), a, g->st));
+    Temps tmp(g);
+    int* rest;
+    TALLOC(tmp, rest, int, g->ng);
+    CK(launch_knn(view_of(g), a, g->ng, rest, g->d_int + 7, g->st));
     out->pos = g->pos;
     out->nbr = g->nbr;
     out->S = g->S;

@@ -195,7 +195,10 @@ extern "C" int pd_knn_cost_static(const int32_t* xyz_dev, int64_t n, int k, doub
     a.flg_out = flg;
     a.hz_out = hz;
     a.cost_out = cost_s;
-    SCK(launch_knn(g, a, st));
+    int *rest, *nrest;
+    SGET(rest, int, n);
+    SGET(nrest, int, 1);
+    SCK(launch_knn(g, a, n, rest, nrest, st));
     SCK(launch_knn_out(pos, cost_s, nbr, n, S, k, cost_dev, knn_dev, st));
     SCK(cudaStreamSynchronize(st));
     return PD_OK;

@@ -178,6 +178,8 @@ struct KnnArgs {
     // candidates (inP, its bitmap inPb, cand, *ncand); lam_out of those of qlist2
     // takes the k-th squared distance over keys below the threshold.
     RoundDev* finish;         // full searches: the round to add up
+    int ordered;              // equal distances in Morton order (term 0; with a term they are
+                              //   always in input order)
     const int* qlist;
     const int* qcount;
     const int* qlist2;
@@ -190,8 +192,11 @@ struct KnnArgs {
     const u64* cmin;          // filtered searches: least live key primary of every aligned
                               //   32-position chunk (chunks above the threshold are skipped)
 };
-// Full searches of every point (a.qflag: of the flagged ones), a warp per leaf group.
-cudaError_t launch_knn(const GridView& g, const KnnArgs& a, cudaStream_t st);
+// Full searches of every point (a.qflag: of the flagged ones), a warp per leaf
+// group, then a warp for each query that is left.  rest: n ints and nrest: one
+// int, device scratch.
+cudaError_t launch_knn(const GridView& g, const KnnArgs& a, int64_t n, int* rest, int* nrest,
+                       cudaStream_t st);
 // Searches of the listed queries, one warp each; at most cap of them.
 cudaError_t launch_knn_queries(const GridView& g, const KnnArgs& a, int64_t cap, cudaStream_t st);
 // Internal neighbour-weight term: unit weights with equal distances ordered by
