@@ -1160,6 +1160,7 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
     h.band_max = band_max;
     h.density_k1 = g->density_k1;
     h.band_mode = getenv("PD_BAND_MODE") ? atoi(getenv("PD_BAND_MODE")) : 1;
+    h.density = cp->term == PD_TERM_NONE;
     h.fix_iters = g->density_k1 ? PD_FIX_ITERS : PD_FIX_ITERS_KK;
     if (g->density_k1 && getenv("PD_FIX_SWEEPS"))  // fewer sweeps: more rounds settled on the host
         h.fix_iters = std::max(1, std::min(PD_FIX_ITERS, atoi(getenv("PD_FIX_SWEEPS"))));
@@ -1326,8 +1327,8 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
             h.removed = (unsigned long long)removed;
             if (!g->density_k1) {
                 // an overflowing round always narrows the band, as before
-                h.band = next_band(h.band, h.band_max, h.band_mode,
-                                        h.cap_over + (h.overflow ? 1 : 0), h.ncand, h.removed);
+                h.band = next_band(h.band, h.band_max, h.band_mode, h.density, h.live,
+                                   h.cap_over + (h.overflow ? 1 : 0), h.ncand, h.removed);
                 CK(cudaMemcpyAsync(&rd->band, &h.band, sizeof(h.band), cudaMemcpyHostToDevice,
                                    g->st));
             }

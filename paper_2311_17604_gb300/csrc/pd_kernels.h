@@ -105,6 +105,7 @@ struct RoundDev {
     int changed[PD_FIX_ITERS];
     int fix_unconverged;
     int density_k1;
+    int density;    // no colour or orientation weights: any band gives the same result
     int band_mode;  // 0: shrink on overflow only; 1: also on poor yield
     int fix_iters;  // device fixpoint sweeps per round (<= PD_FIX_ITERS)
     // packed batch (NULL seg: one scan).  Then tau_prim above is the least
@@ -224,15 +225,24 @@ inline unsigned list_blocks(int64_t n, int64_t per, int per_sm) {
 // The candidate band of the next round (k >= 2 and weighted costs) from this
 // round's counts; the same arithmetic runs on the device after a normal round
 // and on the host after a round it settled.
+//   density: any band gives the same result.  A poor yield then never narrows
+// it below PD_BAND_LEAST keys: a round costs its passes over the cloud whatever
+// it removes, and a dense spot without lower keys nearby yields few points of a
+// wide band but fewer still of a narrow one.  Only candidate lists that
+// overflow (cap_over, which make the danger test expensive) narrow it further.
+#define PD_BAND_LEAST 1024
 __device__ __host__ inline double next_band(double band, double band_max, int band_mode,
+                                            int density, long long live,
                                             unsigned long long cap_over, long long ncand,
                                             unsigned long long removed) {
     bool shrink = cap_over != 0;
     double grow = 1.5;
     if (band_mode == 1) {
         double yield = ncand > 0 ? (double)removed / ncand : 1.0;
-        shrink = shrink || yield < 0.5;
-        grow = yield > 0.8 ? 1.25 : 1.0;
+        const bool least = density && band * (double)live <= PD_BAND_LEAST;
+        shrink = shrink || (yield < 0.5 && !least);
+        grow = yield > 0.8 ? (density ? 1.5 : 1.25) : 1.0;
+        if (density && least && !shrink) grow = 1.5;
     }
     double b = shrink ? band * 0.5 : band * grow;
     if (b > band_max) b = band_max;
@@ -255,8 +265,8 @@ __device__ inline void round_finish(RoundDev* rd) {
     // points it finally removes: the band must not depend on whether the
     // device fixpoint happened to converge within its sweeps
     if (!rd->density_k1 && !(rd->overflow || rd->fix_unconverged)) {
-        rd->band = next_band(rd->band, rd->band_max, rd->band_mode, rd->cap_over, rd->ncand,
-                             rd->removed);
+        rd->band = next_band(rd->band, rd->band_max, rd->band_mode, rd->density, rd->live,
+                             rd->cap_over, rd->ncand, rd->removed);
     }
 }
 #endif

@@ -197,7 +197,9 @@ __device__ inline int cover_level(const GridView& g, int ux, int uy, int uz, int
 // end (32 bitmap words, then 32 points a step, the next step's loads issued
 // before this step's are used) instead of walked one by one, and octree nodes
 // above DG_SCAN points are entered by their children (9.8M outdoor points, k =
-// 4, 287 rounds: 95.6 -> 47.3 ms).
+// 4, 287 rounds: 95.6 -> 47.3 ms).  Candidates that the shields at hand leave open
+// are gathered before the ball is streamed, so that it is streamed once per 32 of
+// them (1.0M room points, k = 4, 112 rounds at 2 %: 9.7 -> 7.2 ms).
 struct DangerSmem {
     int c_j[DG_WARPS][DG_CAP];
     u64 c_d[DG_WARPS][DG_CAP];
@@ -317,85 +319,128 @@ __device__ void danger_one(const GridView& g, int x, const u64* __restrict__ pri
             sn_i = v.w;
         }
     }
-    // 2. counting, 32 candidates at a time
+    // 2. counting, 32 candidates at a time: this lane's
+    int p = -1, ip = 0, cnt = 0;
+    u64 dp = 0, pp = 0, dmax = 0, kmax = 0;
+    bool done = true;
+    auto take = [&](int at, int nlist) {
+        done = at >= nlist;
+        p = done ? -1 : c_j[at];
+        dp = done ? 0 : c_d[at];
+        pp = done ? 0 : prim[p];
+        ip = done ? 0 : g.pos[p].w;
+        cnt = 0;
+    };
+    // the farthest distance and the largest key of the open candidates
+    auto reach = [&]() {
+        dmax = done ? 0 : dp;
+        kmax = done ? 0 : pp;
+        for (int o = 16; o; o >>= 1) {
+            const u64 d = __shfl_xor_sync(FULLM, dmax, o), q = __shfl_xor_sync(FULLM, kmax, o);
+            dmax = d > dmax ? d : dmax;
+            kmax = q > kmax ? q : kmax;
+        }
+    };
+    // the open candidates move to the front of the list, from place `to` on
+    auto keep_open = [&](int to) -> int {
+        const unsigned m = __ballot_sync(FULLM, !done);
+        __syncwarp();  // this batch was read
+        if (!done) {
+            const int at = to + __popc(m & ((1u << lane) - 1u));
+            c_j[at] = p;
+            c_d[at] = dp;
+        }
+        __syncwarp();
+        return to + __popc(m);
+    };
+    // Streams the lanes' ranges [b, b + len): true once every count reached k.
+    auto stream = [&](uint32_t b, uint32_t len) -> bool {
+        const uint32_t inc = warp_inclusive(len, lane);
+        const uint32_t total = __shfl_sync(FULLM, inc, 31);
+        uint32_t jn = 0;  // a step's point: its fields loaded one step ahead
+        int4 vn = make_int4(0, 0, 0, 0);
+        u64 kn = 0;
+        uint8_t an = 0;
+        auto load = [&](uint32_t t) {
+            const int r = range_of(inc, t < total ? t : total - 1);
+            jn = __shfl_sync(FULLM, b, r) +
+                 (t - (__shfl_sync(FULLM, inc, r) - __shfl_sync(FULLM, len, r)));
+            an = 0;
+            if (t < total) {
+                an = alive[jn];
+                vn = g.pos[jn];
+                kn = prim[jn];
+            }
+        };
+        if (total) load(lane);
+        for (uint32_t base = 0; base < total; base += 32) {
+            const uint32_t j = jn;
+            const int4 v = vn;
+            const u64 ky = kn;
+            const uint8_t al = an;
+            load(base + 32 + lane);
+            // only points within the farthest open candidate and of smaller
+            // key than the largest can shield: they are compacted into the
+            // staging buffer
+            const u64 d2 = sqd(v, xp);
+            const bool near = al && (int)j != x && d2 <= dmax && ky <= kmax;
+            const unsigned nb = __ballot_sync(FULLM, near);
+            if (!nb) continue;
+            if (near) {
+                const int slot = __popc(nb & ((1u << lane) - 1u));
+                u.st.d[slot] = d2;
+                u.st.k[slot] = ky;
+                u.st.o[slot] = v.w;
+                u.st.j[slot] = (int)j;
+            }
+            __syncwarp();
+            const int mm = __popc(nb);
+            if (!done) {
+                for (int tt = 0; tt < mm; tt++) {
+                    if (u.st.j[tt] == p) continue;
+                    if (u.st.d[tt] <= dp && key_gt(pp, ip, u.st.k[tt], u.st.o[tt])) {
+                        if (++cnt >= k) {
+                            done = true;
+                            break;
+                        }
+                    }
+                }
+            }
+            __syncwarp();
+            if (__all_sync(FULLM, done)) return true;
+        }
+        return false;
+    };
+    // x's stored neighbours as shields
+    int no = 0;
     for (int a0 = 0; a0 < nc; a0 += 32) {
-        int a = a0 + lane;
-        bool done = a >= nc;
-        int p = done ? -1 : c_j[a];
-        u64 dp = done ? 0 : c_d[a];
-        u64 pp = done ? 0 : prim[p];
-        int ip = done ? 0 : g.pos[p].w;
-        int cnt = 0;
+        take(a0 + lane, nc);
         for (int i = 0; i < PD_DG_SMAX; i++) {
             const int yj = __shfl_sync(FULLM, sn_j, i), yi = __shfl_sync(FULLM, sn_i, i);
             const u64 yd = __shfl_sync(FULLM, sn_d, i), yk = __shfl_sync(FULLM, sn_k, i);
             if (yj >= 0 && yj != p && yd <= dp && key_gt(pp, ip, yk, yi)) cnt++;
         }
         if (cnt >= k) done = true;
-        cnt = 0;  // the stream below recounts every point (stored ones included)
-        if (__all_sync(FULLM, done)) continue;
-        u64 dmax = done ? 0 : dp;  // farthest candidate of this batch
-        for (int o2 = 16; o2; o2 >>= 1) {
-            u64 other = __shfl_xor_sync(FULLM, dmax, o2);
-            dmax = other > dmax ? other : dmax;
+        no = keep_open(no);
+    }
+    // many left: the points of the nearest cells as shields.  A candidate is
+    // dangerous only if its key is among the k smallest of all points closer to
+    // x, so few survive a hundred shields, and only batches of survivors stream
+    // the whole ball.
+    if (no > 32) {
+        const int m = no;
+        no = 0;
+        for (int a0 = 0; a0 < m; a0 += 32) {
+            take(a0 + lane, m);
+            reach();
+            const bool in = rt && lane < 7 && cell.count() <= DG_SCAN && cell.box <= dmax;
+            stream(cell.b, in ? cell.count() : 0);
+            no = keep_open(no);
         }
-        // Streams the lanes' ranges [b, b + len): true once every count reached k.
-        auto stream = [&](uint32_t b, uint32_t len) -> bool {
-            const uint32_t inc = warp_inclusive(len, lane);
-            const uint32_t total = __shfl_sync(FULLM, inc, 31);
-            uint32_t jn = 0;  // a step's point: its fields loaded one step ahead
-            int4 vn = make_int4(0, 0, 0, 0);
-            u64 kn = 0;
-            uint8_t an = 0;
-            auto load = [&](uint32_t t) {
-                const int r = range_of(inc, t < total ? t : total - 1);
-                jn = __shfl_sync(FULLM, b, r) +
-                     (t - (__shfl_sync(FULLM, inc, r) - __shfl_sync(FULLM, len, r)));
-                an = 0;
-                if (t < total) {
-                    an = alive[jn];
-                    vn = g.pos[jn];
-                    kn = prim[jn];
-                }
-            };
-            if (total) load(lane);
-            for (uint32_t base = 0; base < total; base += 32) {
-                const uint32_t j = jn;
-                const int4 v = vn;
-                const u64 ky = kn;
-                const uint8_t al = an;
-                load(base + 32 + lane);
-                // only points within the farthest open candidate can shield:
-                // they are compacted into the staging buffer
-                const u64 d2 = sqd(v, xp);
-                const bool near = al && (int)j != x && d2 <= dmax;
-                const unsigned nb = __ballot_sync(FULLM, near);
-                if (!nb) continue;
-                if (near) {
-                    const int slot = __popc(nb & ((1u << lane) - 1u));
-                    u.st.d[slot] = d2;
-                    u.st.k[slot] = ky;
-                    u.st.o[slot] = v.w;
-                    u.st.j[slot] = (int)j;
-                }
-                __syncwarp();
-                const int mm = __popc(nb);
-                if (!done) {
-                    for (int tt = 0; tt < mm; tt++) {
-                        if (u.st.j[tt] == p) continue;
-                        if (u.st.d[tt] <= dp && key_gt(pp, ip, u.st.k[tt], u.st.o[tt])) {
-                            if (++cnt >= k) {
-                                done = true;
-                                break;
-                            }
-                        }
-                    }
-                }
-                __syncwarp();
-                if (__all_sync(FULLM, done)) return true;
-            }
-            return false;
-        };
+    }
+    for (int a0 = 0; a0 < no; a0 += 32) {
+        take(a0 + lane, no);
+        reach();
         // small nodes at once, then the large ones by their children, nearest first
         WarpNode n = cell;
         const bool in = rt && n.box <= dmax;

@@ -116,12 +116,14 @@ __device__ void sel_take(State& S, const SelBin& f, long long r, int pass, Round
 }
 
 // What a round examines: everything above the target (k = 1), or a band of
-// the largest keys, at most a quarter of what must go.
+// the largest keys.
 __device__ inline long long sel_rank(const RoundDev* rd, long long live, long long need) {
     if (rd->density_k1) return need;
     const long long band = (long long)(rd->band * (double)live);
-    const long long quarter = (need + 3) / 4;
-    const long long rank = band < quarter ? band : quarter;
+    // with weights a quarter of what must go at most: their rounds are not
+    // provably the sequential order, and narrower ones stay closer to it
+    const long long most = rd->density ? need : (need + 3) / 4;
+    const long long rank = band < most ? band : most;
     return rank < 1 ? 1 : rank;
 }
 
