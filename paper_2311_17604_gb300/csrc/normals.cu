@@ -469,7 +469,7 @@ struct StepSmem {
     float dout[BT_ROWS][4];               // d loss / d o (divided by n)
     float red[BT_THREADS][4];             // end-of-kernel reductions
     float db1w[4][NH];                    // per-warp column sums of dh1
-    int row[BT_ROWS];
+    int64_t row[BT_ROWS];                 // feature row of each tile row
 };
 
 // Programmatic dependent launch: a launch that carries the attribute may start
@@ -530,13 +530,13 @@ __global__ void __launch_bounds__(BT_THREADS, BT_BLOCKS_PER_SM)
         const int nr = (int)min((int64_t)BT_ROWS, n - r0);
         const bool first = tile == blockIdx.x;
         __syncthreads();  // the previous tile's readers are done
-        if (tid < BT_ROWS) sm.row[tid] = tid < nr ? (int)rows.at(r0 + tid) : -1;
+        if (tid < BT_ROWS) sm.row[tid] = tid < nr ? rows.at(r0 + tid) : -1;
         __syncthreads();
         for (int i = tid; i < BT_ROWS * (NF / 8); i += BT_THREADS) {
             const int r = i / (NF / 8), c = 8 * (i % (NF / 8));
             uint4 v = make_uint4(0, 0, 0, 0);
             if (r < nr) {
-                const uint16_t* src = feat + (int64_t)sm.row[r] * NF + c;
+                const uint16_t* src = feat + sm.row[r] * NF + c;
                 if (vec_feat) {
                     v = *reinterpret_cast<const uint4*>(src);
                 } else {
