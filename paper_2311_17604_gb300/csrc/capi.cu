@@ -509,8 +509,7 @@ extern "C" int pd_build_grid(pd_ctx* ctx, const int32_t* xyz_dev, const uint8_t*
         Temps tmp(g);
         TALLOC(tmp, perm, uint32_t, n);
         Scratch s = scratch_of(g);
-        CK(launch_morton(xyz_dev, n, g->origin, g->shift, g->code, perm, g->st));
-        CK(radix_sort_pairs(g->code, perm, n, 3 * g->B, s, g->st));
+        CK(sort_points(xyz_dev, n, g->origin, g->shift, 3 * g->B, g->code, perm, s, g->st));
         ALLOC(g->pos, int4, n);
         if (rgb_dev) ALLOC(g->rgb, uchar4, n);
         CK(launch_gather(xyz_dev, rgb_dev, nullptr, perm, n, g->pos, g->rgb, nullptr, g->st));

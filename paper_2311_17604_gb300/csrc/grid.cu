@@ -46,22 +46,255 @@ cudaError_t launch_bbox(const int32_t* xyz, int64_t n, int* out6, cudaStream_t s
     return cudaGetLastError();
 }
 
-// ------------------------------------------------------------------ Morton
-__global__ void morton_kernel(const int32_t* __restrict__ xyz, int64_t n, int3 o, int shift,
-                              u64* __restrict__ keys, uint32_t* __restrict__ vals) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    uint32_t ux = (uint32_t)(xyz[3 * i] - o.x) >> shift;
-    uint32_t uy = (uint32_t)(xyz[3 * i + 1] - o.y) >> shift;
-    uint32_t uz = (uint32_t)(xyz[3 * i + 2] - o.z) >> shift;
-    keys[i] = morton3(ux, uy, uz);
-    vals[i] = (uint32_t)i;
+// ------------------------------------------------------------------ Morton order
+// Morton codes sorted with their input indices: a stable LSD radix sort of 8-bit
+// digits that reads and writes every pair once per pass.  The digits' totals
+// over the cloud do not depend on the order, so the code kernel counts all of
+// them at once; a pass then needs, for a tile, only the counts of the tiles
+// before it, which the tiles publish and look up while they run (the decoupled
+// look-back of Merrill and Garland, "Single-pass Parallel Prefix Scan with
+// Decoupled Look-back", NVIDIA NVR-2016-002; in a radix sort: Adinets and
+// Merrill, "Onesweep", arXiv 2206.01784).  Bound: the scattered writes and the
+// ranking.  A histogram launch, a scan of the tiles' counts (three to five
+// launches) and a scatter per pass read every key twice and were launch-bound
+// below a million points: neighbours and costs of 1.0M points 1016 -> 951 us, of
+// 7.4k 307 -> 262, the decimation of 200k 2.90 -> 2.77 ms, of 100M 134.0 -> 131.9.
+#define RS_T 256
+#define RS_MAXP 8  // passes of at most 3 PD_MAXLEVEL = 63 bits
+#define RS_SPIN 20000
+
+struct SortState {
+    uint32_t total[RS_MAXP][256];  // of each digit over the cloud
+    uint32_t ticket[RS_MAXP];      // next tile of a pass
+};
+
+__global__ void __launch_bounds__(256)
+    morton_kernel(const int32_t* __restrict__ xyz, int64_t n, int3 o, int shift,
+                  u64* __restrict__ keys, int passes, SortState* ss) {
+    __shared__ uint32_t h[RS_MAXP][256];
+    const int lane = threadIdx.x & 31;
+    for (int p = 0; p < passes; p++) h[p][threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t step = (int64_t)gridDim.x * 256;
+    for (int64_t b = blockIdx.x * (int64_t)256; b < n; b += step) {  // uniform over the block
+        const int64_t i = b + threadIdx.x;
+        const bool in = i < n;
+        u64 k = 0;
+        if (in) {
+            const uint32_t ux = (uint32_t)(xyz[3 * i] - o.x) >> shift;
+            const uint32_t uy = (uint32_t)(xyz[3 * i + 1] - o.y) >> shift;
+            const uint32_t uz = (uint32_t)(xyz[3 * i + 2] - o.z) >> shift;
+            k = morton3(ux, uy, uz);
+            keys[i] = k;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        if (!m) continue;
+        // neighbours in the scan share their leading digits: one addition then
+        for (int p = 0; p < passes; p++) {
+            const uint32_t d = (uint32_t)(k >> (8 * p)) & 255;
+            const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);  // lane 0 is in
+            if (__all_sync(0xffffffffu, !in || d == d0)) {
+                if (lane == 0) atomicAdd(&h[p][d0], (uint32_t)__popc(m));
+            } else if (in) {
+                atomicAdd(&h[p][d], 1u);
+            }
+        }
+    }
+    __syncthreads();
+    for (int p = 0; p < passes; p++)
+        if (h[p][threadIdx.x]) atomicAdd(&ss->total[p][threadIdx.x], h[p][threadIdx.x]);
 }
 
-cudaError_t launch_morton(const int32_t* xyz, int64_t n, int3 origin, int shift, u64* keys,
-                          uint32_t* vals, cudaStream_t st) {
-    morton_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(xyz, n, origin, shift, keys, vals); note_launch();
-    return cudaGetLastError();
+// Exclusive prefix sums of a and b over the 256 threads of a block.
+__device__ __forceinline__ void scan256(uint32_t& a, uint32_t& b, uint32_t (&ws)[2][8]) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t x = a, y = b;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xffffffffu, x, o), v = __shfl_up_sync(0xffffffffu, y, o);
+        if (lane >= o) {
+            x += u;
+            y += v;
+        }
+    }
+    if (lane == 31) {
+        ws[0][w] = x;
+        ws[1][w] = y;
+    }
+    __syncthreads();
+    x -= a;
+    y -= b;
+    for (int i = 0; i < w; i++) {
+        x += ws[0][i];
+        y += ws[1][i];
+    }
+    a = x;
+    b = y;
+}
+
+// One pass over tiles of 256 x PER keys, a warp ranking 32 x PER consecutive
+// ones.  The tile's pairs are placed in digit order in shared memory and written
+// from there, so that neighbouring threads write neighbouring addresses of a
+// digit's run.  status[tile][digit]: (tag, count), the tag 2 pass + 1 for the
+// tile's own count and 2 pass + 2 for the sum up to and including it (a pass
+// thus never takes an earlier one's words).  Tiles are handed out in order, so a
+// tile only waits for tiles that run; after RS_SPIN polls it counts the other
+// tile's digit itself, so that no wait is without end.
+template <int PER>
+__global__ void __launch_bounds__(RS_T, 2)
+    radix_pass_kernel(const u64* __restrict__ kin, const uint32_t* __restrict__ vin,
+                      u64* __restrict__ kout, uint32_t* __restrict__ vout, int64_t n, int pass,
+                      SortState* ss, u64* status) {
+    const int TILE = RS_T * PER;
+    __shared__ u64 sk[RS_T * PER];     // the tile's keys, then its values
+    __shared__ uint32_t wc[8][256];    // counts of a warp, then of the warps before it
+    __shared__ uint32_t first[256];    // first slot of a digit in the tile
+    __shared__ uint32_t to[256];       // where slot x of a digit goes: to[digit] + x
+    __shared__ uint32_t ws[2][8];
+    __shared__ int s_tile;
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31, shift = 8 * pass;
+    if (t == 0) s_tile = (int)atomicAdd(&ss->ticket[pass], 1u);
+#pragma unroll
+    for (int i = 0; i < 8; i++) wc[i][t] = 0;
+    __syncthreads();
+    const int tile = s_tile;
+    const int64_t base = (int64_t)tile * TILE;
+    const int tn = (int)min((int64_t)TILE, n - base);
+    u64 k[PER];
+    uint32_t v[PER];
+#pragma unroll
+    for (int j = 0; j < PER; j++) {
+        const int x = w * 32 * PER + j * 32 + lane;
+        // past the end: digit 255, behind every key of the cloud
+        k[j] = x < tn ? kin[base + x] : ~0ull;
+        v[j] = x < tn ? (vin ? vin[base + x] : (uint32_t)(base + x)) : 0u;
+    }
+    // slot of each key: its rank among the warp's keys of its digit for now
+    uint32_t slot[PER];
+#pragma unroll
+    for (int j = 0; j < PER; j++) {
+        const uint32_t d = (uint32_t)(k[j] >> shift) & 255;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const uint32_t before = wc[w][d];
+        __syncwarp();
+        if (lane == __ffs(peers) - 1) wc[w][d] = before + __popc(peers);
+        __syncwarp();
+        slot[j] = before + __popc(peers & ((1u << lane) - 1u));
+    }
+    __syncthreads();
+    // thread t: digit t
+    uint32_t cnt = 0;
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        const uint32_t c = wc[i][t];
+        wc[i][t] = cnt;
+        cnt += c;
+    }
+    uint32_t lo = cnt, gbase = ss->total[pass][t];
+    if (t == 255) cnt -= (uint32_t)(TILE - tn);
+    const uint32_t own = 2 * pass + 1, sum = own + 1;
+    volatile u64* mine = status + (int64_t)tile * 256 + t;
+    *mine = ((u64)(tile ? own : sum) << 32) | cnt;
+    scan256(lo, gbase, ws);
+    first[t] = lo;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < PER; j++) {
+        const uint32_t d = (uint32_t)(k[j] >> shift) & 255;
+        slot[j] += first[d] + wc[w][d];
+        sk[slot[j]] = k[j];
+    }
+    // the digit's keys in the tiles before: eight of their words at a time
+    uint32_t before = 0;
+    bool found = false;
+    for (int p = tile - 1; p >= 0 && !found; p -= 8) {
+        u64 s[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++)
+            s[i] = p - i >= 0 ? *(volatile u64*)(status + (int64_t)(p - i) * 256 + t) : 0;
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            if (p - i < 0 || found) continue;
+            u64 x = s[i];
+            for (int spin = 0; (uint32_t)(x >> 32) < own && spin < RS_SPIN; spin++)
+                x = *(volatile u64*)(status + (int64_t)(p - i) * 256 + t);
+            if ((uint32_t)(x >> 32) < own) {
+                uint32_t c = 0;
+                const int64_t b = (int64_t)(p - i) * TILE;  // a full tile: it is not the last
+                for (int y = 0; y < TILE; y++) c += ((uint32_t)(kin[b + y] >> shift) & 255) == t;
+                x = c;
+            }
+            before += (uint32_t)x;
+            found = (uint32_t)(x >> 32) == sum;
+        }
+    }
+    if (tile) *mine = ((u64)sum << 32) | (before + cnt);
+    to[t] = gbase + before - lo;
+    __syncthreads();
+    uint32_t at[PER];
+#pragma unroll
+    for (int j = 0; j < PER; j++) {
+        const int x = j * RS_T + t;
+        if (x < tn) {
+            const u64 q = sk[x];
+            at[j] = to[(uint32_t)(q >> shift) & 255] + (uint32_t)x;
+            kout[at[j]] = q;
+        }
+    }
+    __syncthreads();
+    uint32_t* sv = reinterpret_cast<uint32_t*>(sk);
+#pragma unroll
+    for (int j = 0; j < PER; j++) sv[slot[j]] = v[j];
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < PER; j++) {
+        const int x = j * RS_T + t;
+        if (x < tn) vout[at[j]] = sv[x];
+    }
+}
+
+cudaError_t sort_points(const int32_t* xyz, int64_t n, int3 origin, int shift, int bits, u64* keys,
+                        uint32_t* vals, const Scratch& s, cudaStream_t st) {
+    const int passes = (bits + 7) / 8;
+    if (n < 1 || passes < 1 || passes > RS_MAXP) return cudaErrorInvalidValue;
+    // half tiles below four full ones per SM: more of them in flight
+    const bool half = n < (int64_t)device_sms() * 4 * RS_T * 16;
+    const int tile = RS_T * (half ? 8 : 16);
+    const int64_t tiles = (n + tile - 1) / tile;
+    const size_t words = (size_t)tiles * 256;
+    u64* k2 = (u64*)s.get(n * sizeof(u64));
+    uint32_t* v2 = (uint32_t*)s.get(n * sizeof(uint32_t));
+    u64* status = (u64*)s.get(words * sizeof(u64) + sizeof(SortState));
+    cudaError_t e = cudaSuccess;
+    if (!k2 || !v2 || !status) e = cudaErrorMemoryAllocation;
+    SortState* ss = reinterpret_cast<SortState*>(status + words);
+    if (!e) e = cudaMemsetAsync(status, 0, words * sizeof(u64) + sizeof(SortState), st);
+    if (!e) {
+        // the last pass writes keys and vals
+        int64_t blocks = (n + 255) / 256;
+        const int64_t lim = (int64_t)device_sms() * 8;
+        if (blocks > lim) blocks = lim;
+        morton_kernel<<<(unsigned)blocks, 256, 0, st>>>(xyz, n, origin, shift,
+                                                       passes & 1 ? k2 : keys, passes, ss);
+        note_launch();
+        e = cudaGetLastError();
+    }
+    for (int p = 0; p < passes && !e; p++) {
+        const bool last = ((passes - p) & 1) != 0;  // this pass writes keys, the next one k2
+        const u64* ki = last ? k2 : keys;
+        const uint32_t* vi = p == 0 ? nullptr : last ? v2 : vals;
+        u64* ko = last ? keys : k2;
+        uint32_t* vo = last ? vals : v2;
+        if (half)
+            radix_pass_kernel<8><<<(unsigned)tiles, RS_T, 0, st>>>(ki, vi, ko, vo, n, p, ss, status);
+        else
+            radix_pass_kernel<16><<<(unsigned)tiles, RS_T, 0, st>>>(ki, vi, ko, vo, n, p, ss, status);
+        note_launch();
+        e = cudaGetLastError();
+    }
+    s.put(status);
+    s.put(v2);
+    s.put(k2);
+    return e;
 }
 
 // ------------------------------------------------------------------ scan
@@ -121,135 +354,6 @@ cudaError_t exclusive_scan_u32(uint32_t* data, int64_t len, const Scratch& s, cu
     if (!e) scan_add_kernel<<<(unsigned)nb, 256, 0, st>>>(data, len, sums); note_launch();
     s.put(sums);
     return e ? e : cudaGetLastError();
-}
-
-// ------------------------------------------------------------------ radix sort
-// Tiles of 2048 keys: 256 threads x 8 sub-tiles of 256 consecutive keys.
-#define RS_TILE 2048
-
-__global__ void radix_hist_kernel(const u64* __restrict__ keys, int64_t n, int shift,
-                                  uint32_t* counts, int nblk) {
-    __shared__ uint32_t h[256];
-    int t = threadIdx.x;
-    h[t] = 0;
-    __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * RS_TILE;
-    for (int j = 0; j < 8; j++) {
-        int64_t i = base + j * 256 + t;
-        if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255], 1u);
-    }
-    __syncthreads();
-    counts[(int64_t)t * nblk + blockIdx.x] = h[t];
-}
-
-// Scatter of one 8-bit digit.  The tile's keys are first placed in digit
-// order in shared memory (stable: sub-tile by sub-tile, warp by warp, lane by
-// lane), then written out in that order, so that consecutive threads write
-// consecutive addresses of one digit's run.  offs is the exclusive scan of the
-// digit-major [digit][tile] counts: the tile's own count of digit d is the gap
-// to the next entry (n at the very end).
-__global__ void radix_scatter_kernel(const u64* __restrict__ kin, const uint32_t* __restrict__ vin,
-                                     u64* __restrict__ kout, uint32_t* __restrict__ vout,
-                                     int64_t n, int shift, const uint32_t* __restrict__ offs,
-                                     int nblk) {
-    __shared__ u64 sk[RS_TILE];
-    __shared__ uint32_t sv[RS_TILE];
-    __shared__ uint32_t goff[256];
-    __shared__ uint32_t tpre[256];  // first slot of digit d in the tile's sorted order
-    __shared__ uint32_t run[256];
-    __shared__ uint32_t wsum[8];
-    __shared__ uint16_t wcnt[8][257];
-    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-    const int64_t gi = (int64_t)t * nblk + blockIdx.x;
-    const uint32_t go = offs[gi];
-    const uint32_t next = gi + 1 < (int64_t)256 * nblk ? offs[gi + 1] : (uint32_t)n;
-    goff[t] = go;
-    run[t] = 0;
-    // exclusive scan of the tile's per-digit counts over the 256 digits
-    {
-        const uint32_t c = next - go;
-        uint32_t x = c;
-        for (int o = 1; o < 32; o <<= 1) {
-            uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) wsum[w] = x;
-        __syncthreads();
-        uint32_t before = 0;
-        for (int ww = 0; ww < w; ww++) before += wsum[ww];
-        tpre[t] = before + x - c;
-    }
-    const int64_t base = (int64_t)blockIdx.x * RS_TILE;
-    for (int j = 0; j < RS_TILE / 256; j++) {
-        for (int x = t; x < 8 * 257; x += 256) (&wcnt[0][0])[x] = 0;
-        __syncthreads();
-        const int64_t i = base + j * 256 + t;
-        const bool valid = i < n;
-        const u64 k = valid ? kin[i] : 0ull;
-        const uint32_t v = valid ? vin[i] : 0u;
-        const int d = valid ? (int)((k >> shift) & 255) : 256;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        const int lrank = __popc(peers & ((1u << lane) - 1u));
-        if (lane == __ffs(peers) - 1) wcnt[w][d] = (uint16_t)__popc(peers);
-        __syncthreads();
-        {
-            uint32_t acc = run[t];
-            for (int ww = 0; ww < 8; ww++) {
-                uint32_t c = wcnt[ww][t];
-                wcnt[ww][t] = (uint16_t)acc;
-                acc += c;
-            }
-            run[t] = acc;
-        }
-        __syncthreads();
-        if (valid) {
-            const uint32_t lp = tpre[d] + wcnt[w][d] + (uint32_t)lrank;
-            sk[lp] = k;
-            sv[lp] = v;
-        }
-        __syncthreads();  // wcnt is cleared at the top of the next sub-tile
-    }
-    const int tn = (int)min((int64_t)RS_TILE, n - base);
-    for (int x = t; x < tn; x += 256) {
-        const u64 k = sk[x];
-        const int d = (int)((k >> shift) & 255);
-        const uint32_t p = goff[d] + ((uint32_t)x - tpre[d]);
-        kout[p] = k;
-        vout[p] = sv[x];
-    }
-}
-
-cudaError_t radix_sort_pairs(u64* keys, uint32_t* vals, int64_t n, int bits, const Scratch& s,
-                             cudaStream_t st) {
-    if (n <= 1) return cudaSuccess;
-    int nblk = (int)((n + RS_TILE - 1) / RS_TILE);
-    u64* k2 = (u64*)s.get(n * sizeof(u64));
-    uint32_t* v2 = (uint32_t*)s.get(n * sizeof(uint32_t));
-    uint32_t* counts = (uint32_t*)s.get((size_t)256 * nblk * sizeof(uint32_t));
-    cudaError_t e = cudaSuccess;
-    if (!k2 || !v2 || !counts) e = cudaErrorMemoryAllocation;
-    u64 *ka = keys, *kb = k2;
-    uint32_t *va = vals, *vb = v2;
-    int passes = (bits + 7) / 8;
-    for (int p = 0; p < passes && !e; p++) {
-        radix_hist_kernel<<<nblk, 256, 0, st>>>(ka, n, 8 * p, counts, nblk); note_launch();
-        e = cudaGetLastError();
-        if (!e) e = exclusive_scan_u32(counts, (int64_t)256 * nblk, s, st);
-        if (!e) {
-            radix_scatter_kernel<<<nblk, 256, 0, st>>>(ka, va, kb, vb, n, 8 * p, counts, nblk); note_launch();
-            e = cudaGetLastError();
-        }
-        u64* tk = ka; ka = kb; kb = tk;
-        uint32_t* tv = va; va = vb; vb = tv;
-    }
-    if (!e && ka != keys) {
-        e = cudaMemcpyAsync(keys, ka, n * sizeof(u64), cudaMemcpyDefault, st);
-        if (!e) e = cudaMemcpyAsync(vals, va, n * sizeof(uint32_t), cudaMemcpyDefault, st);
-    }
-    s.put(counts);
-    s.put(v2);
-    s.put(k2);
-    return e;
 }
 
 // ------------------------------------------------------------------ gather

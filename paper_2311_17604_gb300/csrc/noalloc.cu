@@ -133,8 +133,7 @@ extern "C" int pd_knn_cost_static(const int32_t* xyz_dev, int64_t n, int k, doub
     uint32_t* perm;
     SGET(code, u64, n);
     SGET(perm, uint32_t, n);
-    SCK(launch_morton(xyz_dev, n, g.origin, g.shift, code, perm, st));
-    SCK(radix_sort_pairs(code, perm, n, 3 * g.B, s, st));
+    SCK(sort_points(xyz_dev, n, g.origin, g.shift, 3 * g.B, code, perm, s, st));
     int4* pos;
     SGET(pos, int4, n);
     SCK(launch_gather(xyz_dev, nullptr, nullptr, perm, n, pos, nullptr, nullptr, st));

@@ -21,12 +21,10 @@ struct Scratch {
 
 // ---------------------------------------------------------------- grid.cu
 cudaError_t launch_bbox(const int32_t* xyz, int64_t n, int* out6, cudaStream_t st);
-cudaError_t launch_morton(const int32_t* xyz, int64_t n, int3 origin, int shift, u64* keys,
-                          uint32_t* vals, cudaStream_t st);
-// Stable LSD radix sort of (keys, vals) on bits [0, bits); results land in
-// keys/vals (ping-pong through tmp buffers).
-cudaError_t radix_sort_pairs(u64* keys, uint32_t* vals, int64_t n, int bits, const Scratch& s,
-                             cudaStream_t st);
+// Morton codes ((x - origin) >> shift, `bits` bits) in ascending order, equal ones
+// in input order, in keys; their input indices in vals.
+cudaError_t sort_points(const int32_t* xyz, int64_t n, int3 origin, int shift, int bits, u64* keys,
+                        uint32_t* vals, const Scratch& s, cudaStream_t st);
 cudaError_t exclusive_scan_u32(uint32_t* data, int64_t len, const Scratch& s, cudaStream_t st);
 cudaError_t launch_gather(const int32_t* xyz, const uint8_t* rgb, const float* nrm,
                           const uint32_t* perm, int64_t n, int4* pos, uchar4* rgb_s,
