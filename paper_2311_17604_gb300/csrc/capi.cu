@@ -1422,15 +1422,17 @@ static int wup_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* ke
     if (rc) return rc;
     const int k = cp->k, S = g->S;
     const int64_t cap = g->n;
-    uint8_t *wdirty, *pick;
-    u64* mark_p;
-    int* mark_i;
     int* rest;
     RALLOC(rest, int, cap);
-    RALLOC(wdirty, uint8_t, cap);
-    RALLOC(pick, uint8_t, cap);
-    RALLOC(mark_p, u64, cap);
-    RALLOC(mark_i, int, cap);
+    WupBuffers wb;
+    RALLOC(wb.cand, uint8_t, cap);
+    RALLOC(wb.beaten, uint8_t, cap);
+    RALLOC(wb.list[0], int, cap);
+    RALLOC(wb.list[1], int, cap);
+    RALLOC(wb.wd, WupDev, 1);
+    uint8_t* least;
+    RALLOC(least, uint8_t, wup_least_bytes());
+    wb.block_least = least;
     SelBuffers sb;
     RALLOC(sb.p, u64, cap);
     RALLOC(sb.i, int, cap);
@@ -1438,10 +1440,6 @@ static int wup_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* ke
     CK(cudaMemsetAsync(sb.hist, 0, 4096 * sizeof(uint32_t), g->st));
     RoundDev* rd;
     RALLOC(rd, RoundDev, 1);
-    u64* tmin;
-    int* imin;
-    RALLOC(tmin, u64, 1);
-    RALLOC(imin, int, 1);
     int64_t live = g->n, built = g->n;
     int iters = 0;
     while (live > m) {
@@ -1462,7 +1460,6 @@ static int wup_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* ke
             a.qflag = g->alive;
             CK(launch_knn(view_of(g), a, g->ng, rest, g->d_int + 7, g->st));
         }
-        CK(cudaMemsetAsync(wdirty, 0, g->ng, g->st));
         // 2. w_up: the (live - m)-th largest key is the smallest one above it
         RoundDev h;
         memset(&h, 0, sizeof(h));
@@ -1474,28 +1471,36 @@ static int wup_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* ke
             Span t(T, &g->stats.ms_select);
             CK(round_launch_select(g->prim, g->pos, g->alive, g->ng, sb,
                                    g->ng > ((int64_t)4 << 20), rd, g->st));
-            CK(wup_launch_exact_tau(g->prim, g->pos, g->alive, g->ng, rd, tmin, imin, g->st));
+            CK(wup_launch_list(bufview(g, &c2), g->alive, g->ng, rd, wb, g->st));
         }
-        // 3. removal rounds above w_up
-        for (int r = 0;; r++) {
-            CK(wup_launch_round(bufview(g, &c2), g->alive, wdirty, g->ng, S, k, rd, mark_p,
-                                mark_i, pick, g->st));
-            unsigned long long removed = 0;
-            CK(cudaMemcpyAsync(&removed, &rd->removed, sizeof(removed), cudaMemcpyDeviceToHost,
-                               g->st));
+        // 3. removal rounds above w_up, WUP_BATCH to a host read
+        int64_t most = live - m;
+        for (int r = 0, stop = 0; !stop;) {
+            CK(wup_launch_rounds(bufview(g, &c2), g->alive, most, S, k, rd, wb, g->st));
+            WupDev hw;
+            CK(cudaMemcpyAsync(&hw, wb.wd, sizeof(hw), cudaMemcpyDeviceToHost, g->st));
             CK(cudaStreamSynchronize(g->st));
-            g->stats.rounds++;
-            g->stats.live_rounds += live;
-            if ((int64_t)removed > live - m || (r == 0 && removed == 0)) {
-                set_err(g->ctx, "pd_decimate_wup: a round removed %s%lld points", "",
-                        (long long)removed);
-                return PD_EINTERNAL;
+            for (int j = 0; j < WUP_BATCH && !stop; j++, r++) {
+                const unsigned long long removed = hw.removed[j];
+                g->stats.rounds++;
+                g->stats.live_rounds += live;
+                if ((int64_t)removed > live - m || (r == 0 && removed == 0)) {
+                    set_err(g->ctx, "pd_decimate_wup: a round removed %s%lld points", "",
+                            (long long)removed);
+                    return PD_EINTERNAL;
+                }
+                live -= (int64_t)removed;
+                if (g->trace)
+                    fprintf(stderr, "pd wup iteration %d round %d removed %llu live %lld\n", iters,
+                            r, removed, (long long)live);
+                stop = removed == 0 || live <= m;
             }
-            live -= (int64_t)removed;
-            if (g->trace)
-                fprintf(stderr, "pd wup iteration %d round %d removed %llu live %lld\n", iters, r,
-                        removed, (long long)live);
-            if (removed == 0 || live <= m) break;
+            most = hw.count[0];
+            if (!stop && most == 0) {  // the round that would find nothing
+                g->stats.rounds++;
+                g->stats.live_rounds += live;
+                stop = 1;
+            }
         }
     }
     g->stats.iterations = iters;

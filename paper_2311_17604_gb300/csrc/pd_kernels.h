@@ -359,15 +359,24 @@ cudaError_t launch_mlp_init(float* prm, u64 seed, cudaStream_t st);
 cudaError_t launch_normal_fallback(const float* mlp, const float* onorm, const float* pca,
                                    int64_t n, float min_norm, float* out, cudaStream_t st);
 // ---------------------------------------------------------------- wup.cu
-// The paper's iterative w_up scheme: one removal round (marks, picks, removal,
-// stored-list update).  S <= 8, k <= S.
-// Replace the selection's bin boundary by the smallest live key at or above
-// it (the exact rank-th largest key).  tmin, imin: device scratch words.
-cudaError_t wup_launch_exact_tau(const u64* prim, const int4* pos, const uint8_t* alive,
-                                 int64_t n, RoundDev* rd, u64* tmin, int* imin, cudaStream_t st);
-cudaError_t wup_launch_round(const BufView& b, uint8_t* alive, uint8_t* wdirty, int64_t n, int S,
-                             int k, RoundDev* rd, u64* mark_p, int* mark_i, uint8_t* pick,
-                             cudaStream_t st);
+#define WUP_BATCH 4  // removal rounds between two host reads
+struct WupDev {
+    int count[2];     // candidates in either list
+    unsigned ticket;
+    unsigned long long removed[WUP_BATCH];
+};
+struct WupBuffers {
+    uint8_t *cand, *beaten;  // per point: a candidate; one of smaller key than an adjacent one
+    int* list[2];
+    WupDev* wd;
+    void* block_least;       // wup_least_bytes() of scratch
+};
+int64_t wup_blocks();
+size_t wup_least_bytes();
+cudaError_t wup_launch_list(const BufView& b, const uint8_t* alive, int64_t n, RoundDev* rd,
+                            const WupBuffers& w, cudaStream_t st);
+cudaError_t wup_launch_rounds(const BufView& b, uint8_t* alive, int64_t most, int S, int k,
+                              const RoundDev* rd, const WupBuffers& w, cudaStream_t st);
 
 // ---------------------------------------------------------------- batch.cu
 // One scan of a packed batch (device array, host-built): its caller-owned
