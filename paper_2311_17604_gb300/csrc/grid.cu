@@ -80,8 +80,9 @@ struct SortState {
 };
 
 __global__ void __launch_bounds__(256)
-    morton_kernel(const int32_t* __restrict__ xyz, int64_t n, int3 o, int shift,
-                  u64* __restrict__ keys, int passes, SortState* ss) {
+    morton_kernel(const int32_t* xyz, int64_t n, int3 o, int shift,
+                  u64* keys, int passes, SortState* ss) {
+    chain();
     __shared__ uint32_t h[RS_MAXP][256];
     const int lane = threadIdx.x & 31;
     for (int p = 0; p < passes; p++) h[p][threadIdx.x] = 0;
@@ -152,9 +153,10 @@ __device__ __forceinline__ void scan256(uint32_t& a, uint32_t& b, uint32_t (&ws)
 // tile's digit itself, so that no wait is without end.
 template <int PER>
 __global__ void __launch_bounds__(RS_T, 2)
-    radix_pass_kernel(const u64* __restrict__ kin, const uint32_t* __restrict__ vin,
-                      u64* __restrict__ kout, uint32_t* __restrict__ vout, int64_t n, int pass,
+    radix_pass_kernel(const u64* kin, const uint32_t* vin,
+                      u64* kout, uint32_t* vout, int64_t n, int pass,
                       SortState* ss, u64* status) {
+    chain();
     const int TILE = RS_T * PER;
     __shared__ u64 sk[RS_T * PER];     // the tile's keys, then its values
     __shared__ uint32_t wc[8][256];    // counts of a warp, then of the warps before it
@@ -286,7 +288,7 @@ cudaError_t sort_points(const int32_t* xyz, int64_t n, int3 origin, int shift, i
         int64_t blocks = (n + 255) / 256;
         const int64_t lim = (int64_t)device_sms() * 8;
         if (blocks > lim) blocks = lim;
-        morton_kernel<<<(unsigned)blocks, 256, 0, st>>>(xyz, n, origin, shift,
+        launch_chained(morton_kernel, (unsigned)blocks, 256, 0, st, xyz, n, origin, shift,
                                                        passes & 1 ? k2 : keys, passes, ss);
         note_launch();
         e = cudaGetLastError();
@@ -298,9 +300,11 @@ cudaError_t sort_points(const int32_t* xyz, int64_t n, int3 origin, int shift, i
         u64* ko = last ? keys : k2;
         uint32_t* vo = last ? vals : v2;
         if (half)
-            radix_pass_kernel<8><<<(unsigned)tiles, RS_T, 0, st>>>(ki, vi, ko, vo, n, p, ss, status);
+            launch_chained(radix_pass_kernel<8>, (unsigned)tiles, RS_T, 0, st, ki, vi, ko, vo, n,
+                           p, ss, status);
         else
-            radix_pass_kernel<16><<<(unsigned)tiles, RS_T, 0, st>>>(ki, vi, ko, vo, n, p, ss, status);
+            launch_chained(radix_pass_kernel<16>, (unsigned)tiles, RS_T, 0, st, ki, vi, ko, vo, n,
+                           p, ss, status);
         note_launch();
         e = cudaGetLastError();
     }
@@ -370,10 +374,11 @@ cudaError_t exclusive_scan_u32(uint32_t* data, int64_t len, const Scratch& s, cu
 }
 
 // ------------------------------------------------------------------ gather
-__global__ void gather_kernel(const int32_t* __restrict__ xyz, const uint8_t* __restrict__ rgb,
-                              const float* __restrict__ nrm, const uint32_t* __restrict__ perm,
-                              int64_t n, int4* __restrict__ pos, uchar4* __restrict__ rgb_s,
-                              float4* __restrict__ nrm_s) {
+__global__ void gather_kernel(const int32_t* xyz, const uint8_t* rgb,
+                              const float* nrm, const uint32_t* perm,
+                              int64_t n, int4* pos, uchar4* rgb_s,
+                              float4* nrm_s) {
+    chain();
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= n) return;
     uint32_t i = perm[s];
@@ -392,8 +397,9 @@ __global__ void gather_kernel(const int32_t* __restrict__ xyz, const uint8_t* __
 cudaError_t launch_gather(const int32_t* xyz, const uint8_t* rgb, const float* nrm,
                           const uint32_t* perm, int64_t n, int4* pos, uchar4* rgb_s,
                           float4* nrm_s, cudaStream_t st) {
-    gather_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-        xyz, rgb_s ? rgb : nullptr, nrm_s ? nrm : nullptr, perm, n, pos, rgb_s, nrm_s); note_launch();
+    launch_chained(gather_kernel, (unsigned)((n + 255) / 256), 256, 0, st, xyz,
+                   rgb_s ? rgb : nullptr, nrm_s ? nrm : nullptr, perm, n, pos, rgb_s, nrm_s);
+    note_launch();
     return cudaGetLastError();
 }
 
@@ -416,8 +422,9 @@ cudaError_t launch_gather_nrm(const float* nrm, const int4* pos, int64_t n, floa
 // consecutive Morton positions around s shares the level-L prefix.  With
 // Ls(j) = smallest level at which code[j] and code[j+T] share a cell, the
 // leaf level of s is min over j in [s-T, s] of Ls(j), minus one.
-__global__ void leaf_level_kernel(const u64* __restrict__ code, int64_t n, int T, int B,
-                                  uint8_t* __restrict__ leaf) {
+__global__ void leaf_level_kernel(const u64* code, int64_t n, int T, int B,
+                                  uint8_t* leaf) {
+    chain();
     extern __shared__ uint8_t ls[];
     int64_t b0 = (int64_t)blockIdx.x * 256;
     for (int x = threadIdx.x; x < 256 + T; x += 256) {
@@ -441,7 +448,9 @@ __global__ void leaf_level_kernel(const u64* __restrict__ code, int64_t n, int T
 
 cudaError_t launch_leaf_levels(const u64* code, int64_t n, int T, int B, uint8_t* leaf,
                                cudaStream_t st) {
-    leaf_level_kernel<<<(unsigned)((n + 255) / 256), 256, 256 + T, st>>>(code, n, T, B, leaf); note_launch();
+    launch_chained(leaf_level_kernel, (unsigned)((n + 255) / 256), 256, 256 + T, st, code, n, T,
+                   B, leaf);
+    note_launch();
     return cudaGetLastError();
 }
 
@@ -462,8 +471,9 @@ __device__ inline int tail_level(const u64* code, int64_t i, int64_t n, int B) {
 }
 
 // Octree nodes: one per (level L >= the point's leaf level, run head).
-__global__ void node_count_kernel(const u64* __restrict__ code, const uint8_t* __restrict__ leaf,
+__global__ void node_count_kernel(const u64* code, const uint8_t* leaf,
                                   int64_t n, int B, unsigned long long* count) {
+    chain();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     unsigned c = 0;
     if (i < n) {
@@ -478,7 +488,9 @@ cudaError_t launch_node_count(const u64* code, const uint8_t* leaf, int64_t n, i
                               unsigned long long* count, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(count, 0, sizeof(unsigned long long), st);
     if (e) return e;
-    node_count_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(code, leaf, n, B, count); note_launch();
+    launch_chained(node_count_kernel, (unsigned)((n + 255) / 256), 256, 0, st, code, leaf, n, B,
+                   count);
+    note_launch();
     return cudaGetLastError();
 }
 
@@ -492,8 +504,9 @@ __device__ inline long long hash_insert(HashSlot* tab, u64 mask, u64 key) {
     return -1;
 }
 
-__global__ void node_insert_kernel(const u64* __restrict__ code, const uint8_t* __restrict__ leaf,
+__global__ void node_insert_kernel(const u64* code, const uint8_t* leaf,
                                    int64_t n, int B, HashSlot* tab, u64 mask) {
+    chain();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int hh = head_level(code, i, B), ht = tail_level(code, i, n, B);
@@ -513,7 +526,9 @@ cudaError_t launch_node_insert(const u64* code, const uint8_t* leaf, int64_t n, 
                                HashSlot* tab, u64 mask, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(tab, 0, (mask + 1) * sizeof(HashSlot), st);
     if (e) return e;
-    node_insert_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(code, leaf, n, B, tab, mask); note_launch();
+    launch_chained(node_insert_kernel, (unsigned)((n + 255) / 256), 256, 0, st, code, leaf, n, B,
+                   tab, mask);
+    note_launch();
     return cudaGetLastError();
 }
 
@@ -529,6 +544,7 @@ __device__ inline bool leaf_range(const GridView& g, int64_t s, uint32_t& b, uin
 // (leaves above 32 points only occur at level 0) and s - b is a multiple of
 // 32, b the leaf's first position (from the cell table).
 __global__ void leaf_groups_kernel(GridView g, int64_t n, int4* groups, int* ngroups) {
+    chain();
     const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     bool start = false;
     int cnt = 0, L = 0;
@@ -554,7 +570,9 @@ cudaError_t launch_leaf_groups(const GridView& g, int64_t n, int4* groups, int* 
                                cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(ngroups, 0, sizeof(int), st);
     if (e) return e;
-    leaf_groups_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(g, n, groups, ngroups); note_launch();
+    launch_chained(leaf_groups_kernel, (unsigned)((n + 255) / 256), 256, 0, st, g, n, groups,
+                   ngroups);
+    note_launch();
     return cudaGetLastError();
 }
 

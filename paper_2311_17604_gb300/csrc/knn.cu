@@ -411,6 +411,7 @@ __device__ __forceinline__ int near_group(const GridView& g, const KnnArgs& a, i
 template <int S, bool W>
 __global__ void __launch_bounds__(NEAR_WARPS * 32, S == 8 ? 4 : 2)
     knn_kernel(GridView g, KnnArgs a, int* rest, int* nrest) {
+    chain();
     __shared__ NearSmem s_m[NEAR_WARPS];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gid = blockIdx.x * NEAR_WARPS + w;
@@ -927,6 +928,7 @@ __device__ __forceinline__ void warp_query(const GridView& g, const KnnArgs& a, 
 template <bool FILTERED, bool W, bool ORDER>
 __global__ void __launch_bounds__(PD_WARPS * 32, ORDER ? 8 : 10)
     knn_query_kernel(GridView g, KnnArgs a) {
+    chain();
     __shared__ WarpRanges s_r[PD_WARPS];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (!FILTERED && a.finish && blockIdx.x == 0 && threadIdx.x == 0) round_finish(a.finish);
@@ -940,8 +942,9 @@ __global__ void __launch_bounds__(PD_WARPS * 32, ORDER ? 8 : 10)
 }
 
 // Every point (every flagged one) to the list.
-__global__ void list_queries_kernel(const uint8_t* __restrict__ qflag, int64_t n, int* rest,
+__global__ void list_queries_kernel(const uint8_t* qflag, int64_t n, int* rest,
                                     int* nrest) {
+    chain();
     const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const bool in = s < n && (!qflag || qflag[s]);
     const int slot = block_append(in, nrest);
@@ -953,14 +956,14 @@ cudaError_t launch_knn_queries(const GridView& g, const KnnArgs& a, int64_t cap,
     const bool filtered = a.qlist2 != nullptr;
     const dim3 gr(list_blocks(cap, 128, 10)), bl(PD_WARPS * 32);
     if (filtered) {
-        if (a.term != 0) knn_query_kernel<true, true, true><<<gr, bl, 0, st>>>(g, a);
-        else knn_query_kernel<true, false, false><<<gr, bl, 0, st>>>(g, a);
+        if (a.term != 0) launch_chained(knn_query_kernel<true, true, true>, gr, bl, 0, st, g, a);
+        else launch_chained(knn_query_kernel<true, false, false>, gr, bl, 0, st, g, a);
     } else if (a.term != 0) {
-        knn_query_kernel<false, true, true><<<gr, bl, 0, st>>>(g, a);
+        launch_chained(knn_query_kernel<false, true, true>, gr, bl, 0, st, g, a);
     } else if (a.ordered) {
-        knn_query_kernel<false, false, true><<<gr, bl, 0, st>>>(g, a);
+        launch_chained(knn_query_kernel<false, false, true>, gr, bl, 0, st, g, a);
     } else {
-        knn_query_kernel<false, false, false><<<gr, bl, 0, st>>>(g, a);
+        launch_chained(knn_query_kernel<false, false, false>, gr, bl, 0, st, g, a);
     }
     note_launch();
     return cudaGetLastError();
@@ -977,13 +980,14 @@ cudaError_t launch_knn(const GridView& g, const KnnArgs& a, int64_t n, int* rest
     // entry too, which the list's 16 and their successor do not settle
     const bool all_rest = a.S == 17 && a.term != 0 && a.term != PD_TERM_INDEX_TIE;
     if (a.S == 8) {
-        if (a.term != 0) knn_kernel<8, true><<<gr, bl, 0, st>>>(g, a, rest, nrest);
-        else knn_kernel<8, false><<<gr, bl, 0, st>>>(g, a, rest, nrest);
+        if (a.term != 0) launch_chained(knn_kernel<8, true>, gr, bl, 0, st, g, a, rest, nrest);
+        else launch_chained(knn_kernel<8, false>, gr, bl, 0, st, g, a, rest, nrest);
     } else if (a.S == 17 && !all_rest) {
-        if (a.term != 0) knn_kernel<17, true><<<gr, bl, 0, st>>>(g, a, rest, nrest);
-        else knn_kernel<17, false><<<gr, bl, 0, st>>>(g, a, rest, nrest);
+        if (a.term != 0) launch_chained(knn_kernel<17, true>, gr, bl, 0, st, g, a, rest, nrest);
+        else launch_chained(knn_kernel<17, false>, gr, bl, 0, st, g, a, rest, nrest);
     } else if (a.S == 17) {
-        list_queries_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a.qflag, n, rest, nrest);
+        launch_chained(list_queries_kernel, (unsigned)((n + 255) / 256), 256, 0, st, a.qflag, n,
+                       rest, nrest);
     } else {
         return cudaErrorInvalidValue;
     }

@@ -113,8 +113,9 @@ __device__ __forceinline__ uint32_t ratio_bf16(int v, float inv, double rms) {
 // moment sums are exact int64, so the covariance scaled by m^2 is the exact
 // integer m * sum(u v) - sum(u) sum(v) before its conversion to binary64.
 __global__ void __launch_bounds__(128)
-    features_kernel(const int4* __restrict__ pos, const int* __restrict__ nbr, int S, int64_t n,
-                    uint4* __restrict__ feat, float* __restrict__ pca, uint8_t* valid) {
+    features_kernel(const int4* pos, const int* nbr, int S, int64_t n,
+                    uint4* feat, float* pca, uint8_t* valid) {
+    chain();
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= n) return;
     int4 p = pos[s];
@@ -935,7 +936,8 @@ cudaError_t launch_iota(int* out, int64_t n, cudaStream_t st) {
 cudaError_t launch_features(const int4* pos, const int* nbr, int S, int64_t n, uint16_t* feat,
                             float* pca, uint8_t* valid, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    features_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(pos, nbr, S, n, (uint4*)feat,
+    launch_chained(features_kernel, (unsigned)((n + 127) / 128), 128, 0, st, pos, nbr, S, n,
+                   (uint4*)feat,
                                                                 pca, valid);
     note_launch();
     return cudaGetLastError();

@@ -233,6 +233,39 @@ __device__ __forceinline__ int keep_live8(const uint8_t* __restrict__ alive, int
 extern long long g_launch_count;
 inline void note_launch() { __atomic_fetch_add(&g_launch_count, 1, __ATOMIC_RELAXED); }
 
+// Programmatic dependent launch: a chained launch may be set up while the kernel
+// ahead of it in the stream still runs, and its blocks take the places that the
+// last blocks of that kernel leave free.  Every kernel launched this way begins
+// with chain(): the launch after it may start, then it waits until the kernel
+// ahead has completed (that one waited for its own predecessor, so all before it
+// have).  Nothing comes before the wait; the kernels' pointers are not
+// __restrict__, which would let the compiler take their loads for constants and
+// move them there.  A small or ordinary call is tens to hundreds of short launches:
+// static pass of 7.4k points 237 -> 213 us, decimation of 200k points, k = 1, 2.65 ->
+// 2.52 ms, w_up of 700k points 9.5 -> 7.8 ms.  The long kernels of the k >= 2 rounds
+// (buffer update, candidate test, danger test, pair fixpoint) are launched plainly:
+// blocks that wait take places from those that work (9.8M outdoor points, k = 4, 133
+// ms, 140 with all of them chained; a packed batch of 3.8M 130 and 135).
+__device__ __forceinline__ void chain() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                  cudaStream_t st, A... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 // Block-level aggregation of counters and list appends: one global atomic
 // per block instead of one per warp (atomics on one address serialise in L2,
 // and a full-grid kernel over a billion points has 31M warps).  Every thread

@@ -537,9 +537,10 @@ __global__ void keep_kernel(const int4* __restrict__ pos, const uint8_t* __restr
 }
 
 // cost / neighbour output in input order (pd_knn_cost)
-__global__ void knn_out_kernel(const int4* __restrict__ pos, const double* __restrict__ cost_s,
-                               const int* __restrict__ nbr, int64_t n, int S, int k,
+__global__ void knn_out_kernel(const int4* pos, const double* cost_s,
+                               const int* nbr, int64_t n, int S, int k,
                                double* cost, int32_t* knn) {
+    chain();
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= n) return;
     int i = pos[s].w;
@@ -664,7 +665,8 @@ cudaError_t launch_keep(const int4* pos, const uint8_t* alive, int64_t n, uint8_
 }
 cudaError_t launch_knn_out(const int4* pos, const double* cost_s, const int* nbr, int64_t n, int S,
                            int k, double* cost, int32_t* knn, cudaStream_t st) {
-    knn_out_kernel<<<GRID1(n), 0, st>>>(pos, cost_s, nbr, n, S, k, cost, knn); note_launch();
+    launch_chained(knn_out_kernel, GRID1(n), 0, st, pos, cost_s, nbr, n, S, k, cost, knn);
+    note_launch();
     return cudaGetLastError();
 }
 cudaError_t launch_newpos(const int* list, int64_t nl, int* newpos, cudaStream_t st) {

@@ -25,11 +25,12 @@ __device__ __forceinline__ void list_append(bool want, int s, int* count, int* l
 }
 
 // ------------------------------------------------------------------ k = 1
-__global__ void k1d_cand_kernel(const u64* __restrict__ prim, const int4* __restrict__ pos,
-                                const uint8_t* __restrict__ alive, const int* __restrict__ nbr,
-                                const int* __restrict__ nbr0,
-                                const uint8_t* __restrict__ flg, int64_t n, int S, RoundDev* rd,
+__global__ void k1d_cand_kernel(const u64* prim, const int4* pos,
+                                const uint8_t* alive, const int* nbr,
+                                const int* nbr0,
+                                const uint8_t* flg, int64_t n, int S, RoundDev* rd,
                                 uint8_t* inP, int* cand, int* slow, int* dep) {
+    chain();
     const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     bool c = false, sl = false, dp = false;
     const bool in = s < n;
@@ -77,10 +78,11 @@ __global__ void k1d_cand_kernel(const u64* __restrict__ prim, const int4* __rest
 
 // overflowing shells: accept iff every live point at distance d1 has a
 // smaller key (grid-stride over the slow list)
-__global__ void k1d_slow_kernel(GridView g, const u64* __restrict__ prim,
-                                const uint8_t* __restrict__ alive, const u64* __restrict__ rk2,
-                                const int* __restrict__ slow, RoundDev* rd, uint8_t* inP,
+__global__ void k1d_slow_kernel(GridView g, const u64* prim,
+                                const uint8_t* alive, const u64* rk2,
+                                const int* slow, RoundDev* rd, uint8_t* inP,
                                 int* cand) {
+    chain();
     int ns = rd->nslow;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ns; t += gridDim.x * blockDim.x) {
         int s = slow[t];
@@ -150,10 +152,11 @@ __device__ __forceinline__ void fix_sweeps(RoundDev* rd, int iter, Sweep sweep) 
     if (any) rd->changed[iter] = 1;
 }
 
-__global__ void k1d_fix_kernel(const int* __restrict__ cand, const int4* __restrict__ pos,
-                               const int* __restrict__ nbr, const uint8_t* __restrict__ flg, int S,
-                               const uint8_t* __restrict__ inP, uint8_t* rej, int iter,
+__global__ void k1d_fix_kernel(const int* cand, const int4* pos,
+                               const int* nbr, const uint8_t* flg, int S,
+                               const uint8_t* inP, uint8_t* rej, int iter,
                                RoundDev* rd) {
+    chain();
     const volatile uint8_t* vrej = rej;
     const int nc = rd->ndep;  // cand: the dep list (only its members can be rejected)
     fix_sweeps(rd, iter, [&]() {
@@ -199,8 +202,9 @@ __global__ void pairs_fix_kernel(const int2* __restrict__ pairs, int pair_cap,
 // Removes the accepted candidates unless the round must be settled on the
 // host (danger overflow, or a fixpoint that did not converge in the fixed
 // number of sweeps); candidate marks are cleared in the normal case.
-__global__ void removed_kernel(const int* __restrict__ cand, uint8_t* inP, uint8_t* rej,
+__global__ void removed_kernel(const int* cand, uint8_t* inP, uint8_t* rej,
                                uint8_t* alive, RoundDev* rd) {
+    chain();
     __shared__ int hold;
     if (threadIdx.x == 0) {
         int fi = rd->fix_iters;
@@ -226,8 +230,9 @@ __global__ void removed_kernel(const int* __restrict__ cand, uint8_t* inP, uint8
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(&rd->removed, (unsigned long long)c);
 }
 
-__global__ void dirtyd_kernel(const uint8_t* __restrict__ alive, const int* __restrict__ nbr,
+__global__ void dirtyd_kernel(const uint8_t* alive, const int* nbr,
                               int64_t n, int S, int kchk, int* list, RoundDev* rd) {
+    chain();
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     bool d = false;
     if (s < n && alive[s]) {
@@ -252,8 +257,9 @@ __global__ void dirtyd_kernel(const uint8_t* __restrict__ alive, const int* __re
 // and more threads in flight measured faster (rules of the 100M-point scan
 // 52.9 -> 51.5 ms)
 __global__ void __launch_bounds__(256, 6)
-    k1d_update_kernel(BufView b, const uint8_t* __restrict__ alive, int64_t n, int* list,
+    k1d_update_kernel(BufView b, const uint8_t* alive, int64_t n, int* list,
                       RoundDev* rd) {
+    chain();
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     bool req = false;
     if (s < n) {
@@ -649,11 +655,16 @@ cudaError_t round_launch_k1(const GridView& g, const u64* prim, const uint8_t* a
                             int64_t n, int S, RoundDev* rd, uint8_t* inP, uint8_t* rej, int* cand,
                             int* slow, int* dep, int fix_iters, cudaStream_t st) {
     if (fix_iters < 1 || fix_iters > PD_FIX_ITERS) return cudaErrorInvalidValue;
-    k1d_cand_kernel<<<GRID1(n), 0, st>>>(prim, g.pos, alive, nbr, nbr0, flg, n, S, rd, inP, cand,
+    launch_chained(k1d_cand_kernel, GRID1(n), 0, st, prim, g.pos, alive, nbr, nbr0, flg, n, S, rd,
+                   inP, cand,
                                          slow, dep); note_launch();
-    k1d_slow_kernel<<<list_blocks(n, 4096, 4), 128, 0, st>>>(g, prim, alive, rk2, slow, rd, inP, cand); note_launch();
+    launch_chained(k1d_slow_kernel, list_blocks(n, 4096, 4), 128, 0, st, g, prim, alive, rk2,
+                   slow, rd, inP, cand);
+    note_launch();
     for (int it = 0; it < fix_iters; it++) {
-        k1d_fix_kernel<<<list_blocks(n, 2048, 8), 256, 0, st>>>(dep, g.pos, nbr, flg, S, inP, rej, it, rd); note_launch();
+        launch_chained(k1d_fix_kernel, list_blocks(n, 2048, 8), 256, 0, st, dep, g.pos, nbr, flg,
+                       S, inP, rej, it, rd);
+        note_launch();
     }
     return cudaGetLastError();
 }
@@ -661,20 +672,22 @@ cudaError_t round_launch_k1(const GridView& g, const u64* prim, const uint8_t* a
 cudaError_t round_launch_pairs_fix(const int2* pairs, int pair_cap, const uint8_t* inP,
                                    uint8_t* rej, int64_t n, RoundDev* rd, cudaStream_t st) {
     for (int it = 0; it < PD_FIX_ITERS_KK; it++) {
-        pairs_fix_kernel<<<list_blocks(n, 4096, 8), 256, 0, st>>>(pairs, pair_cap, inP, rej, it, rd); note_launch();
+        pairs_fix_kernel<<<list_blocks(n, 4096, 8), 256, 0, st>>>(pairs, pair_cap, inP, rej, it, rd);
+        note_launch();
     }
     return cudaGetLastError();
 }
 
 cudaError_t round_launch_remove(const int* cand, uint8_t* inP, uint8_t* rej, uint8_t* alive,
                                 int64_t n, RoundDev* rd, cudaStream_t st) {
-    removed_kernel<<<list_blocks(n, 4096, 8), 256, 0, st>>>(cand, inP, rej, alive, rd); note_launch();
+    launch_chained(removed_kernel, list_blocks(n, 4096, 8), 256, 0, st, cand, inP, rej, alive, rd);
+    note_launch();
     return cudaGetLastError();
 }
 
 cudaError_t round_launch_dirty(const uint8_t* alive, const int* nbr, int64_t n, int S, int kchk,
                                int* list, RoundDev* rd, cudaStream_t st) {
-    dirtyd_kernel<<<GRID1(n), 0, st>>>(alive, nbr, n, S, kchk, list, rd); note_launch();
+    launch_chained(dirtyd_kernel, GRID1(n), 0, st, alive, nbr, n, S, kchk, list, rd); note_launch();
     return cudaGetLastError();
 }
 
@@ -684,7 +697,7 @@ namespace pd {
 cudaError_t round_launch_k1_update(const BufView& b, const uint8_t* alive, int64_t n, int S,
                                    int* list, RoundDev* rd, cudaStream_t st) {
     if (S != 8) return cudaErrorInvalidValue;
-    k1d_update_kernel<<<GRID1(n), 0, st>>>(b, alive, n, list, rd); note_launch();
+    launch_chained(k1d_update_kernel, GRID1(n), 0, st, b, alive, n, list, rd); note_launch();
     return cudaGetLastError();
 }
 cudaError_t round_launch_kk_update(const BufView& b, const uint8_t* alive, int64_t n, int S, int k,

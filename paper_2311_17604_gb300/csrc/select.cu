@@ -191,8 +191,9 @@ __device__ __forceinline__ void sel_count(const u64* __restrict__ prim,
 // One full pass.  hist: 4096 words per cloud or scan, zero on entry and exit.
 template <int PASS, bool SEG>
 __global__ void __launch_bounds__(SEL_T)
-    sel_pass_kernel(const u64* __restrict__ prim, const uint8_t* __restrict__ alive, int64_t n,
-                    uint32_t* hist, RoundDev* rd, SegDev* seg, const int* __restrict__ items) {
+    sel_pass_kernel(const u64* prim, const uint8_t* alive, int64_t n,
+                    uint32_t* hist, RoundDev* rd, SegDev* seg, const int* items) {
+    chain();
     __shared__ uint32_t h[4096];
     if (PASS == 0 && blockIdx.x == 0 && threadIdx.x == 0) {  // the round's counters
         rd->ncand = rd->nslow = rd->nsrc = rd->npairs = rd->ndep = 0;
@@ -288,9 +289,10 @@ __global__ void __launch_bounds__(SEL_T)
 // Lists the live keys that agree with both leading digits.
 template <bool SEG>
 __global__ void __launch_bounds__(SEL_T)
-    sel_list_kernel(const u64* __restrict__ prim, const int4* __restrict__ pos,
-                    const uint8_t* __restrict__ alive, int64_t n, u64* lp, int* li, RoundDev* rd,
-                    SegDev* seg, const int* __restrict__ items) {
+    sel_list_kernel(const u64* prim, const int4* pos,
+                    const uint8_t* alive, int64_t n, u64* lp, int* li, RoundDev* rd,
+                    SegDev* seg, const int* items) {
+    chain();
     __shared__ int s_w[SEL_T / 32], s_at;
     const int nitems = SEG ? rd->seg_chunk0[rd->nseg] : (int)gridDim.x;
     for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
@@ -363,8 +365,9 @@ __global__ void __launch_bounds__(SEL_T)
 // A remaining digit over a long list (many equal keys, as a voxelised cloud
 // has): the whole grid counts, the last block finds.
 __global__ void __launch_bounds__(SEL_T)
-    sel_digit_kernel(const u64* __restrict__ lp, const int* __restrict__ li, int pass,
+    sel_digit_kernel(const u64* lp, const int* li, int pass,
                      uint32_t* hist, RoundDev* rd) {
+    chain();
     __shared__ uint32_t h[4096];
     if (rd->done) return;
     for (int x = threadIdx.x; x < 4096; x += SEL_T) h[x] = 0;
@@ -406,8 +409,9 @@ __global__ void __launch_bounds__(SEL_T)
 
 template <bool SEG>
 __global__ void __launch_bounds__(SEL_T)
-    sel_rest_kernel(const u64* __restrict__ lp, const int* __restrict__ li, RoundDev* rd,
+    sel_rest_kernel(const u64* lp, const int* li, RoundDev* rd,
                     SegDev* seg) {
+    chain();
     __shared__ uint32_t h[4096];
     __shared__ u64 sp[SEL_SMEM];
     __shared__ int si[SEL_SMEM];
@@ -524,13 +528,15 @@ static cudaError_t launch_rest(const u64* lp, const int* li, RoundDev* rd, SegDe
     c.gridDim = dim3((unsigned)(nseg * nb));
     c.blockDim = dim3(SEL_T);
     c.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)nb;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     c.attrs = at;
-    c.numAttrs = 1;
+    c.numAttrs = 2;
     note_launch();
     return cudaLaunchKernelEx(&c, sel_rest_kernel<SEG>, lp, li, rd, seg);
 }
@@ -542,14 +548,17 @@ cudaError_t round_launch_select(const u64* prim, const int4* pos, const uint8_t*
     if (blocks > lim) blocks = lim;
     if (blocks < 1) blocks = 1;
     const unsigned g = (unsigned)blocks;
-    sel_pass_kernel<0, false><<<g, SEL_T, 0, st>>>(prim, alive, n, b.hist, rd, nullptr, nullptr);
-    sel_pass_kernel<1, false><<<g, SEL_T, 0, st>>>(prim, alive, n, b.hist, rd, nullptr, nullptr);
-    sel_list_kernel<false><<<g, SEL_T, 0, st>>>(prim, pos, alive, n, b.p, b.i, rd, nullptr,
+    launch_chained(sel_pass_kernel<0, false>, g, SEL_T, 0, st, prim, alive, n, b.hist, rd,
+                   nullptr, nullptr);
+    launch_chained(sel_pass_kernel<1, false>, g, SEL_T, 0, st, prim, alive, n, b.hist, rd,
+                   nullptr, nullptr);
+    launch_chained(sel_list_kernel<false>, g, SEL_T, 0, st, prim, pos, alive, n, b.p, b.i, rd,
+                   nullptr,
                                                nullptr);
     for (int i = 0; i < 3; i++) note_launch();
     if (long_list) {
         for (int pass = 2; pass < 8; pass++) {
-            sel_digit_kernel<<<g, SEL_T, 0, st>>>(b.p, b.i, pass, b.hist, rd);
+            launch_chained(sel_digit_kernel, g, SEL_T, 0, st, b.p, b.i, pass, b.hist, rd);
             note_launch();
         }
         return cudaGetLastError();
@@ -568,9 +577,12 @@ cudaError_t seg_launch_select(const u64* prim, const int4* pos, const uint8_t* a
     const int64_t lim = (int64_t)device_sms() * 8;
     if (blocks > lim) blocks = lim;
     const unsigned g = (unsigned)blocks;
-    sel_pass_kernel<0, true><<<g, SEL_T, 0, st>>>(prim, alive, ng, hist, rd, seg, items);
-    sel_pass_kernel<1, true><<<g, SEL_T, 0, st>>>(prim, alive, ng, hist, rd, seg, items);
-    sel_list_kernel<true><<<g, SEL_T, 0, st>>>(prim, pos, alive, ng, b.p, b.i, rd, seg, items);
+    launch_chained(sel_pass_kernel<0, true>, g, SEL_T, 0, st, prim, alive, ng, hist, rd, seg,
+                   items);
+    launch_chained(sel_pass_kernel<1, true>, g, SEL_T, 0, st, prim, alive, ng, hist, rd, seg,
+                   items);
+    launch_chained(sel_list_kernel<true>, g, SEL_T, 0, st, prim, pos, alive, ng, b.p, b.i, rd,
+                   seg, items);
     for (int i = 0; i < 3; i++) note_launch();
     const cudaError_t e = cudaGetLastError();
     return e ? e : launch_rest<true>(b.p, b.i, rd, seg, nseg, st);

@@ -28,7 +28,7 @@
 // read; now three launches over the list, four rounds a host read (wasted ones
 // find an empty list).  What bounds a round is its three launches.
 // 700k room points, k = 6, to 20 % (15 iterations, 224 rounds): 18.3 -> 9.5 ms, of which
-// the rounds 14.1 -> 6.2.
+// the rounds 14.1 -> 6.2 (7.8 ms with chained launches).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -70,9 +70,10 @@ __device__ __forceinline__ WupKey wup_block_least(WupKey k) {
 }
 
 __global__ void __launch_bounds__(256)
-    wup_list_kernel(const u64* __restrict__ prim, const int4* __restrict__ pos,
-                    const uint8_t* __restrict__ alive, int64_t n, RoundDev* rd, uint8_t* cand,
+    wup_list_kernel(const u64* prim, const int4* pos,
+                    const uint8_t* alive, int64_t n, RoundDev* rd, uint8_t* cand,
                     uint8_t* beaten, int* list, WupDev* wd, WupKey* block_least) {
+    chain();
     const u64 tp = rd->tau_prim;
     const int ti = rd->tau_idx;
     WupKey least = {~0ull, 0x7fffffff};
@@ -115,8 +116,9 @@ __global__ void __launch_bounds__(256)
 }
 
 __global__ void __launch_bounds__(256)
-    wup_beat_kernel(const BufView b, const uint8_t* __restrict__ cand, const int* __restrict__ list,
+    wup_beat_kernel(const BufView b, const uint8_t* cand, const int* list,
                     int in, int slot, int k, WupDev* wd, uint8_t* beaten) {
+    chain();
     if (blockIdx.x == 0 && threadIdx.x == 0) {  // for the launches of this round
         wd->count[in ^ 1] = 0;
         wd->removed[slot] = 0;
@@ -145,8 +147,9 @@ __global__ void __launch_bounds__(256)
 }
 
 __global__ void __launch_bounds__(256)
-    wup_pick_kernel(const int* __restrict__ list, int in, int slot, WupDev* wd, uint8_t* cand,
+    wup_pick_kernel(const int* list, int in, int slot, WupDev* wd, uint8_t* cand,
                     uint8_t* beaten, uint8_t* alive) {
+    chain();
     const int n = wd->count[in];
     unsigned long long c = 0;
     for (int t = blockIdx.x * 256 + threadIdx.x; t < n; t += gridDim.x * 256) {
@@ -165,8 +168,9 @@ __global__ void __launch_bounds__(256)
 // Removed points leave the stored lists (order kept); the cost is the sum of
 // 1 / d^2 over the first k stored points left, nearest first, in binary64.
 __global__ void __launch_bounds__(256)
-    wup_update_kernel(BufView b, const uint8_t* __restrict__ alive, const int* __restrict__ list,
+    wup_update_kernel(BufView b, const uint8_t* alive, const int* list,
                       int* next, int in, int k, const RoundDev* rd, uint8_t* cand, WupDev* wd) {
+    chain();
     const int n = wd->count[in];
     const u64 tp = rd->tau_prim;
     const int ti = rd->tau_idx;
@@ -218,7 +222,8 @@ cudaError_t wup_launch_list(const BufView& b, const uint8_t* alive, int64_t n, R
     if (e) return e;
     int64_t blocks = (n + 255) / 256;
     if (blocks > wup_blocks()) blocks = wup_blocks();
-    wup_list_kernel<<<(unsigned)blocks, 256, 0, st>>>(b.prim, b.pos, alive, n, rd, w.cand, w.beaten,
+    launch_chained(wup_list_kernel, (unsigned)blocks, 256, 0, st, b.prim, b.pos, alive, n, rd,
+                   w.cand, w.beaten,
                                                      w.list[0], w.wd, (WupKey*)w.block_least);
     note_launch();
     return cudaGetLastError();
@@ -237,9 +242,12 @@ cudaError_t wup_launch_rounds(const BufView& b, uint8_t* alive, int64_t most, in
     const unsigned g = list_blocks(most, 256, 8);
     for (int j = 0; j < WUP_BATCH; j++) {
         const int in = j & 1;
-        wup_beat_kernel<<<g, 256, 0, st>>>(b, w.cand, w.list[in], in, j, k, w.wd, w.beaten);
-        wup_pick_kernel<<<g, 256, 0, st>>>(w.list[in], in, j, w.wd, w.cand, w.beaten, alive);
-        wup_update_kernel<<<g, 256, 0, st>>>(b, alive, w.list[in], w.list[in ^ 1], in, k, rd,
+        launch_chained(wup_beat_kernel, g, 256, 0, st, b, w.cand, w.list[in], in, j, k, w.wd,
+                       w.beaten);
+        launch_chained(wup_pick_kernel, g, 256, 0, st, w.list[in], in, j, w.wd, w.cand, w.beaten,
+                       alive);
+        launch_chained(wup_update_kernel, g, 256, 0, st, b, alive, w.list[in], w.list[in ^ 1], in,
+                       k, rd,
                                              w.cand, w.wd);
         for (int i = 0; i < 3; i++) note_launch();
     }
