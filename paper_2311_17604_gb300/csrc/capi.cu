@@ -851,13 +851,14 @@ BufView bufview(pd_grid* g, const pd_cost_params* cp) {
 }
 
 // Full searches of list[0 .. rd->nreq): the points whose stored neighbours no
-// longer settle their cost.
-int knn_requery(pd_grid* g, const pd_cost_params* cp, const int* list, RoundDev* rd) {
+// longer settle their cost.  take: a counter that the round has opened, or NULL.
+int knn_requery(pd_grid* g, const pd_cost_params* cp, const int* list, RoundDev* rd, int* take) {
     KnnArgs a = base_args(g, cp);
     if (g->density_k1 && g->k1_exact_rq > 0) a.r_exact = g->k1_exact_rq;
     a.finish = rd;
     a.qlist = list;
     a.qcount = &rd->nreq;
+    a.take = take;
     CK(launch_knn_queries(view_of(g), a, g->ng, g->st));
     return PD_OK;
 }
@@ -1205,6 +1206,7 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
                     a.qcount = &rd->nfq;
                     a.qlist2 = lq;
                     a.qcount2 = &rd->nlq;
+                    a.take = &rd->take_filt;
                     a.lam_out = lam;
                     a.inP = inP;
                     a.inPb = inPb;
@@ -1234,7 +1236,7 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
             if (g->trace) cudaEventRecord(tq0, g->st);
             {
                 Span t(T, &g->stats.ms_knn_requery);
-                rc = knn_requery(g, cp, rq, rd);
+                rc = knn_requery(g, cp, rq, rd, &rd->take_req);
                 if (rc) return rc;
             }
             if (g->trace) cudaEventRecord(tq1, g->st);
@@ -1319,7 +1321,7 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
                 CK(round_launch_dirty(g->alive, g->nbr, g->ng, S, kchk, rq, rd, g->st));
             {
                 Span t(T, &g->stats.ms_knn_requery);
-                rc = knn_requery(g, cp, rq, rd);
+                rc = knn_requery(g, cp, rq, rd, nullptr);
                 if (rc) return rc;
             }
             h.live -= removed;

@@ -340,6 +340,13 @@ __device__ __forceinline__ void block_append_n(const bool (&want)[N], int* const
         slot[i] = s_w[i][32] + s_w[i][w] + __popc(m[i] & ((1u << lane) - 1u));
 }
 
+// The next item of a list that the warps of a launch share; every lane calls it.
+__device__ __forceinline__ int warp_take(int* next, int lane) {
+    int t = 0;
+    if (lane == 0) t = atomicAdd(next, 1);
+    return __shfl_sync(0xffffffffu, t, 0);
+}
+
 // Streaming multiprocessors of the current device (queried once per device
 // and cached); persistent and grid-stride launches size their grids from it.
 int device_sms();

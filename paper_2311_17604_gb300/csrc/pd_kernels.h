@@ -99,6 +99,7 @@ struct RoundDev {
     int finished;              // the round's counts are added up
     int ncand, nslow, nsrc, npairs, overflow;
     int nreq, nfq, nlq;  // this round's re-searches, filtered and lambda searches
+    int take_src, take_filt, take_req;  // next item of those lists, past each warp's first
     int ndep;  // k = 1: candidates with a shell member of larger input index
     int changed[PD_FIX_ITERS];
     int fix_unconverged;
@@ -179,6 +180,7 @@ struct KnnArgs {
     RoundDev* finish;         // full searches: the round to add up
     int ordered;              // equal distances in Morton order (term 0; with a term they are
                               //   always in input order)
+    int* take;                // optional, zero: a short list's queries are taken one by one
     const int* qlist;
     const int* qcount;
     const int* qlist2;

@@ -198,6 +198,7 @@ __global__ void __launch_bounds__(SEL_T)
     if (PASS == 0 && blockIdx.x == 0 && threadIdx.x == 0) {  // the round's counters
         rd->ncand = rd->nslow = rd->nsrc = rd->npairs = rd->ndep = 0;
         rd->nreq = rd->nfq = rd->nlq = 0;
+        rd->take_src = rd->take_filt = rd->take_req = 0;
         rd->overflow = 0;
         rd->removed = 0;
         rd->cap_over = 0;
