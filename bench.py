@@ -210,11 +210,11 @@ def knn_bytes(k):
 ROUND_BYTES_PER_LIVE = 16
 ALU_OPS_PER_PAIR = 9   # 3 subtractions, 3 multiply-adds, compare, select, loop: exact int distance test
 
-# DRAM bytes per query of the first full kNN pass (knn_kernel<8,0,0,0>), from an
+# DRAM bytes per query of the first full kNN pass (knn_kernel<8,0>), from an
 # ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of a one-station
 # site scan at the leaf capacity below; reported only while the kNN sources
 # hash to src_sha and the timed run uses the same leaf capacity and k.
-KNN_TRAFFIC = {"k": 1, "leaf_max": 32, "bytes_per_query": 113.9, "src_sha": "d96e267f93cc3f0e"}
+KNN_TRAFFIC = {"k": 1, "leaf_max": 32, "bytes_per_query": 114.6, "src_sha": "2295f1f2784fbbe6"}
 KNN_SOURCES = ["paper_2311_17604_gb300/csrc/knn.cu", "paper_2311_17604_gb300/csrc/pd_internal.cuh",
                "paper_2311_17604_gb300/csrc/pd_kernels.h"]
 
@@ -272,7 +272,7 @@ def rooflines(stats, n, k, leaf, passes, step_ms, clk, device):
               "knn_requery": msr, "select": mean("ms_select"),
               "rules_other": mean("ms_rules") - mean("ms_select"),
               "total": mean("ms_total")}
-    return {"bound": "hbm", "kernel": "knn_kernel<8,0,0,0>: the first full kNN/cost pass (one "
+    return {"bound": "hbm", "kernel": "knn_kernel<8,0>: the first full kNN/cost pass (one "
                                       "launch per step)",
             "achieved": first_ach, "peak": peak, "unit": "GB/s", "frac": first_ach / peak,
             "hbm_frac": first_ach / peak, "peak_kind": kind, "traffic": traffic1,
