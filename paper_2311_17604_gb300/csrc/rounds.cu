@@ -540,9 +540,8 @@ __global__ void keep_kernel(const int4* __restrict__ pos, const uint8_t* __restr
 }
 
 // cost / neighbour output in input order (pd_knn_cost)
-__global__ void knn_out_kernel(const int4* pos, const double* cost_s,
-                               const int* nbr, int64_t n, int S, int k,
-                               double* cost, int32_t* knn) {
+__global__ void knn_out_kernel(const int4* pos, const double* cost_s, const int* nbr, int64_t n,
+                               int S, int k, double* cost, int32_t* knn) {
     chain();
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= n) return;

@@ -2,10 +2,10 @@
 //
 // One round is a fixed sequence of launches whose sizes never depend on
 // counts computed in the round: the threshold tau comes from an on-device
-// radix select, candidate / source / pair lists are appended with atomics and
-// walked by grid-stride or persistent kernels, neighbour searches run over
-// the leaf groups with a per-point flag, and the fixpoint runs a fixed number
-// of sweeps.  The host reads the small RoundDev block once per round.
+// radix select (select.cu), candidate / source / pair / query lists are appended
+// with atomics and walked by grid-stride or persistent kernels, and the fixpoint
+// runs a fixed number of launches.  The host reads the small RoundDev block once
+// per round.
 // The rules themselves (R2, A, B) are documented in rounds.cu.
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -25,11 +25,9 @@ __device__ __forceinline__ void list_append(bool want, int s, int* count, int* l
 }
 
 // ------------------------------------------------------------------ k = 1
-__global__ void k1d_cand_kernel(const u64* prim, const int4* pos,
-                                const uint8_t* alive, const int* nbr,
-                                const int* nbr0,
-                                const uint8_t* flg, int64_t n, int S, RoundDev* rd,
-                                uint8_t* inP, int* cand, int* slow, int* dep) {
+__global__ void k1d_cand_kernel(const u64* prim, const int4* pos, const uint8_t* alive,
+                                const int* nbr, const int* nbr0, const uint8_t* flg, int64_t n,
+                                int S, RoundDev* rd, uint8_t* inP, int* cand, int* slow, int* dep) {
     chain();
     const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     bool c = false, sl = false, dp = false;
@@ -78,10 +76,8 @@ __global__ void k1d_cand_kernel(const u64* prim, const int4* pos,
 
 // overflowing shells: accept iff every live point at distance d1 has a
 // smaller key (grid-stride over the slow list)
-__global__ void k1d_slow_kernel(GridView g, const u64* prim,
-                                const uint8_t* alive, const u64* rk2,
-                                const int* slow, RoundDev* rd, uint8_t* inP,
-                                int* cand) {
+__global__ void k1d_slow_kernel(GridView g, const u64* prim, const uint8_t* alive, const u64* rk2,
+                                const int* slow, RoundDev* rd, uint8_t* inP, int* cand) {
     chain();
     int ns = rd->nslow;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ns; t += gridDim.x * blockDim.x) {
@@ -152,10 +148,9 @@ __device__ __forceinline__ void fix_sweeps(RoundDev* rd, int iter, Sweep sweep) 
     if (any) rd->changed[iter] = 1;
 }
 
-__global__ void k1d_fix_kernel(const int* cand, const int4* pos,
-                               const int* nbr, const uint8_t* flg, int S,
-                               const uint8_t* inP, uint8_t* rej, int iter,
-                               RoundDev* rd) {
+__global__ void k1d_fix_kernel(const int* cand, const int4* pos, const int* nbr,
+                               const uint8_t* flg, int S, const uint8_t* inP, uint8_t* rej,
+                               int iter, RoundDev* rd) {
     chain();
     const volatile uint8_t* vrej = rej;
     const int nc = rd->ndep;  // cand: the dep list (only its members can be rejected)
@@ -202,8 +197,8 @@ __global__ void pairs_fix_kernel(const int2* __restrict__ pairs, int pair_cap,
 // Removes the accepted candidates unless the round must be settled on the
 // host (danger overflow, or a fixpoint that did not converge in the fixed
 // number of sweeps); candidate marks are cleared in the normal case.
-__global__ void removed_kernel(const int* cand, uint8_t* inP, uint8_t* rej,
-                               uint8_t* alive, RoundDev* rd) {
+__global__ void removed_kernel(const int* cand, uint8_t* inP, uint8_t* rej, uint8_t* alive,
+                               RoundDev* rd) {
     chain();
     __shared__ int hold;
     if (threadIdx.x == 0) {
@@ -230,8 +225,8 @@ __global__ void removed_kernel(const int* cand, uint8_t* inP, uint8_t* rej,
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(&rd->removed, (unsigned long long)c);
 }
 
-__global__ void dirtyd_kernel(const uint8_t* alive, const int* nbr,
-                              int64_t n, int S, int kchk, int* list, RoundDev* rd) {
+__global__ void dirtyd_kernel(const uint8_t* alive, const int* nbr, int64_t n, int S, int kchk,
+                              int* list, RoundDev* rd) {
     chain();
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     bool d = false;
@@ -257,8 +252,7 @@ __global__ void dirtyd_kernel(const uint8_t* alive, const int* nbr,
 // and more threads in flight measured faster (rules of the 100M-point scan
 // 52.9 -> 51.5 ms)
 __global__ void __launch_bounds__(256, 6)
-    k1d_update_kernel(BufView b, const uint8_t* alive, int64_t n, int* list,
-                      RoundDev* rd) {
+    k1d_update_kernel(BufView b, const uint8_t* alive, int64_t n, int* list, RoundDev* rd) {
     chain();
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     bool req = false;
@@ -656,8 +650,8 @@ cudaError_t round_launch_k1(const GridView& g, const u64* prim, const uint8_t* a
                             int* slow, int* dep, int fix_iters, cudaStream_t st) {
     if (fix_iters < 1 || fix_iters > PD_FIX_ITERS) return cudaErrorInvalidValue;
     launch_chained(k1d_cand_kernel, GRID1(n), 0, st, prim, g.pos, alive, nbr, nbr0, flg, n, S, rd,
-                   inP, cand,
-                                         slow, dep); note_launch();
+                   inP, cand, slow, dep);
+    note_launch();
     launch_chained(k1d_slow_kernel, list_blocks(n, 4096, 4), 128, 0, st, g, prim, alive, rk2,
                    slow, rd, inP, cand);
     note_launch();
@@ -687,7 +681,8 @@ cudaError_t round_launch_remove(const int* cand, uint8_t* inP, uint8_t* rej, uin
 
 cudaError_t round_launch_dirty(const uint8_t* alive, const int* nbr, int64_t n, int S, int kchk,
                                int* list, RoundDev* rd, cudaStream_t st) {
-    launch_chained(dirtyd_kernel, GRID1(n), 0, st, alive, nbr, n, S, kchk, list, rd); note_launch();
+    launch_chained(dirtyd_kernel, GRID1(n), 0, st, alive, nbr, n, S, kchk, list, rd);
+    note_launch();
     return cudaGetLastError();
 }
 
@@ -697,7 +692,8 @@ namespace pd {
 cudaError_t round_launch_k1_update(const BufView& b, const uint8_t* alive, int64_t n, int S,
                                    int* list, RoundDev* rd, cudaStream_t st) {
     if (S != 8) return cudaErrorInvalidValue;
-    launch_chained(k1d_update_kernel, GRID1(n), 0, st, b, alive, n, list, rd); note_launch();
+    launch_chained(k1d_update_kernel, GRID1(n), 0, st, b, alive, n, list, rd);
+    note_launch();
     return cudaGetLastError();
 }
 cudaError_t round_launch_kk_update(const BufView& b, const uint8_t* alive, int64_t n, int S, int k,

@@ -191,8 +191,8 @@ __device__ __forceinline__ void sel_count(const u64* __restrict__ prim,
 // One full pass.  hist: 4096 words per cloud or scan, zero on entry and exit.
 template <int PASS, bool SEG>
 __global__ void __launch_bounds__(SEL_T)
-    sel_pass_kernel(const u64* prim, const uint8_t* alive, int64_t n,
-                    uint32_t* hist, RoundDev* rd, SegDev* seg, const int* items) {
+    sel_pass_kernel(const u64* prim, const uint8_t* alive, int64_t n, uint32_t* hist,
+                    RoundDev* rd, SegDev* seg, const int* items) {
     chain();
     __shared__ uint32_t h[4096];
     if (PASS == 0 && blockIdx.x == 0 && threadIdx.x == 0) {  // the round's counters
@@ -290,9 +290,8 @@ __global__ void __launch_bounds__(SEL_T)
 // Lists the live keys that agree with both leading digits.
 template <bool SEG>
 __global__ void __launch_bounds__(SEL_T)
-    sel_list_kernel(const u64* prim, const int4* pos,
-                    const uint8_t* alive, int64_t n, u64* lp, int* li, RoundDev* rd,
-                    SegDev* seg, const int* items) {
+    sel_list_kernel(const u64* prim, const int4* pos, const uint8_t* alive, int64_t n, u64* lp,
+                    int* li, RoundDev* rd, SegDev* seg, const int* items) {
     chain();
     __shared__ int s_w[SEL_T / 32], s_at;
     const int nitems = SEG ? rd->seg_chunk0[rd->nseg] : (int)gridDim.x;
@@ -366,8 +365,7 @@ __global__ void __launch_bounds__(SEL_T)
 // A remaining digit over a long list (many equal keys, as a voxelised cloud
 // has): the whole grid counts, the last block finds.
 __global__ void __launch_bounds__(SEL_T)
-    sel_digit_kernel(const u64* lp, const int* li, int pass,
-                     uint32_t* hist, RoundDev* rd) {
+    sel_digit_kernel(const u64* lp, const int* li, int pass, uint32_t* hist, RoundDev* rd) {
     chain();
     __shared__ uint32_t h[4096];
     if (rd->done) return;
@@ -410,8 +408,7 @@ __global__ void __launch_bounds__(SEL_T)
 
 template <bool SEG>
 __global__ void __launch_bounds__(SEL_T)
-    sel_rest_kernel(const u64* lp, const int* li, RoundDev* rd,
-                    SegDev* seg) {
+    sel_rest_kernel(const u64* lp, const int* li, RoundDev* rd, SegDev* seg) {
     chain();
     __shared__ uint32_t h[4096];
     __shared__ u64 sp[SEL_SMEM];
@@ -554,8 +551,7 @@ cudaError_t round_launch_select(const u64* prim, const int4* pos, const uint8_t*
     launch_chained(sel_pass_kernel<1, false>, g, SEL_T, 0, st, prim, alive, n, b.hist, rd,
                    nullptr, nullptr);
     launch_chained(sel_list_kernel<false>, g, SEL_T, 0, st, prim, pos, alive, n, b.p, b.i, rd,
-                   nullptr,
-                                               nullptr);
+                   nullptr, nullptr);
     for (int i = 0; i < 3; i++) note_launch();
     if (long_list) {
         for (int pass = 2; pass < 8; pass++) {

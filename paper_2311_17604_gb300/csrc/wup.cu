@@ -70,9 +70,9 @@ __device__ __forceinline__ WupKey wup_block_least(WupKey k) {
 }
 
 __global__ void __launch_bounds__(256)
-    wup_list_kernel(const u64* prim, const int4* pos,
-                    const uint8_t* alive, int64_t n, RoundDev* rd, uint8_t* cand,
-                    uint8_t* beaten, int* list, WupDev* wd, WupKey* block_least) {
+    wup_list_kernel(const u64* prim, const int4* pos, const uint8_t* alive, int64_t n,
+                    RoundDev* rd, uint8_t* cand, uint8_t* beaten, int* list, WupDev* wd,
+                    WupKey* block_least) {
     chain();
     const u64 tp = rd->tau_prim;
     const int ti = rd->tau_idx;
@@ -116,8 +116,8 @@ __global__ void __launch_bounds__(256)
 }
 
 __global__ void __launch_bounds__(256)
-    wup_beat_kernel(const BufView b, const uint8_t* cand, const int* list,
-                    int in, int slot, int k, WupDev* wd, uint8_t* beaten) {
+    wup_beat_kernel(const BufView b, const uint8_t* cand, const int* list, int in, int slot,
+                    int k, WupDev* wd, uint8_t* beaten) {
     chain();
     if (blockIdx.x == 0 && threadIdx.x == 0) {  // for the launches of this round
         wd->count[in ^ 1] = 0;
@@ -147,8 +147,8 @@ __global__ void __launch_bounds__(256)
 }
 
 __global__ void __launch_bounds__(256)
-    wup_pick_kernel(const int* list, int in, int slot, WupDev* wd, uint8_t* cand,
-                    uint8_t* beaten, uint8_t* alive) {
+    wup_pick_kernel(const int* list, int in, int slot, WupDev* wd, uint8_t* cand, uint8_t* beaten,
+                    uint8_t* alive) {
     chain();
     const int n = wd->count[in];
     unsigned long long c = 0;
@@ -168,8 +168,8 @@ __global__ void __launch_bounds__(256)
 // Removed points leave the stored lists (order kept); the cost is the sum of
 // 1 / d^2 over the first k stored points left, nearest first, in binary64.
 __global__ void __launch_bounds__(256)
-    wup_update_kernel(BufView b, const uint8_t* alive, const int* list,
-                      int* next, int in, int k, const RoundDev* rd, uint8_t* cand, WupDev* wd) {
+    wup_update_kernel(BufView b, const uint8_t* alive, const int* list, int* next, int in, int k,
+                      const RoundDev* rd, uint8_t* cand, WupDev* wd) {
     chain();
     const int n = wd->count[in];
     const u64 tp = rd->tau_prim;
@@ -223,8 +223,7 @@ cudaError_t wup_launch_list(const BufView& b, const uint8_t* alive, int64_t n, R
     int64_t blocks = (n + 255) / 256;
     if (blocks > wup_blocks()) blocks = wup_blocks();
     launch_chained(wup_list_kernel, (unsigned)blocks, 256, 0, st, b.prim, b.pos, alive, n, rd,
-                   w.cand, w.beaten,
-                                                     w.list[0], w.wd, (WupKey*)w.block_least);
+                   w.cand, w.beaten, w.list[0], w.wd, (WupKey*)w.block_least);
     note_launch();
     return cudaGetLastError();
 }
@@ -247,8 +246,7 @@ cudaError_t wup_launch_rounds(const BufView& b, uint8_t* alive, int64_t most, in
         launch_chained(wup_pick_kernel, g, 256, 0, st, w.list[in], in, j, w.wd, w.cand, w.beaten,
                        alive);
         launch_chained(wup_update_kernel, g, 256, 0, st, b, alive, w.list[in], w.list[in ^ 1], in,
-                       k, rd,
-                                             w.cand, w.wd);
+                       k, rd, w.cand, w.wd);
         for (int i = 0; i < 3; i++) note_launch();
     }
     return cudaGetLastError();
