@@ -80,8 +80,8 @@ struct SortState {
 };
 
 __global__ void __launch_bounds__(256)
-    morton_kernel(const int32_t* xyz, int64_t n, int3 o, int shift,
-                  u64* keys, int passes, SortState* ss) {
+    morton_kernel(const int32_t* xyz, int64_t n, int3 o, int shift, u64* keys, int passes,
+                  SortState* ss) {
     chain();
     __shared__ uint32_t h[RS_MAXP][256];
     const int lane = threadIdx.x & 31;
@@ -153,9 +153,8 @@ __device__ __forceinline__ void scan256(uint32_t& a, uint32_t& b, uint32_t (&ws)
 // tile's digit itself, so that no wait is without end.
 template <int PER>
 __global__ void __launch_bounds__(RS_T, 2)
-    radix_pass_kernel(const u64* kin, const uint32_t* vin,
-                      u64* kout, uint32_t* vout, int64_t n, int pass,
-                      SortState* ss, u64* status) {
+    radix_pass_kernel(const u64* kin, const uint32_t* vin, u64* kout, uint32_t* vout, int64_t n,
+                      int pass, SortState* ss, u64* status) {
     chain();
     const int TILE = RS_T * PER;
     __shared__ u64 sk[RS_T * PER];     // the tile's keys, then its values
@@ -278,18 +277,20 @@ cudaError_t sort_points(const int32_t* xyz, int64_t n, int3 origin, int shift, i
     const size_t words = (size_t)tiles * 256;
     u64* k2 = (u64*)s.get(n * sizeof(u64));
     uint32_t* v2 = (uint32_t*)s.get(n * sizeof(uint32_t));
-    u64* status = (u64*)s.get(words * sizeof(u64) + sizeof(SortState));
+    u64* status = (u64*)s.get(words * sizeof(u64));
+    // apart: a small block stays in device memory, where its atomics belong
+    SortState* ss = (SortState*)s.get(sizeof(SortState));
     cudaError_t e = cudaSuccess;
-    if (!k2 || !v2 || !status) e = cudaErrorMemoryAllocation;
-    SortState* ss = reinterpret_cast<SortState*>(status + words);
-    if (!e) e = cudaMemsetAsync(status, 0, words * sizeof(u64) + sizeof(SortState), st);
+    if (!k2 || !v2 || !status || !ss) e = cudaErrorMemoryAllocation;
+    if (!e) e = cudaMemsetAsync(status, 0, words * sizeof(u64), st);
+    if (!e) e = cudaMemsetAsync(ss, 0, sizeof(SortState), st);
     if (!e) {
         // the last pass writes keys and vals
         int64_t blocks = (n + 255) / 256;
         const int64_t lim = (int64_t)device_sms() * 8;
         if (blocks > lim) blocks = lim;
         launch_chained(morton_kernel, (unsigned)blocks, 256, 0, st, xyz, n, origin, shift,
-                                                       passes & 1 ? k2 : keys, passes, ss);
+                       passes & 1 ? k2 : keys, passes, ss);
         note_launch();
         e = cudaGetLastError();
     }
@@ -308,6 +309,7 @@ cudaError_t sort_points(const int32_t* xyz, int64_t n, int3 origin, int shift, i
         note_launch();
         e = cudaGetLastError();
     }
+    s.put(ss);
     s.put(status);
     s.put(v2);
     s.put(k2);
@@ -374,9 +376,8 @@ cudaError_t exclusive_scan_u32(uint32_t* data, int64_t len, const Scratch& s, cu
 }
 
 // ------------------------------------------------------------------ gather
-__global__ void gather_kernel(const int32_t* xyz, const uint8_t* rgb,
-                              const float* nrm, const uint32_t* perm,
-                              int64_t n, int4* pos, uchar4* rgb_s,
+__global__ void gather_kernel(const int32_t* xyz, const uint8_t* rgb, const float* nrm,
+                              const uint32_t* perm, int64_t n, int4* pos, uchar4* rgb_s,
                               float4* nrm_s) {
     chain();
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -422,8 +423,7 @@ cudaError_t launch_gather_nrm(const float* nrm, const int4* pos, int64_t n, floa
 // consecutive Morton positions around s shares the level-L prefix.  With
 // Ls(j) = smallest level at which code[j] and code[j+T] share a cell, the
 // leaf level of s is min over j in [s-T, s] of Ls(j), minus one.
-__global__ void leaf_level_kernel(const u64* code, int64_t n, int T, int B,
-                                  uint8_t* leaf) {
+__global__ void leaf_level_kernel(const u64* code, int64_t n, int T, int B, uint8_t* leaf) {
     chain();
     extern __shared__ uint8_t ls[];
     int64_t b0 = (int64_t)blockIdx.x * 256;
@@ -471,8 +471,8 @@ __device__ inline int tail_level(const u64* code, int64_t i, int64_t n, int B) {
 }
 
 // Octree nodes: one per (level L >= the point's leaf level, run head).
-__global__ void node_count_kernel(const u64* code, const uint8_t* leaf,
-                                  int64_t n, int B, unsigned long long* count) {
+__global__ void node_count_kernel(const u64* code, const uint8_t* leaf, int64_t n, int B,
+                                  unsigned long long* count) {
     chain();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     unsigned c = 0;
@@ -504,8 +504,8 @@ __device__ inline long long hash_insert(HashSlot* tab, u64 mask, u64 key) {
     return -1;
 }
 
-__global__ void node_insert_kernel(const u64* code, const uint8_t* leaf,
-                                   int64_t n, int B, HashSlot* tab, u64 mask) {
+__global__ void node_insert_kernel(const u64* code, const uint8_t* leaf, int64_t n, int B,
+                                   HashSlot* tab, u64 mask) {
     chain();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
