@@ -113,8 +113,8 @@ __device__ __forceinline__ uint32_t ratio_bf16(int v, float inv, double rms) {
 // moment sums are exact int64, so the covariance scaled by m^2 is the exact
 // integer m * sum(u v) - sum(u) sum(v) before its conversion to binary64.
 __global__ void __launch_bounds__(128)
-    features_kernel(const int4* pos, const int* nbr, int S, int64_t n,
-                    uint4* feat, float* pca, uint8_t* valid) {
+    features_kernel(const int4* pos, const int* nbr, int S, int64_t n, uint4* feat, float* pca,
+                    uint8_t* valid) {
     chain();
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= n) return;
@@ -251,8 +251,11 @@ __device__ __forceinline__ void load_weights(__nv_bfloat16* dst, int ld, const f
 }
 
 
-#define MLP_WARPS 8
-#define MLP_BLOCKS_PER_SM 2
+// 4 warps and 46 KB a block: within what a launch takes without an attribute call
+// on the host (a call of 1500 rows: 16.2 us with the host side, 17.8 with 16-row tiles
+// and 8 warps, 3 to 5 more with the attribute call)
+#define MLP_WARPS 4
+#define MLP_BLOCKS_PER_SM 4
 #define MT 2                  // 16-row tiles of a warp's step: they share the weight fragments
 #define MLP_ROWS (16 * MT)
 
@@ -303,13 +306,13 @@ __device__ __forceinline__ void mlp_layer(float (&c)[MT][8][4], const uint32_t (
 // memory once per block; the next rows arrive by 16-byte asynchronous copies
 // while these are computed.  Outputs per row: unit normal and |o|.
 // Bound: mma.sync itself, about 512 multiply-adds per clock and SM here (one or two
-// tiles a step, 8 to 32 warps per SM all measure 192 us or more for 4.0M rows).
+// tiles a step, 8 to 32 warps per SM all measure 192 us or more for 4.0M rows; blocks
+// of 4 warps 201).
 // Fragments and features by 4-byte loads, as before, took 231 us.
 __global__ void __launch_bounds__(MLP_WARPS * 32, MLP_BLOCKS_PER_SM)
     mlp_forward_kernel(const float* __restrict__ prm, const uint16_t* __restrict__ feat,
                        int64_t n, float* outn, float* onorm, bool vec_prm, bool vec_feat) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    MlpSmem& sm = *reinterpret_cast<MlpSmem*>(smraw);
+    __shared__ __align__(16) MlpSmem sm;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const int lr = lane & 7, lm = lane >> 3;
     const int64_t nsteps = (n + MLP_ROWS - 1) / MLP_ROWS;
@@ -937,38 +940,27 @@ cudaError_t launch_features(const int4* pos, const int* nbr, int S, int64_t n, u
                             float* pca, uint8_t* valid, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     launch_chained(features_kernel, (unsigned)((n + 127) / 128), 128, 0, st, pos, nbr, S, n,
-                   (uint4*)feat,
-                                                                pca, valid);
+                   (uint4*)feat, pca, valid);
     note_launch();
     return cudaGetLastError();
-}
-
-static int sm_count() {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > 0 ? sms : 1;
 }
 
 cudaError_t launch_mlp_forward(const float* prm, const uint16_t* feat, int64_t n, float* outn,
                                float* onorm, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    static_assert(sizeof(MlpSmem) <= 227 * 1024 / MLP_BLOCKS_PER_SM - 1024, "shared memory");
-    cudaError_t e = cudaFuncSetAttribute(
-        mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MlpSmem));
-    if (e) return e;
+    static_assert(sizeof(MlpSmem) <= 48 * 1024, "shared memory");
     int64_t steps = (n + MLP_ROWS - 1) / MLP_ROWS;
     int64_t blocks = (steps + MLP_WARPS - 1) / MLP_WARPS;
-    int64_t cap = (int64_t)sm_count() * MLP_BLOCKS_PER_SM;
+    int64_t cap = (int64_t)device_sms() * MLP_BLOCKS_PER_SM;
     if (blocks > cap) blocks = cap;
     // wider loads where the caller's arrays are aligned for them
-    mlp_forward_kernel<<<(unsigned)blocks, MLP_WARPS * 32, sizeof(MlpSmem), st>>>(
+    mlp_forward_kernel<<<(unsigned)blocks, MLP_WARPS * 32, 0, st>>>(
         prm, feat, n, outn, onorm, ((uintptr_t)prm & 15) == 0, ((uintptr_t)feat & 15) == 0);
     note_launch();
     return cudaGetLastError();
 }
 
-static int64_t bt_blocks() { return (int64_t)sm_count() * BT_BLOCKS_PER_SM; }
+static int64_t bt_blocks() { return (int64_t)device_sms() * BT_BLOCKS_PER_SM; }
 
 int64_t mlp_backward_part_floats() { return bt_blocks() * (N_PARAMS + 1); }
 
