@@ -501,7 +501,8 @@ struct WarpList {
     static const int SORT_AT = 12;
     WarpKey<PACK> best, last, cap;  // last: the least of cap and the S-th key
     int bpid;
-    // cap_d, cap_t: no key above this one is wanted (cap_d ~0: no cap)
+    // cap_d, cap_t: no key above this one is wanted (cap_d ~0: no cap); cap_t is
+    // below 0xffffffff
     __device__ __forceinline__ void init(u64 cap_d, uint32_t cap_t) {
         best = WarpKey<PACK>::none();
         cap = best;
@@ -599,7 +600,8 @@ struct WarpList32 {
     __device__ __forceinline__ u64 dist() const { return best == ~0u ? ~0ull : best; }
     __device__ __forceinline__ bool has() const { return best != ~0u; }
     __device__ __forceinline__ int id() const { return bid; }
-    __device__ __forceinline__ uint32_t tie() const { return 0; }
+    // as a later level's cap: every key at this distance is wanted
+    __device__ __forceinline__ uint32_t tie() const { return 0xfffffffeu; }
     __device__ __forceinline__ void merge(int o_, int lane) {
         const uint32_t o = __shfl_xor_sync(FULLM, best, o_);
         const int oi = __shfl_xor_sync(FULLM, bid, o_);
