@@ -72,10 +72,17 @@ __device__ inline double nbr_weight(const KnnArgs& a, int q, int j) {
 // 1.0M room points, k = 6, 2.20 -> 0.49; 2.0M, 17 stored, 9.19 -> 3.61 (4 to 6 blocks
 // per SM, batches of 8 keys and 512 candidates all within 3 %: the arithmetic is
 // the bound).
-// What one level in 32 bits cannot settle goes to a list that the
-// warp-per-query kernel finishes: the S-th distance beyond the cube's faces,
-// more than NEAR_MAX candidates, cells too wide for the key, equal distances at
-// the end of a list whose order they decide (W).
+// Where the largest distance does not fit beside a candidate's number (cells of a
+// metre and more: sparse clouds, far returns), the keys hold its leading bits: 24 of
+// them with 8 bits of number, so two distances share a key about once in 10^5, and
+// the exact ones order such a run.  Left to the warp-per-query kernel, those groups
+// made the pass of a cloud with 1 m between its points slower than the chain had
+// (1.0M points, grid and pass: k = 6 1.91 ms with the chain, 3.99 a warp each, 1.06
+// now; k = 1 1.61, 3.54, 0.95; 17 stored 5.53, 5.06, 1.96).
+// What one level cannot settle goes to a list that the warp-per-query kernel
+// finishes: the S-th distance beyond the cube's faces, more than NEAR_MAX
+// candidates, equal distances at the end of a list whose order they decide (W),
+// equal leading bits there.
 #define NEAR_MAX 1024  // candidates of a group
 #define NEAR_WARPS 8
 
@@ -114,14 +121,22 @@ __device__ __forceinline__ void key_sort(uint32_t (&c)[8]) {
     key_cx(c[5], c[6]);
 }
 
-// The E least keys, sorted, and with NEXT the least of all others.
-template <int E, bool NEXT>
+// The E least keys, sorted, and the NX (0, 1, 2) least of all others.
+template <int E, int NX>
 struct NearList {
-    uint32_t k[E], nx;
+    uint32_t k[E], nx, nx2;
     __device__ __forceinline__ void init() {
 #pragma unroll
         for (int i = 0; i < E; i++) k[i] = ~0u;
-        nx = ~0u;
+        nx = nx2 = ~0u;
+    }
+    // a key at or above it changes nothing
+    __device__ __forceinline__ uint32_t last() const {
+        return NX == 2 ? nx2 : (NX == 1 ? nx : k[E - 1]);
+    }
+    __device__ __forceinline__ void pass(uint32_t v) {
+        if (NX == 2) nx2 = min(nx2, max(nx, v));
+        if (NX) nx = min(nx, v);
     }
     // takes NB sorted keys
     template <int NB>
@@ -130,7 +145,7 @@ struct NearList {
         for (int i = 0; i < NB; i++) {
             const uint32_t a = k[E - 1 - i];
             k[E - 1 - i] = min(a, c[i]);
-            if (NEXT) nx = min(nx, max(a, c[i]));
+            pass(max(a, c[i]));
         }
 #pragma unroll
         for (int j = E / 2; j > 0; j >>= 1) {
@@ -144,7 +159,10 @@ struct NearList {
         uint32_t c[E];
 #pragma unroll
         for (int i = 0; i < E; i++) c[i] = __shfl_xor_sync(FULLM, k[i], off);
-        if (NEXT) nx = min(nx, __shfl_xor_sync(FULLM, nx, off));
+        const uint32_t o = NX ? __shfl_xor_sync(FULLM, nx, off) : ~0u;
+        const uint32_t o2 = NX == 2 ? __shfl_xor_sync(FULLM, nx2, off) : ~0u;
+        if (NX) pass(o);
+        if (NX == 2) pass(o2);
         merge(c);
     }
 };
@@ -157,11 +175,11 @@ struct NearSmem {
 };
 
 // The lanes' ranges [b, b + cnt) (numbers from num on) against every query.
-template <int E, bool NEXT, int NB>
+template <int E, int NX, int NB, bool WIDE>
 __device__ __forceinline__ void near_scan(const GridView& g, const KnnArgs& a, NearSmem& sm,
-                                          NearList<E, NEXT>& top, uint32_t b, uint32_t cnt,
-                                          uint32_t num, int4 qp, uint32_t self, int bits, int sub,
-                                          int lpq, int lane) {
+                                          NearList<E, NX>& top, uint32_t b, uint32_t cnt,
+                                          uint32_t num, int4 qp, uint32_t self, int bits, int cut,
+                                          int sub, int lpq, int lane) {
     const unsigned act = __ballot_sync(FULLM, cnt > 0);
     if (!act) return;
     const uint32_t inc = warp_inclusive(cnt, lane);
@@ -212,14 +230,16 @@ __device__ __forceinline__ void near_scan(const GridView& g, const KnnArgs& a, N
                 const int4 c = sm.c[i & 31];
                 const int dx = c.x - qp.x, dy = c.y - qp.y, dz = c.z - qp.z;
                 const uint32_t d2 =
-                    (uint32_t)(dx * dx) + (uint32_t)(dy * dy) + (uint32_t)(dz * dz);
+                    WIDE ? (uint32_t)(((u64)((long long)dx * dx) + (u64)((long long)dy * dy) +
+                                       (u64)((long long)dz * dz)) >> cut)
+                         : (uint32_t)(dx * dx) + (uint32_t)(dy * dy) + (uint32_t)(dz * dz);
                 const bool skip = i >= m || (uint32_t)c.w == self;
                 key[u] = skip ? ~0u : (d2 << bits) | (uint32_t)c.w;
             }
             uint32_t least = key[0];
 #pragma unroll
             for (int u = 1; u < NB; u++) least = min(least, key[u]);
-            if (__any_sync(FULLM, least < (NEXT ? top.nx : top.k[E - 1]))) {
+            if (__any_sync(FULLM, least < top.last())) {
                 key_sort(key);
                 top.merge(key);
             }
@@ -228,84 +248,46 @@ __device__ __forceinline__ void near_scan(const GridView& g, const KnnArgs& a, N
     }
 }
 
-// One leaf group (<= 32 queries) for one warp.  Returns the lane's query when
-// it is left to the warp-per-query kernel, -1 otherwise.
-template <int S, bool W>
-__device__ __forceinline__ int near_group(const GridView& g, const KnnArgs& a, int gid,
-                                          NearSmem& sm, int lane) {
+// A leaf group's queries on the lanes of one warp.
+struct NearGroup {
+    int4 qp;                // this lane's query (an idle lane: the first one's)
+    int q, nq, sub, lpq;    // its position (-1: idle); queries; lane `sub` of its `lpq`
+    int ux, uy, uz, L;
+    WarpNode n;             // this lane's cell
+    uint32_t num, self;     // number of the cell's first candidate; the query's own
+    u64 gbox;               // squared distance from the cell to the box of the queries
+    int bits, cut;          // of a key: its number's bits, distance bits left out
+};
+
+// The search of a group's queries.  Returns the lane's query when it is left to
+// the warp-per-query kernel, -1 otherwise.
+// WIDE: the keys hold d^2 >> cut, so the S nearest are known where the next key's
+// distance bits differ from the last one's, and their order from their positions.
+template <int S, bool W, bool WIDE>
+__device__ __forceinline__ int near_search(const GridView& g, const KnnArgs& a, NearSmem& sm,
+                                           const NearGroup& G, int lane) {
     const int E = S == 8 ? 8 : 16, NB = S == 8 ? 4 : 8;
-    const bool NEXT = W || S > 8;
-    const int4 G = a.groups[gid];
-    const int L = G.z;
-    int q = -1;
-    if (lane < G.y) {
-        q = G.x + lane;
-        if (a.qflag && !a.qflag[q]) q = -1;
-    }
-    // the active queries packed onto the lanes: each gets lpq of them (a power
-    // of two), which share the candidates and merge their lists
-    const unsigned act = __ballot_sync(FULLM, q >= 0);
-    if (!act) return -1;
-    const int nq = __popc(act);
-    int lpq = 32;
-    while (nq * lpq > 32) lpq >>= 1;
-    const int qi = lane / lpq, sub = lane - qi * lpq;
-    {
-        const int src = qi < nq ? (int)__fns(act, 0, qi + 1) : 0;
-        const int qq = __shfl_sync(FULLM, q, src);
-        q = qi < nq ? qq : -1;
-    }
+    const int NX = WIDE ? S - E + 1 : (W || S > 8 ? 1 : 0);
+    const int bits = G.bits, cut = WIDE ? G.cut : 0, q = G.q;
     const bool on = q >= 0;
-    // idle lanes follow the first query (its box and its bound)
-    const int q0 = __shfl_sync(FULLM, q, 0);
-    const int4 qp = g.pos[on ? q : q0];
-    const int ux = qp.x - g.origin.x, uy = qp.y - g.origin.y, uz = qp.z - g.origin.z;
-    const WarpNode n = warp_cells(g, L, g.code[G.x], ux, uy, uz, lane);
-    const uint32_t cnt = n.count();
-    // numbers in Morton order: candidates of the ranges that start before this one
-    uint32_t num = 0, total = 0;
-    for (int i = 0; i < 27; i++) {
-        const uint32_t bi = __shfl_sync(FULLM, n.b, i), ci = __shfl_sync(FULLM, cnt, i);
-        if (bi < n.b) num += ci;
-        total += ci;
-    }
-    int bits = 1;
-    while ((1u << bits) < total) bits++;
-    // d^2 < 12 * 4^(widest cell), two of its edges per axis, must fit beside the number
-    const int edge = __reduce_max_sync(FULLM, cnt > 0 ? n.lv + g.shift : 0);
-    if (total > NEAR_MAX || 2 * edge + bits > 28) return sub == 0 ? q : -1;
-    // the query's own number: its cell is lane 0's
-    const uint32_t self = __shfl_sync(FULLM, num, 0) + (uint32_t)(q - (int)__shfl_sync(FULLM, n.b, 0));
-    // squared distance from this lane's cell to the box of the group's queries
-    u64 gbox;
-    {
-        const int sh = n.lv + g.shift;
-        const int u[3] = {ux, uy, uz}, c[3] = {n.x, n.y, n.z};
-        gbox = 0;
-#pragma unroll
-        for (int x = 0; x < 3; x++) {
-            const int lo = __reduce_min_sync(FULLM, u[x]), hi = __reduce_max_sync(FULLM, u[x]);
-            const int cl = c[x] << sh, ch = cl + ((1 << sh) - 1);
-            const int d = max(max(cl - hi, lo - ch), 0);
-            gbox += (u64)((long long)d * d);
-        }
-    }
-    NearList<E, NEXT> top;
+    const int4 qp = G.qp;
+    const uint32_t cnt = G.n.count(), self = on ? G.self : ~0u;
+    NearList<E, NX> top;
     top.init();
     // the cell and its face neighbours first; the other cells only where they
     // reach the largest S-th distance of the group
-    near_scan<E, NEXT, NB>(g, a, sm, top, n.b, lane < 7 ? cnt : 0, num, qp, on ? self : ~0u, bits,
-                           sub, lpq, lane);
+    near_scan<E, NX, NB, WIDE>(g, a, sm, top, G.n.b, lane < 7 ? cnt : 0, G.num, qp, self, bits,
+                               cut, G.sub, G.lpq, lane);
     {
-        uint32_t far = NEXT ? top.nx : top.k[E - 1];  // partial lists bound the merged one
+        uint32_t far = top.last();  // partial lists bound the merged one
         if (!on) far = 0;
         far = __reduce_max_sync(FULLM, far);
-        const u64 bound = far == ~0u ? ~0ull : far >> bits;
-        near_scan<E, NEXT, NB>(g, a, sm, top, n.b, lane >= 7 && gbox <= bound ? cnt : 0, num, qp,
-                               on ? self : ~0u, bits, sub, lpq, lane);
+        const u64 bound = far == ~0u ? ~0ull : ((u64)((far >> bits) + 1) << cut) - 1;
+        near_scan<E, NX, NB, WIDE>(g, a, sm, top, G.n.b, lane >= 7 && G.gbox <= bound ? cnt : 0,
+                                   G.num, qp, self, bits, cut, G.sub, G.lpq, lane);
         if (a.pairs_out) {
-            const uint32_t mine = lane < 7 || gbox <= bound ? cnt : 0;
-            const uint32_t pairs = __reduce_add_sync(FULLM, mine) * (uint32_t)nq;
+            const uint32_t mine = lane < 7 || G.gbox <= bound ? cnt : 0;
+            const uint32_t pairs = __reduce_add_sync(FULLM, mine) * (uint32_t)G.nq;
             if (lane == 0) {
                 unsigned smid;
                 asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
@@ -313,35 +295,66 @@ __device__ __forceinline__ int near_group(const GridView& g, const KnnArgs& a, i
             }
         }
     }
-    for (int off = lpq >> 1; off >= 1; off >>= 1) top.merge_lane(off);
-    if (!on || sub) return -1;
-    const int R = a.r_exact > 0 && a.r_exact < S ? a.r_exact : S;
-    const int sh = L + g.shift;
-    const u64 gg = L >= g.B ? ~0ull : gap2(g, ux, uy, uz, L, ux >> sh, uy >> sh, uz >> sh);
-    auto dist = [&](uint32_t k) -> u64 { return k == ~0u ? ~0ull : k >> bits; };
-    u64 bound = 0;
-#pragma unroll
-    for (int i = 0; i < E; i++)
-        if (i == R - 1) bound = dist(top.k[i]);
-    if (R > E) bound = dist(top.nx);
-    if (!(gg == ~0ull || bound < gg)) return q;
-    if (W && top.nx != ~0u && dist(top.nx) == dist(top.k[E - 1])) return q;
-    // positions; with W equal distances in the order of the input index
-    int id[E];
+    for (int off = G.lpq >> 1; off >= 1; off >>= 1) top.merge_lane(off);
+    if (!on || G.sub) return -1;
+    // the S nearest: key i, and past the list its successor
+    auto key = [&](int i) -> uint32_t { return i < E ? top.k[i < E ? i : 0] : top.nx; };
+    auto same = [&](uint32_t x, uint32_t y) { return y != ~0u && x >> bits == y >> bits; };
+    if (WIDE && same(key(S - 1), top.last())) return q;
+    int id[S], ix[S];
+    u64 wd[S];  // WIDE: exact distances
     int found = 0;
 #pragma unroll
-    for (int i = 0; i < E; i++) {
-        const bool has = top.k[i] != ~0u;
+    for (int i = 0; i < S; i++) {
+        const bool has = key(i) != ~0u;
         found += has;
-        id[i] = has ? sm.pos[top.k[i] & ((1u << bits) - 1u)] : -1;
+        id[i] = has ? sm.pos[key(i) & ((1u << bits) - 1u)] : -1;
+        if (WIDE) {
+            const int4 v = g.pos[has ? id[i] : 0];
+            wd[i] = has ? sqd(v, qp) : ~0ull;
+            ix[i] = W ? v.w : id[i];
+        }
     }
-    if (W) {
+    if (WIDE) {
+        // (distance, tie) within a run of equal keys
+        bool again = true;
+        while (again) {
+            again = false;
+#pragma unroll
+            for (int i = 0; i + 1 < S; i++) {
+                const bool sw = wd[i] > wd[i + 1] ||
+                                (wd[i] == wd[i + 1] && wd[i] != ~0ull && ix[i] > ix[i + 1]);
+                const u64 d = wd[i];
+                const int x = ix[i], y = id[i];
+                wd[i] = sw ? wd[i + 1] : d;
+                ix[i] = sw ? ix[i + 1] : x;
+                id[i] = sw ? id[i + 1] : y;
+                wd[i + 1] = sw ? d : wd[i + 1];
+                ix[i + 1] = sw ? x : ix[i + 1];
+                id[i + 1] = sw ? y : id[i + 1];
+                again = again || sw;
+            }
+        }
+    }
+    auto dist = [&](int i) -> u64 {
+        return WIDE ? wd[i] : (key(i) == ~0u ? ~0ull : (u64)(key(i) >> bits));
+    };
+    const int R = a.r_exact > 0 && a.r_exact < S ? a.r_exact : S;
+    const int sh = G.L + g.shift;
+    const u64 gg = G.L >= g.B ? ~0ull
+                              : gap2(g, G.ux, G.uy, G.uz, G.L, G.ux >> sh, G.uy >> sh, G.uz >> sh);
+    u64 bound = 0;
+#pragma unroll
+    for (int i = 0; i < S; i++)
+        if (i == R - 1) bound = dist(i);
+    if (!(gg == ~0ull || bound < gg)) return q;
+    if (!WIDE && W) {
+        if (same(top.k[E - 1], top.nx)) return q;
+        // equal distances in the order of the input index
         bool tie = false;
 #pragma unroll
-        for (int i = 0; i + 1 < E; i++)
-            tie = tie || (id[i + 1] >= 0 && top.k[i] >> bits == top.k[i + 1] >> bits);
+        for (int i = 0; i + 1 < E; i++) tie = tie || same(top.k[i], top.k[i + 1]);
         if (tie) {
-            int ix[E];
 #pragma unroll
             for (int i = 0; i < E; i++) ix[i] = id[i] >= 0 ? g.pos[id[i]].w : 0x7fffffff;
             while (tie) {
@@ -361,26 +374,20 @@ __device__ __forceinline__ int near_group(const GridView& g, const KnnArgs& a, i
         }
     }
     // results of the query
-    int nxt = -1;
-    if (S > E && top.nx != ~0u) {
-        nxt = sm.pos[top.nx & ((1u << bits) - 1u)];
-        found++;
-    }
     if (S == 8) {
         store_nbr8(a.nbr, q, reinterpret_cast<int(&)[8]>(id));
     } else {
 #pragma unroll
-        for (int i = 0; i < E; i++) a.nbr[(int64_t)q * S + i] = id[i];
-        a.nbr[(int64_t)q * S + E] = nxt;
+        for (int i = 0; i < S; i++) a.nbr[(int64_t)q * S + i] = id[i];
     }
-    const u64 ds = S > E ? dist(top.nx) : dist(top.k[E - 1]);  // the S-th
+    const u64 ds = dist(S - 1);
     if (a.density_k1) {
         // all S nearest are stored (the k+b buffer); the shell is the prefix at
         // the nearest distance d0, its size kept in flg >> 2
-        const u64 d0 = dist(top.k[0]);
+        const u64 d0 = dist(0);
         int shell = 0;
 #pragma unroll
-        for (int i = 0; i < E; i++) shell += top.k[i] != ~0u && dist(top.k[i]) == d0;
+        for (int i = 0; i < E; i++) shell += dist(i) != ~0ull && dist(i) == d0;
         if (!W && a.nbr0_out) a.nbr0_out[q] = id[0];
         a.prim_out[q] = key_prim_d2(d0);
         a.rk2_out[q] = d0;
@@ -393,19 +400,90 @@ __device__ __forceinline__ int near_group(const GridView& g, const KnnArgs& a, i
     double c = 0.0;
     u64 dk = ~0ull, dn = ~0ull;
 #pragma unroll
-    for (int i = 0; i < E; i++) {
-        const u64 d = dist(top.k[i]);
-        if (i < a.k && id[i] >= 0) c = __dadd_rn(c, __ddiv_rn(nbr_weight(a, q, id[i]), (double)d));
+    for (int i = 0; i < S; i++) {
+        const u64 d = dist(i);
+        if (i < E && i < a.k && id[i] >= 0)
+            c = __dadd_rn(c, __ddiv_rn(nbr_weight(a, q, id[i]), (double)d));
         if (i == a.k - 1) dk = d;
         if (i == a.k) dn = d;
     }
-    if (a.k == E) dn = dist(top.nx);
     a.prim_out[q] = key_prim_cost(c);
     a.rk2_out[q] = dk;
     a.flg_out[q] = (uint8_t)(found > a.k && dn == dk ? 1 : 0);
     if (a.hz_out) a.hz_out[q] = ds;
     if (a.cost_out) a.cost_out[q] = c;
     return -1;
+}
+
+// One leaf group (<= 32 queries) for one warp: sets the search up.
+template <int S, bool W>
+__device__ __forceinline__ int near_group(const GridView& g, const KnnArgs& a, int gid,
+                                          NearSmem& sm, int lane) {
+    const int4 gr = a.groups[gid];
+    NearGroup G;
+    G.L = gr.z;
+    int q = -1;
+    if (lane < gr.y) {
+        q = gr.x + lane;
+        if (a.qflag && !a.qflag[q]) q = -1;
+    }
+    // the active queries packed onto the lanes: each gets lpq of them (a power
+    // of two), which share the candidates and merge their lists
+    const unsigned act = __ballot_sync(FULLM, q >= 0);
+    if (!act) return -1;
+    G.nq = __popc(act);
+    int lpq = 32;
+    while (G.nq * lpq > 32) lpq >>= 1;
+    const int qi = lane / lpq;
+    G.lpq = lpq;
+    G.sub = lane - qi * lpq;
+    {
+        const int src = qi < G.nq ? (int)__fns(act, 0, qi + 1) : 0;
+        const int qq = __shfl_sync(FULLM, q, src);
+        q = qi < G.nq ? qq : -1;
+    }
+    G.q = q;
+    // idle lanes follow the first query (its box and its bound)
+    const int q0 = __shfl_sync(FULLM, q, 0);
+    G.qp = g.pos[q >= 0 ? q : q0];
+    G.ux = G.qp.x - g.origin.x;
+    G.uy = G.qp.y - g.origin.y;
+    G.uz = G.qp.z - g.origin.z;
+    G.n = warp_cells(g, G.L, g.code[gr.x], G.ux, G.uy, G.uz, lane);
+    const uint32_t cnt = G.n.count();
+    // numbers in Morton order: candidates of the ranges that start before this one
+    uint32_t num = 0, total = 0;
+    for (int i = 0; i < 27; i++) {
+        const uint32_t bi = __shfl_sync(FULLM, G.n.b, i), ci = __shfl_sync(FULLM, cnt, i);
+        if (bi < G.n.b) num += ci;
+        total += ci;
+    }
+    G.num = num;
+    int bits = 1;
+    while ((1u << bits) < total) bits++;
+    G.bits = bits;
+    // d^2 < 12 * 4^(widest cell), two of its edges per axis: what of it does not fit
+    // beside the number
+    const int edge = __reduce_max_sync(FULLM, cnt > 0 ? G.n.lv + g.shift : 0);
+    G.cut = 2 * edge + bits - 28;
+    if (total > NEAR_MAX) return G.sub == 0 ? q : -1;
+    // the query's own number: its cell is lane 0's
+    G.self = __shfl_sync(FULLM, num, 0) + (uint32_t)(q - (int)__shfl_sync(FULLM, G.n.b, 0));
+    // squared distance from this lane's cell to the box of the group's queries
+    {
+        const int sh = G.n.lv + g.shift;
+        const int u[3] = {G.ux, G.uy, G.uz}, c[3] = {G.n.x, G.n.y, G.n.z};
+        G.gbox = 0;
+#pragma unroll
+        for (int x = 0; x < 3; x++) {
+            const int lo = __reduce_min_sync(FULLM, u[x]), hi = __reduce_max_sync(FULLM, u[x]);
+            const int cl = c[x] << sh, ch = cl + ((1 << sh) - 1);
+            const int d = max(max(cl - hi, lo - ch), 0);
+            G.gbox += (u64)((long long)d * d);
+        }
+    }
+    return G.cut > 0 ? near_search<S, W, true>(g, a, sm, G, lane)
+                     : near_search<S, W, false>(g, a, sm, G, lane);
 }
 
 template <int S, bool W>
