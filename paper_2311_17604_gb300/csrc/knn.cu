@@ -79,6 +79,9 @@ __device__ inline double nbr_weight(const KnnArgs& a, int q, int j) {
 // made the pass of a cloud with 1 m between its points slower than the chain had
 // (1.0M points, grid and pass: k = 6 1.91 ms with the chain, 3.99 a warp each, 1.06
 // now; k = 1 1.61, 3.54, 0.95; 17 stored 5.53, 5.06, 1.96).
+// Weighted costs of 7 neighbours and more need the 17th entry in order too, hence two
+// successors of the list's 16 (1.0M room points with colours, k = 7: 4.40 ms with the
+// chain, 4.48 a warp each, 2.58 now; k = 16 6.17, 5.08, 4.12).
 // What one level cannot settle goes to a list that the warp-per-query kernel
 // finishes: the S-th distance beyond the cube's faces, more than NEAR_MAX
 // candidates, equal distances at the end of a list whose order they decide (W),
@@ -263,11 +266,14 @@ struct NearGroup {
 // the warp-per-query kernel, -1 otherwise.
 // WIDE: the keys hold d^2 >> cut, so the S nearest are known where the next key's
 // distance bits differ from the last one's, and their order from their positions.
-template <int S, bool W, bool WIDE>
+// W: equal distances in the order of the input index (1: of the first 8 or 16,
+// 2: of all S, which a weighted cost of 7 neighbours or more needs).
+template <int S, int W, bool WIDE>
 __device__ __forceinline__ int near_search(const GridView& g, const KnnArgs& a, NearSmem& sm,
                                            const NearGroup& G, int lane) {
     const int E = S == 8 ? 8 : 16, NB = S == 8 ? 4 : 8;
-    const int NX = WIDE ? S - E + 1 : (W || S > 8 ? 1 : 0);
+    const int T = W == 2 ? S : E;  // entries in order with W
+    const int NX = WIDE ? S - E + 1 : (W ? T - E + 1 : S - E);
     const int bits = G.bits, cut = WIDE ? G.cut : 0, q = G.q;
     const bool on = q >= 0;
     const int4 qp = G.qp;
@@ -349,19 +355,19 @@ __device__ __forceinline__ int near_search(const GridView& g, const KnnArgs& a, 
         if (i == R - 1) bound = dist(i);
     if (!(gg == ~0ull || bound < gg)) return q;
     if (!WIDE && W) {
-        if (same(top.k[E - 1], top.nx)) return q;
+        if (same(key(T - 1), T > E ? top.nx2 : top.nx)) return q;
         // equal distances in the order of the input index
         bool tie = false;
 #pragma unroll
-        for (int i = 0; i + 1 < E; i++) tie = tie || same(top.k[i], top.k[i + 1]);
+        for (int i = 0; i + 1 < T; i++) tie = tie || same(key(i), key(i + 1));
         if (tie) {
 #pragma unroll
-            for (int i = 0; i < E; i++) ix[i] = id[i] >= 0 ? g.pos[id[i]].w : 0x7fffffff;
+            for (int i = 0; i < T; i++) ix[i] = id[i] >= 0 ? g.pos[id[i]].w : 0x7fffffff;
             while (tie) {
                 tie = false;
 #pragma unroll
-                for (int i = 0; i + 1 < E; i++) {
-                    if (top.k[i] >> bits == top.k[i + 1] >> bits && ix[i] > ix[i + 1]) {
+                for (int i = 0; i + 1 < T; i++) {
+                    if (key(i) >> bits == key(i + 1) >> bits && ix[i] > ix[i + 1]) {
                         const int x = ix[i], y = id[i];
                         ix[i] = ix[i + 1];
                         id[i] = id[i + 1];
@@ -416,7 +422,7 @@ __device__ __forceinline__ int near_search(const GridView& g, const KnnArgs& a, 
 }
 
 // One leaf group (<= 32 queries) for one warp: sets the search up.
-template <int S, bool W>
+template <int S, int W>
 __device__ __forceinline__ int near_group(const GridView& g, const KnnArgs& a, int gid,
                                           NearSmem& sm, int lane) {
     const int4 gr = a.groups[gid];
@@ -486,7 +492,7 @@ __device__ __forceinline__ int near_group(const GridView& g, const KnnArgs& a, i
                      : near_search<S, W, false>(g, a, sm, G, lane);
 }
 
-template <int S, bool W>
+template <int S, int W>
 __global__ void __launch_bounds__(NEAR_WARPS * 32, S == 8 ? 4 : 2)
     knn_kernel(GridView g, KnnArgs a, int* rest, int* nrest) {
     chain();
@@ -1029,16 +1035,6 @@ __global__ void __launch_bounds__(PD_WARPS * 32, ORDER ? 8 : 10)
     }
 }
 
-// Every point (every flagged one) to the list.
-__global__ void list_queries_kernel(const uint8_t* qflag, int64_t n, int* rest,
-                                    int* nrest) {
-    chain();
-    const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const bool in = s < n && (!qflag || qflag[s]);
-    const int slot = block_append(in, nrest);
-    if (in) rest[slot] = (int)s;
-}
-
 cudaError_t launch_knn_queries(const GridView& g, const KnnArgs& a, int64_t cap, cudaStream_t st) {
     if (cap <= 0) return cudaSuccess;
     const bool filtered = a.qlist2 != nullptr;
@@ -1064,18 +1060,14 @@ cudaError_t launch_knn(const GridView& g, const KnnArgs& a, int64_t n, int* rest
     if (e) return e;
     const unsigned blocks = (unsigned)((a.ngroups + NEAR_WARPS - 1) / NEAR_WARPS);
     const dim3 gr(blocks), bl(NEAR_WARPS * 32);
-    // 17 stored with weights: the order of equal distances decides the 17th
-    // entry too, which the list's 16 and their successor do not settle
-    const bool all_rest = a.S == 17 && a.term != 0 && a.term != PD_TERM_INDEX_TIE;
     if (a.S == 8) {
-        if (a.term != 0) launch_chained(knn_kernel<8, true>, gr, bl, 0, st, g, a, rest, nrest);
-        else launch_chained(knn_kernel<8, false>, gr, bl, 0, st, g, a, rest, nrest);
-    } else if (a.S == 17 && !all_rest) {
-        if (a.term != 0) launch_chained(knn_kernel<17, true>, gr, bl, 0, st, g, a, rest, nrest);
-        else launch_chained(knn_kernel<17, false>, gr, bl, 0, st, g, a, rest, nrest);
+        if (a.term != 0) launch_chained(knn_kernel<8, 1>, gr, bl, 0, st, g, a, rest, nrest);
+        else launch_chained(knn_kernel<8, 0>, gr, bl, 0, st, g, a, rest, nrest);
     } else if (a.S == 17) {
-        launch_chained(list_queries_kernel, (unsigned)((n + 255) / 256), 256, 0, st, a.qflag, n,
-                       rest, nrest);
+        if (a.term == PD_TERM_INDEX_TIE)
+            launch_chained(knn_kernel<17, 1>, gr, bl, 0, st, g, a, rest, nrest);
+        else if (a.term != 0) launch_chained(knn_kernel<17, 2>, gr, bl, 0, st, g, a, rest, nrest);
+        else launch_chained(knn_kernel<17, 0>, gr, bl, 0, st, g, a, rest, nrest);
     } else {
         return cudaErrorInvalidValue;
     }
