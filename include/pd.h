@@ -132,8 +132,9 @@ void pd_ctx_destroy(pd_ctx* ctx);
  *     mapped host memory (cudaHostAlloc) instead;
  *   - the kernels address those blocks in place (unified addressing), so a
  *     decimation gives the same result at any budget, only slower;
- *   - blocks below 1 MiB (control blocks, counters, histograms: they take
- *     device atomics) always stay in device memory.
+ *   - blocks below 1 MiB (control blocks, counters) and blocks that the rounds
+ *     and searches update with atomics (the candidates' bitmap, a bit a point;
+ *     histograms) always stay in device memory.
  * bytes = 0 lifts the budget: nothing more spills (blocks already in host
  * memory stay there until freed).  Freeing a host block waits for the stream
  * it was used on.  The budget

@@ -105,21 +105,28 @@ static void dev_free(pd_ctx* c, void* p, cudaStream_t st) {
     else cudaFreeAsync(p, st);
 }
 
-// Blocks below this size always stay in device memory: the small control
-// blocks, counters and histograms take device atomics.
+// Blocks below this size always stay in device memory (control blocks, counters).
 #define PD_SPILL_FLOOR ((size_t)1 << 20)
 
-// cold: a block the kernels touch about once (input copies, write-mostly
-// state); under a budget such blocks go to host memory first.
-static void* ctx_alloc(pd_ctx* c, size_t bytes, cudaStream_t st, bool cold = false) {
+// Where a block may lie under a budget.  Cold: the kernels touch it about once (input
+// copies, write-mostly state), so it goes to host memory first.  Device: it takes
+// atomics on every round or query (bitmap of the candidates, histograms), which are
+// slow over the host link, so it stays in device memory whatever its size.  The one
+// block with atomics that may be placed in host memory is the cell table, whose
+// slots a build claims once each (natively atomic over NVLink-C2C): at 16 bytes a
+// slot it is too large to hold back.
+enum Place { PLACE_ANY, PLACE_COLD, PLACE_DEVICE };
+
+static void* ctx_alloc(pd_ctx* c, size_t bytes, cudaStream_t st, Place place = PLACE_ANY) {
     if (bytes == 0) bytes = 16;
     bytes = (bytes + 255) & ~(size_t)255;
     if (!c->tracked.load()) return dev_alloc(c, bytes, st);
     bool host;
     {
         std::lock_guard<std::mutex> lk(c->mem_mu);
-        host = c->dev_budget > 0 && bytes >= PD_SPILL_FLOOR && bytes >= c->spill_min &&
-               (cold || c->dev_used + bytes > c->dev_budget);
+        host = c->dev_budget > 0 && place != PLACE_DEVICE && bytes >= PD_SPILL_FLOOR &&
+               bytes >= c->spill_min &&
+               (place == PLACE_COLD || c->dev_used + bytes > c->dev_budget);
         if (!host) c->dev_used += bytes;  // reserved before the call
     }
     void* p = nullptr;
@@ -276,25 +283,17 @@ GridView view_of(const pd_grid* g) {
         }                                                                      \
     } while (0)
 
-#define ALLOC(ptr, type, count)                                                \
-    do {                                                                       \
-        ptr = (type*)ctx_alloc(g->ctx, sizeof(type) * (size_t)(count), g->st); \
-        if (!ptr) {                                                            \
-            set_err(g->ctx, "allocation of %s failed (%lld bytes)", #ptr,      \
-                    (long long)(sizeof(type) * (size_t)(count)));              \
-            return PD_ENOMEM;                                                  \
-        }                                                                      \
-    } while (0)
-
-#define ALLOC_COLD(ptr, type, count)                                                \
+#define ALLOC_AT(ptr, type, count, place)                                            \
     do {                                                                             \
-        ptr = (type*)ctx_alloc(g->ctx, sizeof(type) * (size_t)(count), g->st, true); \
+        ptr = (type*)ctx_alloc(g->ctx, sizeof(type) * (size_t)(count), g->st, place); \
         if (!ptr) {                                                                  \
             set_err(g->ctx, "allocation of %s failed (%lld bytes)", #ptr,            \
                     (long long)(sizeof(type) * (size_t)(count)));                    \
             return PD_ENOMEM;                                                        \
         }                                                                            \
     } while (0)
+#define ALLOC(ptr, type, count) ALLOC_AT(ptr, type, count, PLACE_ANY)
+#define ALLOC_COLD(ptr, type, count) ALLOC_AT(ptr, type, count, PLACE_COLD)
 
 void gfree(pd_grid* g, void* p) { ctx_free(g->ctx, p, g->st); }
 
@@ -1004,11 +1003,12 @@ struct RoundScratch {
         if (e1) cudaEventDestroy(e1);
     }
 };
-#define RALLOC(ptr, type, count)              \
+#define RALLOC_AT(ptr, type, count, place)    \
     do {                                      \
-        ALLOC(ptr, type, count);              \
+        ALLOC_AT(ptr, type, count, place);    \
         rs.ptrs.push_back((void*)(ptr));      \
     } while (0)
+#define RALLOC(ptr, type, count) RALLOC_AT(ptr, type, count, PLACE_ANY)
 
 // kernel nodes of a captured graph (launch accounting of replayed rounds)
 long long count_kernel_nodes(cudaGraph_t graph) {
@@ -1118,7 +1118,7 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
     CK(cudaMemsetAsync(rej, 0, cap, g->st));
     int pair_cap = 0;
     if (!g->density_k1) {
-        RALLOC(inPb, uint32_t, (cap + 31) / 32);
+        RALLOC_AT(inPb, uint32_t, (cap + 31) / 32, PLACE_DEVICE);
         RALLOC(fq, int, cap);
         RALLOC(lq, int, cap);
         RALLOC(src, int, cap);
@@ -1142,7 +1142,7 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
     RALLOC(rd, RoundDev, 1);
     uint32_t* seg_hist = nullptr;  // packed batch: a 4096-bin histogram per scan
     if (g->nseg) {
-        RALLOC(seg_hist, uint32_t, (size_t)g->nseg * 4096);
+        RALLOC_AT(seg_hist, uint32_t, (size_t)g->nseg * 4096, PLACE_DEVICE);
         CK(cudaMemsetAsync(seg_hist, 0, (size_t)g->nseg * 4096 * sizeof(uint32_t), g->st));
     }
     RoundDev h;
@@ -1585,12 +1585,12 @@ extern "C" int pd_decimate_host(pd_ctx* ctx, const int32_t* xyz_host, const uint
                                 int64_t m, uint8_t* keep_host, void* stream, pd_stats* stats) {
     if (!ctx || !xyz_host || !keep_host || !cp || n < 1) return PD_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    int32_t* xyz = (int32_t*)ctx_alloc(ctx, (size_t)n * 12, st, true);
-    uint8_t* rgb = rgb_host ? (uint8_t*)ctx_alloc(ctx, (size_t)n * 3, st, true) : nullptr;
+    int32_t* xyz = (int32_t*)ctx_alloc(ctx, (size_t)n * 12, st, PLACE_COLD);
+    uint8_t* rgb = rgb_host ? (uint8_t*)ctx_alloc(ctx, (size_t)n * 3, st, PLACE_COLD) : nullptr;
     float* nrm = normals_host && cp->term == PD_TERM_ORIENT
-                     ? (float*)ctx_alloc(ctx, (size_t)n * 12, st, true)
+                     ? (float*)ctx_alloc(ctx, (size_t)n * 12, st, PLACE_COLD)
                      : nullptr;
-    uint8_t* keep = (uint8_t*)ctx_alloc(ctx, (size_t)n, st, true);
+    uint8_t* keep = (uint8_t*)ctx_alloc(ctx, (size_t)n, st, PLACE_COLD);
     int rc = PD_OK;
     if (!xyz || !keep || (rgb_host && !rgb) || (normals_host && cp->term == PD_TERM_ORIENT && !nrm)) {
         set_err(ctx, "pd_decimate_host: allocation failed%s", "", 0);
@@ -1807,8 +1807,8 @@ extern "C" int pd_quality_report(pd_ctx* ctx, const int32_t* xyz_dev, const uint
     sc.free = cs_free;
     sc.self = &cs;
     std::vector<void*> owned;
-    auto get = [&](size_t bytes) {
-        void* p = ctx_alloc(ctx, bytes, st);
+    auto get = [&](size_t bytes, Place place = PLACE_ANY) {
+        void* p = ctx_alloc(ctx, bytes, st, place);
         if (p) owned.push_back(p);
         return p;
     };
@@ -1827,15 +1827,16 @@ extern "C" int pd_quality_report(pd_ctx* ctx, const int32_t* xyz_dev, const uint
             return e_ == cudaErrorMemoryAllocation ? PD_ENOMEM : PD_ECUDA;         \
         }                                                                          \
     } while (0)
-#define QGET(ptr, type, count)                                                     \
+#define QGET_AT(ptr, type, count, place)                                           \
     do {                                                                           \
-        ptr = (type*)get(sizeof(type) * (size_t)(count));                          \
+        ptr = (type*)get(sizeof(type) * (size_t)(count), place);                   \
         if (!ptr) {                                                                \
             set_err(ctx, "pd_quality_report: allocation of %s failed (%lld)", #ptr, \
                     (long long)(count));                                   \
             return PD_ENOMEM;                                                      \
         }                                                                          \
     } while (0)
+#define QGET(ptr, type, count) QGET_AT(ptr, type, count, PLACE_ANY)
         QCK(cudaEventRecord(e0, st));
         // the retained points, in input order
         const int32_t* xyz = xyz_dev;
@@ -1904,7 +1905,7 @@ extern "C" int pd_quality_report(pd_ctx* ctx, const int32_t* xyz_dev, const uint
         QGET(r2, u64, nr);
         QGET(sn, u64, nr);
         QGET(sn2, u64, nr);
-        QGET(hist, uint32_t, (size_t)nr * H);
+        QGET_AT(hist, uint32_t, (size_t)nr * H, PLACE_DEVICE);
         int* next;
         QGET(next, int, 1);
         std::vector<u64> hr2(nr);
