@@ -61,6 +61,13 @@ __device__ inline double nbr_weight(const KnnArgs& a, int q, int j) {
     return 1.0;
 }
 
+// Pairs scanned, to this SM's slot.
+__device__ __forceinline__ void add_pairs(const KnnArgs& a, uint32_t pairs) {
+    unsigned smid;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
+    atomicAdd(&a.pairs_out[smid % PD_PAIR_SLOTS], (unsigned long long)pairs);
+}
+
 // ------------------------------------------------------------------ one warp per leaf group
 // The full pass: a thread (or several) per query of a leaf group, one level.
 // The candidates of the 27 cells get local numbers in Morton order, so that a
@@ -294,11 +301,7 @@ __device__ __forceinline__ int near_search(const GridView& g, const KnnArgs& a, 
         if (a.pairs_out) {
             const uint32_t mine = lane < 7 || G.gbox <= bound ? cnt : 0;
             const uint32_t pairs = __reduce_add_sync(FULLM, mine) * (uint32_t)G.nq;
-            if (lane == 0) {
-                unsigned smid;
-                asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
-                atomicAdd(&a.pairs_out[smid % PD_PAIR_SLOTS], (unsigned long long)pairs);
-            }
+            if (lane == 0) add_pairs(a, pairs);
         }
     }
     for (int off = G.lpq >> 1; off >= 1; off >>= 1) top.merge_lane(off);
@@ -754,6 +757,7 @@ struct WarpList32 {
 struct WarpRanges {  // non-empty ranges laid end to end
     uint32_t first[33];  // prefix counts
     uint32_t start[32];
+    uint32_t pairs;      // candidates of the query so far (where a.pairs_out asks)
 };
 
 template <int FILT>
@@ -809,6 +813,7 @@ struct WarpSearch {
             wr.start[at] = b;
         }
         if (lane == 0) wr.first[__popc(act)] = total;
+        if (FILT == FILT_NONE && a.pairs_out && lane == 0) wr.pairs += total;
         __syncwarp();
         int r = 0;
         uint32_t t = lane;
@@ -989,6 +994,7 @@ __device__ __forceinline__ void warp_query(const GridView& g, const KnnArgs& a, 
     }
     u64 cap_d = ~0ull;  // the S-th key found so far bounds the next level's search
     uint32_t cap_t = 0;
+    if (FILT == FILT_NONE && lane == 0) wr.pairs = 0;
     for (;; L++) {
         const WarpNode n = warp_cells(g, L, c0, ux, uy, uz, lane);
         const int sh = L + g.shift;
@@ -1002,6 +1008,7 @@ __device__ __forceinline__ void warp_query(const GridView& g, const KnnArgs& a, 
                                                            uy, uz, gg, cap_d, cap_t, lane);
         if (done || L >= g.B) break;
     }
+    if (FILT == FILT_NONE && a.pairs_out && lane == 0) add_pairs(a, wr.pairs);
 }
 
 #define TAKE_MOST 16  // queries per warp up to which a list is taken one by one
