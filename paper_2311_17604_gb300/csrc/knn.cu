@@ -39,26 +39,7 @@ __device__ inline u64 gap2(const GridView& g, int ux, int uy, int uz, int L, int
 }
 
 __device__ inline double nbr_weight(const KnnArgs& a, int q, int j) {
-    if (a.term == 1) {  // colour deviation
-        uchar4 p = a.rgb[q], r = a.rgb[j];
-        double dr = (double)p.x - (double)r.x;
-        double dg = (double)p.y - (double)r.y;
-        double db = (double)p.z - (double)r.z;
-        double s = __dmul_rn(dr, dr);
-        s = __dadd_rn(s, __dmul_rn(dg, dg));
-        s = __dadd_rn(s, __dmul_rn(db, db));
-        double dist = __dsqrt_rn(s);
-        double scale = __dmul_rn(255.0, __dsqrt_rn(3.0));
-        return __dsub_rn(1.0, __dmul_rn(a.weight, __ddiv_rn(dist, scale)));
-    }
-    if (a.term == 2) {  // orientation, Eq. 13 with |n_p . n_q|
-        float4 p = a.nrm[q], r = a.nrm[j];
-        double d = __dmul_rn((double)p.x, (double)r.x);
-        d = __dadd_rn(d, __dmul_rn((double)p.y, (double)r.y));
-        d = __dadd_rn(d, __dmul_rn((double)p.z, (double)r.z));
-        return __dsub_rn(1.0, __dmul_rn(a.weight, __dsub_rn(1.0, fabs(d))));
-    }
-    return 1.0;
+    return term_weight(a.term, a.weight, a.rgb, a.nrm, q, j);
 }
 
 // Pairs scanned, to this SM's slot.

@@ -155,6 +155,16 @@ __device__ inline unsigned long long key_prim_cost(double c) {
 __device__ inline bool key_gt(unsigned long long pa, int ia, unsigned long long pb, int ib) {
     return pa > pb || (pa == pb && ia > ib);
 }
+// Digit `pass` (12 bits) of the 96-bit key (prim << 32 | input index), most
+// significant first: passes 0-4 read prim, 5 straddles, 6-7 read the index.
+__device__ inline uint32_t key_digit(unsigned long long prim, int idx, int pass) {
+    const int lo = 84 - 12 * pass;  // lowest bit of the digit
+    const uint32_t ui = (uint32_t)idx;
+    if (lo >= 32) return (uint32_t)(prim >> (lo - 32)) & 0xfffu;
+    if (lo + 12 <= 32) return (ui >> lo) & 0xfffu;
+    // straddle: bits [lo, 32) of idx and [0, lo + 12 - 32) of prim
+    return ((uint32_t)(prim << (32 - lo)) | (ui >> lo)) & 0xfffu;
+}
 
 // Per-neighbour weight of the optional cost terms (section "Additional cost
 // terms"): 1 - a * ||rgb_p - rgb_q|| / (255 sqrt 3) for colour, 1 - a * (1 -
@@ -352,8 +362,6 @@ __device__ __forceinline__ int warp_take(int* next, int lane) {
 int device_sms();
 
 // ---------------------------------------------------------------- warp utils
-__device__ inline int warp_lane() { return threadIdx.x & 31; }
-
 // The 3x3x3 cells around a query cell in the order they are scanned: the
 // cell itself, the 6 face neighbours, the 12 edge and the 8 corner neighbours
 // (cell o = (dx+1) + 3 (dy+1) + 9 (dz+1)).  Nearer cells first tighten the

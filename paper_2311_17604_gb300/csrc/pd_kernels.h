@@ -89,7 +89,7 @@ struct RoundDev {
     long long live, m, need, rank;
     double band, band_max;
     unsigned long long removed, cap_over;
-    unsigned long long tot_requery, tot_filtered, tot_sources, tot_updated, tot_lambda;
+    unsigned long long tot_requery, tot_filtered, tot_sources, tot_lambda;
     unsigned long long tau_prim;
     int tau_idx;
     int done;
@@ -204,15 +204,6 @@ cudaError_t launch_knn_queries(const GridView& g, const KnnArgs& a, int64_t cap,
 // input index (the normals' 16-NN order).
 #define PD_TERM_INDEX_TIE 3
 
-// ---------------------------------------------------------------- rounds.cu
-struct SelectResult {
-    u64 prim;
-    int idx;
-};
-
-}  // namespace pd
-
-namespace pd {
 // ---------------------------------------------------------------- rounds_dev.cu
 // Sizes of launches that walk lists whose length the device knows: n / per
 // blocks, at most `per_sm` per multiprocessor (an idle block costs about as

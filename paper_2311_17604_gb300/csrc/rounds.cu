@@ -58,17 +58,8 @@ __global__ void dup_remove_kernel(const uint8_t* __restrict__ dup, const int4* _
 }
 
 // ------------------------------------------------------------------ selection
-// Digit `pass` (12 bits) of the 96-bit key (prim << 32 | input index),
-// most significant first: passes 0-4 read prim, 5 straddles, 6-7 read idx.
-__device__ inline uint32_t key_digit(u64 prim, int idx, int pass) {
-    int lo = 84 - 12 * pass;  // lowest bit of the digit
-    uint32_t ui = (uint32_t)idx;
-    if (lo >= 32) return (uint32_t)(prim >> (lo - 32)) & 0xfffu;
-    if (lo + 12 <= 32) return (ui >> lo) & 0xfffu;
-    // straddle: bits [lo, 32) of idx and [0, lo + 12 - 32) of prim
-    int nlow = 32 - lo;
-    return ((uint32_t)(prim << nlow) | (ui >> lo)) & 0xfffu;
-}
+// By the host, digit by digit: the largest key of a round that the device did not
+// settle, and the coincident points to remove.  The rounds' own is select.cu.
 __device__ inline bool prefix_match(u64 prim, int idx, int npass, const uint32_t* pre) {
     for (int p = 0; p < npass; p++)
         if (key_digit(prim, idx, p) != pre[p]) return false;

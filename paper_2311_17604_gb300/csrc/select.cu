@@ -32,16 +32,6 @@ namespace cg = cooperative_groups;
 #define SEL_CLUSTER 8      // blocks of the cluster that settles a list
 #define SEL_CLUSTER_MAX 64 // scans of a batch up to which each has a cluster of its own
 
-// Digit `pass` (12 bits) of the key, most significant first.
-__device__ inline uint32_t sel_digit(u64 prim, int idx, int pass) {
-    int lo = 84 - 12 * pass;
-    uint32_t ui = (uint32_t)idx;
-    if (lo >= 32) return (uint32_t)(prim >> (lo - 32)) & 0xfffu;
-    if (lo + 12 <= 32) return (ui >> lo) & 0xfffu;
-    int nlow = 32 - lo;
-    return ((uint32_t)(prim << nlow) | (ui >> lo)) & 0xfffu;
-}
-
 struct SelBin {
     int bin;                      // -1: the rank is beyond the count
     unsigned long long cum, cnt;  // keys above the bin, keys in it
@@ -148,8 +138,7 @@ struct SelItem {
     long long lo, hi;
     unsigned items;  // of this scan
 };
-__device__ inline SelItem sel_item(const RoundDev* rd, const SegDev* seg, const int* items, int w,
-                                   int64_t n) {
+__device__ inline SelItem sel_item(const RoundDev* rd, const SegDev* seg, const int* items, int w) {
     SelItem it;
     it.seg = items[w];
     const SegDev& s = seg[it.seg];
@@ -212,7 +201,7 @@ __global__ void __launch_bounds__(SEL_T)
         it.seg = 0;
         uint32_t pre0 = 0;
         if (SEG) {
-            it = sel_item(rd, seg, items, w, n);
+            it = sel_item(rd, seg, items, w);
             if (PASS > 0 && seg[it.seg].done) continue;
             if (PASS > 0) pre0 = seg[it.seg].pre[0];
         } else {
@@ -300,7 +289,7 @@ __global__ void __launch_bounds__(SEL_T)
         uint32_t want;
         int* count;
         if (SEG) {
-            const SelItem it = sel_item(rd, seg, items, w, n);
+            const SelItem it = sel_item(rd, seg, items, w);
             SegDev& S = seg[it.seg];
             if (S.done) continue;
             lo = it.lo;
@@ -379,8 +368,8 @@ __global__ void __launch_bounds__(SEL_T)
         const u64 p = lp[j];
         const int id = li[j];
         bool ok = true;
-        for (int q = 2; q < pass; q++) ok = ok && sel_digit(p, id, q) == pre[q];
-        if (ok) atomicAdd(&h[sel_digit(p, id, pass)], 1u);
+        for (int q = 2; q < pass; q++) ok = ok && key_digit(p, id, q) == pre[q];
+        if (ok) atomicAdd(&h[key_digit(p, id, pass)], 1u);
     }
     __syncthreads();
     for (int x = threadIdx.x; x < 4096; x += SEL_T)
@@ -484,8 +473,8 @@ __global__ void __launch_bounds__(SEL_T)
             long long r = l.r, left = len;  // keys that agree with the digits so far
             for (int pass = 2; pass < 8; pass++) {
                 SelBin f;
-                if (sel_digit(dp, (int)di, pass) == 0) {
-                    f.bin = (int)sel_digit(p0, x0, pass);
+                if (key_digit(dp, (int)di, pass) == 0) {
+                    f.bin = (int)key_digit(p0, x0, pass);
                     f.cum = 0;
                     f.cnt = (unsigned long long)left;
                 } else {
@@ -494,8 +483,8 @@ __global__ void __launch_bounds__(SEL_T)
                     for (int j = threadIdx.x; j < len; j += SEL_T) {
                         bool ok = true;
                         for (int q = 2; q < pass; q++)
-                            ok = ok && sel_digit(sp[j], si[j], q) == pre[q];
-                        if (ok) atomicAdd(&h[sel_digit(sp[j], si[j], pass)], 1u);
+                            ok = ok && key_digit(sp[j], si[j], q) == pre[q];
+                        if (ok) atomicAdd(&h[key_digit(sp[j], si[j], pass)], 1u);
                     }
                     __syncthreads();
                     f = sel_bin([&](int b) { return h[b]; }, r);
@@ -522,8 +511,8 @@ __global__ void __launch_bounds__(SEL_T)
                 const u64 p = lp[l.base + j];
                 const int id = li[l.base + j];
                 bool ok = true;
-                for (int q = 2; q < pass; q++) ok = ok && sel_digit(p, id, q) == pre[q];
-                if (ok) atomicAdd(&h[sel_digit(p, id, pass)], 1u);
+                for (int q = 2; q < pass; q++) ok = ok && key_digit(p, id, q) == pre[q];
+                if (ok) atomicAdd(&h[key_digit(p, id, pass)], 1u);
             }
             __syncthreads();
             if (br > 0) {
