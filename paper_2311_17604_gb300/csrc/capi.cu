@@ -1166,10 +1166,13 @@ int decimate_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* keep
         h.fix_iters = std::max(1, std::min(PD_FIX_ITERS, atoi(getenv("PD_FIX_SWEEPS"))));
     CK(cudaMemcpyAsync(rd, &h, sizeof(h), cudaMemcpyHostToDevice, g->st));
     int64_t built = live;
-    bool long_list = live > ((int64_t)32 << 20);  // then: whether the last round's list was long
+    bool long_list = live > PD_SEL_FIRST;  // then: whether the last round's list was long
     // small clouds are bound by launches: from the third round on, a round's
     // launches are captured into a CUDA graph and replayed (PD_ROUND_GRAPH:
-    // 1 always, 0 never; default for grids up to 32M points and packed batches)
+    // 1 always, 0 never; default for grids up to 32M points and packed batches).
+    // Launched and replayed, ms: k = 1, 200k room points 2.75, 2.63, 2.0M site 7.27,
+    // 6.99, 12M 18.9, 18.6, 31M 42.2, 41.9, 50M 64.8, 65.2; k = 4, 200k room 19.4,
+    // 15.4, 9.8M outdoor 135, 126, 31M site 815, 778
     bool round_graph = g->n <= ((int64_t)32 << 20) || g->nseg > 0;
     if (getenv("PD_ROUND_GRAPH")) round_graph = atoi(getenv("PD_ROUND_GRAPH")) != 0;
     void* graph_pos = nullptr;
@@ -1470,6 +1473,9 @@ static int wup_impl(pd_grid* g, const pd_cost_params* cp, int64_t m, uint8_t* ke
         h.density_k1 = 1;  // rank: all that must go
         CK(cudaMemcpyAsync(rd, &h, sizeof(h), cudaMemcpyHostToDevice, g->st));
         {
+            // an iteration selects once, so nothing is known of its list: gridded
+            // clouds, cluster and whole grid, 1.0M points 14.6 and 14.1 ms, 4.0M 51.0
+            // and 48.3; others 0.7M 9.7 and 10.0, 5.0M 33.5 and 33.7
             Span t(T, &g->stats.ms_select);
             CK(round_launch_select(g->prim, g->pos, g->alive, g->ng, sb,
                                    g->ng > ((int64_t)4 << 20), rd, g->st));

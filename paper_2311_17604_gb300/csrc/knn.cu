@@ -992,7 +992,9 @@ __device__ __forceinline__ void warp_query(const GridView& g, const KnnArgs& a, 
     if (FILT == FILT_NONE && a.pairs_out && lane == 0) add_pairs(a, wr.pairs);
 }
 
-#define TAKE_MOST 16  // queries per warp up to which a list is taken one by one
+// Queries per warp up to which a list is taken one by one: 9.8M outdoor points, k = 4,
+// 129 ms with 0 and 4, 126 with 16, 64 and no limit; packed and room scans within 1 %.
+#define TAKE_MOST 16
 
 // FILTERED: qlist holds the points whose cost over smaller keys is wanted
 // (condition (A)), qlist2 the danger sources whose lambda is wanted.  ORDER:

@@ -221,6 +221,10 @@ inline unsigned list_blocks(int64_t n, int64_t per, int per_sm) {
 // it removes, and a dense spot without lower keys nearby yields few points of a
 // wide band but fewer still of a narrow one.  Only candidate lists that
 // overflow (cap_over, which make the danger test expensive) narrow it further.
+// Without a floor, with 256, 1024, 4096 keys (k = 4 unless stated): 31M site points
+// 831, 815, 781 ms; 2.4M outdoor, k = 2, 65.9, 63.3, 60.8; 12M site 150, 147, 148, 167;
+// four outdoor scans of 9.8M 122 to 125, 120 to 124, 121 to 128, 166; room scans within
+// 2 % of each other.
 #define PD_BAND_LEAST 1024
 __device__ __host__ inline double next_band(double band, double band_max, int band_mode,
                                             int density, long long live,
@@ -265,7 +269,13 @@ __device__ inline void round_finish(RoundDev* rd) {
 // band), and the round's counters opened.  long_list: the list of the keys that
 // agree in their leading digits is walked by the whole grid, not by one cluster
 // (the caller's guess from the round before, PD_SEL_LONG; either is correct).
-#define PD_SEL_LONG 262144
+// Selections of a gridded cloud's 3 rounds, cluster and whole grid: lists of 64k keys
+// 0.120 and 0.134 ms, 166k 0.165 and 0.137, 343k 0.241 and 0.143, 2.0M 0.97 and 0.21.
+// In a first round the list is not known: on a cloud whose keys differ the whole
+// grid's five further launches cost 0.02 to 0.03 ms, on a gridded one the cluster
+// 0.25 ms at 0.7M points and 5 of 16 ms at 8.0M (PD_SEL_FIRST).
+#define PD_SEL_LONG 131072
+#define PD_SEL_FIRST (1 << 20)
 cudaError_t round_launch_select(const u64* prim, const int4* pos, const uint8_t* alive, int64_t n,
                                 SelBuffers& b, bool long_list, RoundDev* rd, cudaStream_t st);
 // dep: list of the candidates that have a shell member of larger input index

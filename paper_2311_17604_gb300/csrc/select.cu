@@ -5,12 +5,11 @@
 // leading 12-bit digits (sign and exponent, then 12 mantissa bits): each counts
 // its digit in a shared histogram per block, and the block that finishes last
 // finds the digit's bin.  A third pass lists the keys that agree with both
-// digits, a thousandth of the points or so, and one cluster of 8 blocks (one
-// block per scan where a batch holds many) settles the remaining digits over
-// that list.  The leading digit alone would keep a whole power of two of keys,
-// so listing after it moved most of the points once more per round: a radix
-// select with a histogram, a find and a compaction launch per digit took 23
-// launches.  Measured, selection of all rounds of one decimation: 9.8M outdoor
+// digits, a thousandth of the points or so, and one cluster of 8 blocks (of eight
+// scans where a batch holds many) settles the remaining digits over that list.  The
+// leading digit alone would keep a whole power of two of keys, so listing after it
+// moved most of the points once more per round: a radix select with a histogram, a
+// find and a compaction launch per digit took 23 launches.  Measured, selection of all rounds of one decimation: 9.8M outdoor
 // points, k = 4 (287 rounds) 35.4 -> 17 ms; 3.8M points in a packed batch of 12 (612
 // rounds) 135 -> 28.5 ms; 200k room points, k = 1 (19 rounds) 1.30 -> 0.38 ms.
 //
@@ -30,7 +29,11 @@ namespace cg = cooperative_groups;
 
 #define SEL_T 512          // threads per block
 #define SEL_CLUSTER 8      // blocks of the cluster that settles a list
-#define SEL_CLUSTER_MAX 64 // scans of a batch up to which each has a cluster of its own
+// Scans of a batch up to which each has a cluster of its own.  Above, eight share one:
+// a launch of mostly idle blocks costs more than long lists one after the other (400
+// small scans 7.66 ms with a cluster each, 7.50; 1000 13.7, 13.3; 100 9.14, 9.18; 70
+// voxelised scans, long lists all, 57.7 and 61.0).
+#define SEL_CLUSTER_MAX 256
 
 struct SelBin {
     int bin;                      // -1: the rank is beyond the count

@@ -54,7 +54,7 @@ def test_wup(pd, ctx, lattice, k):
     assert np.array_equal(keep, oracle.decimate_wup(lattice, k, m)[0])
 
 
-@pytest.mark.parametrize("others", [2, 70])
+@pytest.mark.parametrize("others", [2, 70, 300])
 def test_one_scan_of_a_batch(pd, ctx, lattice, others):
     scans = [synth.random_cloud(i, 400 + 37 * i, 3000) for i in range(others)]
     scans.insert(others // 2, lattice)
