@@ -305,9 +305,11 @@ __device__ __forceinline__ void mlp_layer(float (&c)[MT][8][4], const uint32_t (
 // Persistent: a warp takes 32 rows at a time, the weights rounded into shared
 // memory once per block; the next rows arrive by 16-byte asynchronous copies
 // while these are computed.  Outputs per row: unit normal and |o|.
-// Bound: mma.sync itself, about 512 multiply-adds per clock and SM here (one or two
-// tiles a step, 8 to 32 warps per SM all measure 192 us or more for 4.0M rows; blocks
-// of 4 warps 201).
+// Bound: latency.  4.0M rows take 201 us with the tensor pipe 53 % and the schedulers
+// 46 % busy (128 registers, 14 warps in flight per SM); a warp's stalls per issue are
+// 2.7 cycles of fixed latency, 1.2 for the tensor pipe and 1.1 for the rows.  One or two
+// tiles a step and 8 to 32 warps per SM all took 192 us or more; blocks of 8 warps 192,
+// but a small call pays the attribute call above.
 // Fragments and features by 4-byte loads, as before, took 231 us.
 __global__ void __launch_bounds__(MLP_WARPS * 32, MLP_BLOCKS_PER_SM)
     mlp_forward_kernel(const float* __restrict__ prm, const uint16_t* __restrict__ feat,
