@@ -38,10 +38,16 @@ __global__ void dup_flag_kernel(const u64* __restrict__ code, const int4* __rest
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     unsigned c = 0;
     if (s < n) {
+        // coincident points share a code; where cells are wider than 1 mm (clouds
+        // beyond 2^21 mm) so do other points, which may lie between them
         uint8_t f = 0;
-        if (s > 0 && code[s] == code[s - 1]) {
-            int4 a = pos[s], b = pos[s - 1];
-            f = a.x == b.x && a.y == b.y && a.z == b.z;
+        const u64 c0 = code[s];
+        if (s > 0 && code[s - 1] == c0) {
+            const int4 a = pos[s];
+            for (int64_t j = s - 1; j >= 0 && !f && code[j] == c0; j--) {
+                const int4 b = pos[j];
+                f = a.x == b.x && a.y == b.y && a.z == b.z;
+            }
         }
         dup[s] = f;
         c = f;
